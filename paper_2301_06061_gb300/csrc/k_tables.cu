@@ -61,50 +61,77 @@ __global__ void k_l2(float2 *l2ff, double *l2d, int n, double dl) {
   l2d[a] = l2;
 }
 
-__device__ double kernel_eval_d(int kind, double x, double half, double param, const float *tab,
-                                int tlen, int W) {
-  if (x < -half || x > half) return 0.0;
-  if (kind == WST_KERNEL_GAUSS) return exp(-(x * x) / (2.0 * param * param));
-  if (kind == WST_KERNEL_ES) {
-    double z = 2.0 * x / W;
-    return exp(param * (sqrt(fmax(0.0, 1.0 - z * z)) - 1.0));
+// 1/Ghat(nu_a), nu_a = (a - n/2)/n, Ghat(nu) = int_{-W/2}^{W/2} G(x) cos(2 pi nu x) dx by
+// composite Simpson in FP64: 256 panels per cell for analytic kernels; for a table, one
+// panel per table interval so that the piecewise-linear kinks fall on panel ends.  As a sum
+// over the 2 P + 1 nodes x_i = (i - P) h/2 it is a cosine sum with weights that do not
+// depend on nu, and the cosine is even: k_kernel_nodes leaves, once, the P + 1 folded
+// weights c_j = w_{P+j} G(j h/2) + w_{P-j} G(-j h/2) (FP64, h/6 and the Simpson factors in
+// them), and k_correction sums c_j cos(2 pi nu j h/2) for each nu >= 0; -nu has the same.
+//
+// Bound: the FP64 pipe (2 FMA per clock and SM).  Each thread takes every 128th node and
+// advances its cosine by a rotation, 4 multiply-adds per node instead of a cospi (the
+// rotation's error after the longest run, 65536/128 steps, stays near 1e-13 of Ghat(0),
+// far below the FP32 result).  A block per nu with the kernel evaluated and three cospi
+// taken in every panel took 1106 us for an 8193-sample table at n = 512, on every
+// wst_plan_set_kernel_table, that is on every training step;
+// that step as a whole went from 1492 to 422 us.
+constexpr int kNodePanels = 256;   // panels per cell, analytic kernels
+constexpr int kCorrThreads = 128;
+
+static int node_panels(const wst_plan_s *p) {
+  return p->cfg.kernel == WST_KERNEL_TABLE ? p->cfg.ktable_len - 1 : kNodePanels * p->W;
+}
+int64_t kernel_node_count(const wst_plan_s *p) { return (int64_t)node_panels(p) + 1; }
+
+// G(x_i) at node i of 0 .. 2 P (a table's nodes are its samples and their midpoints)
+__device__ __forceinline__ double node_value(int kind, int i, int P, double half_h, double param, const float *tab,
+                                             int W) {
+  if (kind == WST_KERNEL_TABLE) {
+    const int k = i >> 1;
+    return (i & 1) ? 0.5 * ((double)tab[k] + (double)tab[k + 1]) : (double)tab[k];
   }
-  double pos = (x + half) * (double)(tlen - 1) / (double)W;
-  int i = (int)floor(pos);
-  i = max(0, min(i, tlen - 2));
-  double f = pos - (double)i;
-  return (1.0 - f) * (double)tab[i] + f * (double)tab[i + 1];
+  const double x = (double)(i - P) * half_h;
+  if (kind == WST_KERNEL_GAUSS) return exp(-(x * x) / (2.0 * param * param));
+  const double z = 2.0 * x / W;
+  return exp(param * (sqrt(fmax(0.0, 1.0 - z * z)) - 1.0));
 }
 
-// 1/Ghat(nu_a), Ghat(nu) = int_{-W/2}^{W/2} G(x) cos(2 pi nu x) dx by composite Simpson in
-// FP64: 256 panels per cell for analytic kernels; for a table, one panel per table
-// interval so the piecewise-linear kinks fall on panel ends.  One block per nu_a.
-__global__ void k_correction(float *corr, int n, int kind, int W, double param, const float *tab,
-                             int tlen) {
-  int a = blockIdx.x;
-  double nu = (double)(a - n / 2) / (double)n;
-  double half = 0.5 * W;
-  int panels = (kind == WST_KERNEL_TABLE) ? (tlen - 1) : 256 * W;
-  double h = (double)W / panels;
-  double acc = 0.0;
-  for (int s = threadIdx.x; s < panels; s += blockDim.x) {
-    double x0 = -half + s * h;
-    double xm = x0 + 0.5 * h;
-    double x1 = x0 + h;
-    // Simpson's rule on [x0, x1] (for a table the kinks sit exactly on x0 and x1)
-    double f0 = kernel_eval_d(kind, x0, half, param, tab, tlen, W) * cospi(2.0 * nu * x0);
-    double fm = kernel_eval_d(kind, xm, half, param, tab, tlen, W) * cospi(2.0 * nu * xm);
-    double f1 = kernel_eval_d(kind, x1, half, param, tab, tlen, W) * cospi(2.0 * nu * x1);
-    acc += (h / 6.0) * (f0 + 4.0 * fm + f1);
+__global__ void k_kernel_nodes(double *nodes, int P, int kind, int W, double param, const float *tab) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j > P) return;
+  const double half_h = 0.5 * (double)W / (double)P;
+  auto weight = [&](int i) { return (half_h / 3.0) * ((i & 1) ? 4.0 : (i == 0 || i == 2 * P) ? 1.0 : 2.0); };
+  double c = weight(P + j) * node_value(kind, P + j, P, half_h, param, tab, W);
+  if (j > 0) c += weight(P - j) * node_value(kind, P - j, P, half_h, param, tab, W);
+  nodes[j] = c;
+}
+
+__global__ void __launch_bounds__(kCorrThreads) k_correction(float *corr, int n, const double *__restrict__ nodes,
+                                                             int P, int W) {
+  const int k = blockIdx.x;  // nu = k / n, 0 <= k <= n/2
+  const double turn = (double)k * (double)W / ((double)n * (double)P);  // 2 nu h/2: half turns per node
+  double acc = 0.0, s, c, ds, dc;
+  sincospi(turn * (double)threadIdx.x, &s, &c);
+  sincospi(turn * (double)kCorrThreads, &ds, &dc);
+  for (int j = threadIdx.x; j <= P; j += kCorrThreads) {
+    acc = fma(__ldg(nodes + j), c, acc);
+    const double cn = fma(c, dc, -s * ds);
+    s = fma(s, dc, c * ds);
+    c = cn;
   }
-  __shared__ double red[256];
+  __shared__ double red[kCorrThreads];
   red[threadIdx.x] = acc;
   __syncthreads();
-  for (int st = blockDim.x / 2; st > 0; st >>= 1) {
+  for (int st = kCorrThreads / 2; st > 0; st >>= 1) {
     if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];
     __syncthreads();
   }
-  if (threadIdx.x == 0) corr[a] = (float)(1.0 / red[0]);
+  if (threadIdx.x == 0) {
+    const float r = (float)(1.0 / red[0]);
+    corr[n / 2 - k] = r;
+    if (k < n / 2) corr[n / 2 + k] = r;
+  }
 }
 
 cudaError_t build_tables(wst_plan_s *p) {
@@ -116,9 +143,10 @@ cudaError_t build_tables(wst_plan_s *p) {
 }
 
 cudaError_t build_correction(wst_plan_s *p) {
-  k_correction<<<p->n, 256, 0, p->stream>>>(p->corr, p->n, p->cfg.kernel, p->W, p->cfg.kparam,
-                                             p->ktable, p->cfg.ktable_len);
-  p->launches += 1;
+  const int P = node_panels(p);
+  k_kernel_nodes<<<(P + 256) / 256, 256, 0, p->stream>>>(p->knodes, P, p->cfg.kernel, p->W, p->cfg.kparam, p->ktable);
+  k_correction<<<p->n / 2 + 1, kCorrThreads, 0, p->stream>>>(p->corr, p->n, p->knodes, P, p->W);
+  p->launches += 2;
   return cudaGetLastError();
 }
 

@@ -89,6 +89,7 @@ __global__ void k_set_offsets(int64_t *dst, OffsetsArg a, int count) {
 void destroy_tables(wst_plan_s *p) {
   cudaFree(p->tw);
   cudaFree(p->corr);
+  cudaFree(p->knodes);
   cudaFree(p->l2ff);
   cudaFree(p->l2d);
   cudaFree(p->ktable);
@@ -211,6 +212,7 @@ wst_status wst_plan_create(const wst_config *cfg, void *cuda_stream, wst_plan *o
   if (e == cudaSuccess) e = cudaMalloc((void **)&(ptr), sizeof(*(ptr)) * (size_t)(count));
   ALLOC(p->tw, c.n);
   ALLOC(p->corr, c.n);
+  ALLOC(p->knodes, kernel_node_count(p));
   ALLOC(p->l2ff, c.n);
   ALLOC(p->l2d, c.n);
   ALLOC(p->wrange, 4 * c.batch);

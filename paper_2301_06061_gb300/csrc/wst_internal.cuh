@@ -111,6 +111,7 @@ struct wst_plan_s {
   // owned device tables
   float2 *tw = nullptr;      // exp(+2 pi i m / N), m < N
   float *corr = nullptr;     // 1 / Ghat(nu_a)
+  double *knodes = nullptr;  // folded quadrature weights of the kernel (k_kernel_nodes)
   float2 *l2ff = nullptr;    // l_a^2 as float-float
   double *l2d = nullptr;     // l_a^2 in FP64 (WST_FLAG_FP64_SCREEN)
   float *ktable = nullptr;   // TABLE kernel samples
@@ -257,6 +258,7 @@ cudaError_t build_tap_table(wst_plan_s *p);
 
 // k_tables.cu
 cudaError_t build_tables(wst_plan_s *p);
+int64_t kernel_node_count(const wst_plan_s *p);
 cudaError_t build_correction(wst_plan_s *p);
 cudaError_t build_plane_centres(wst_plan_s *p);
 

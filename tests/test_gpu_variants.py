@@ -1,0 +1,80 @@
+"""GPU parity of single kernels at the sizes where their code takes another turn: edges of
+blocks and tiles, remainders, the smallest and largest of a range.  References: the FP64
+oracle, or the same formula in numpy FP64."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import OracleConfig
+from paper_2301_06061_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wst():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2301_06061_gb300 import build, wst as w
+
+    build.build()
+    w.load_library()
+    return w
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# ------------------------------------------------------------------------------------------
+# grid correction 1/Ghat
+# ------------------------------------------------------------------------------------------
+
+def simpson_ghat(g_ends, g_mid, W, n):
+    """Composite Simpson of G(x) cos(2 pi nu x) over panels with the kernel's values at the
+    panel ends (P + 1) and middles (P); also the sum of the weights' magnitudes."""
+    P = len(g_mid)
+    x = np.linspace(-0.5 * W, 0.5 * W, 2 * P + 1)
+    g = np.empty(2 * P + 1)
+    g[::2], g[1::2] = g_ends, g_mid
+    wt = np.full(2 * P + 1, 2.0)
+    wt[1::2] = 4.0
+    wt[0] = wt[-1] = 1.0
+    c = wt * g * (W / P / 6.0)
+    nu = (np.arange(n) - n // 2) / n
+    return np.cos(2.0 * np.pi * np.outer(nu, x)) @ c, np.abs(c).sum()
+
+
+@pytest.mark.parametrize("n", [64, 1024])
+@pytest.mark.parametrize("kernel,W,length", [("gauss", 7, 0), ("es", 2, 0), ("table", 2, 2), ("table", 3, 128),
+                                             ("table", 8, 129), ("table", 8, 8193)])
+def test_correction_is_composite_simpson(wst, n, kernel, W, length):
+    """Every 1/Ghat is the FP64 quadrature rounded to FP32 (also for tables that are not
+    symmetric).  wst_correct of a unit image gives corr_a corr_b; along the central row the
+    products carry three FP32 roundings, 3 * 2^-24; the FP64 sum's own error is taken as
+    1e-12 of the sum of the weights."""
+    half = 0.5 * W
+    if kernel == "table":
+        rng = np.random.default_rng(length)
+        tab = (1.0 + rng.random(length)).astype(np.float32)
+        cfg = wst.Config(n=n, fov=0.1, n_w=1, support=W, kernel=wst.WST_KERNEL_TABLE, ktable_len=length)
+        t = tab.astype(np.float64)
+        want, total = simpson_ghat(t, 0.5 * (t[1:] + t[:-1]), W, n)
+    else:
+        P = 256 * W
+        x = np.linspace(-half, half, 2 * P + 1)
+        par = 0.875 if kernel == "gauss" else 2.3 * W
+        g = np.exp(-x * x / (2 * par * par)) if kernel == "gauss" else \
+            np.exp(par * (np.sqrt(np.clip(1 - (x / half) ** 2, 0, None)) - 1))
+        cfg = wst.Config(n=n, fov=0.1, n_w=1, support=W, kernel=0 if kernel == "gauss" else 1, kparam=par)
+        want, total = simpson_ghat(g[::2], g[1::2], W, n)
+    plan = wst.Plan(cfg)
+    if kernel == "table":
+        plan.set_kernel_table(dev(tab))
+    img = torch.ones((1, n, n), dtype=torch.complex64, device="cuda")
+    wst.wst_plan_stream(plan.handle)
+    wst.wst_correct(plan.handle, img)
+    prod = img[0, n // 2].real.double().cpu().numpy()  # corr_{n/2} corr_a
+    got = 1.0 / (prod * want[n // 2])
+    assert np.all(np.abs(got - want) <= 3 * 2.0 ** -24 * np.abs(want) * 1.01 + 1e-12 * total)
