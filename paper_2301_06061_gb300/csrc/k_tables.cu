@@ -160,8 +160,9 @@ __device__ __forceinline__ float ordered_to_float(uint32_t o) {
 __global__ void k_plane_centres(double *wrange, float4 *wrange_ff, float2 *wcentre, double *wcentre_d, float2 *dwff,
                                 const uint32_t *wminmax, int batch, int n_w, double cfg_lo,
                                 double cfg_hi, int from_data) {
-  int img = blockIdx.x * blockDim.x + threadIdx.x;
-  if (img >= batch) return;
+  const int P = blockIdx.x * blockDim.x + threadIdx.x;  // one thread per global plane
+  if (P >= batch * n_w) return;
+  const int img = P / n_w, k = P - img * n_w;
   double lo = cfg_lo, hi = cfg_hi;
   if (from_data) {
     uint32_t omin = wminmax[2 * img], omax = wminmax[2 * img + 1];
@@ -174,6 +175,10 @@ __global__ void k_plane_centres(double *wrange, float4 *wrange_ff, float2 *wcent
   }
   double scale = (hi > lo) ? (double)n_w / (hi - lo) : 0.0;
   double dw = (hi - lo) / (double)n_w;
+  const double wk = lo + ((double)k + 0.5) * dw;
+  wcentre[P] = ff_split(wk);
+  wcentre_d[P] = wk;
+  if (k != 0) return;
   wrange[4 * img + 0] = lo;
   wrange[4 * img + 1] = scale;
   wrange[4 * img + 2] = dw;
@@ -181,16 +186,11 @@ __global__ void k_plane_centres(double *wrange, float4 *wrange_ff, float2 *wcent
   dwff[img] = ff_split(dw);
   const float2 lo_ff = ff_split(lo), sc_ff = ff_split(scale);
   wrange_ff[img] = make_float4(lo_ff.x, lo_ff.y, sc_ff.x, sc_ff.y);
-  for (int k = 0; k < n_w; ++k) {
-    double wk = lo + ((double)k + 0.5) * dw;
-    wcentre[img * n_w + k] = ff_split(wk);
-    wcentre_d[img * n_w + k] = wk;
-  }
 }
 
 cudaError_t build_plane_centres(wst_plan_s *p) {
   const bool from_data = p->cfg.w_min == p->cfg.w_max;
-  k_plane_centres<<<(p->batch + 63) / 64, 64, 0, p->stream>>>(
+  k_plane_centres<<<(p->n_planes + 63) / 64, 64, 0, p->stream>>>(
       p->wrange, p->wrange_ff, p->wcentre, p->wcentre_d, p->dwff, p->W_.wminmax, p->batch, p->n_w, p->cfg.w_min,
       p->cfg.w_max, from_data ? 1 : 0);
   p->launches += 1;

@@ -77,15 +77,6 @@ Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
   return L;
 }
 
-// batch offsets to the device without a host synchronisation (passed as kernel args)
-struct OffsetsArg {
-  int64_t v[64];
-};
-__global__ void k_set_offsets(int64_t *dst, OffsetsArg a, int count) {
-  int i = threadIdx.x;
-  if (i < count) dst[i] = a.v[i];
-}
-
 void destroy_tables(wst_plan_s *p) {
   cudaFree(p->tw);
   cudaFree(p->corr);
@@ -354,18 +345,10 @@ static wst_status set_vis_common(wst_plan_s *p, int64_t n_vis, const VisCoords &
   W.comp = (p->chunk < p->n_planes) ? (float2 *)(p->ws + L.comp) : nullptr;
   W.bytes = L.total;
   p->launches = 0;
-  for (int i0 = 0; i0 <= p->batch; i0 += 64) {
-    ++p->launches;
-    OffsetsArg a;
-    const int cnt = (p->batch + 1 - i0) < 64 ? (p->batch + 1 - i0) : 64;
-    for (int i = 0; i < cnt; ++i) a.v[i] = off[i0 + i];
-    k_set_offsets<<<1, 64, 0, p->stream>>>(p->batch_off + i0, a, cnt);
-  }
-  WST_CUDA(p, cudaGetLastError(), "batch offsets");
   p->n_vis = n_vis;
   p->has_weight = weight != nullptr;
   WST_CUDA(p, time_begin(p, p->ev_sort, ST_SORT), "event");
-  WST_CUDA(p, sort_visibilities(p, coords, (const float2 *)vis, weight, host_vis), "sort");
+  WST_CUDA(p, sort_visibilities(p, coords, (const float2 *)vis, weight, off.data(), host_vis), "sort");
   WST_CUDA(p, time_end(p, p->ev_sort), "event");
   p->launches_sort = p->launches;
   p->vis_set = true;

@@ -295,9 +295,13 @@ __device__ __forceinline__ float coords_w(const VisCoords &c, int64_t j) {
   return c.w[j];
 }
 
-// k_sort.cu
+// k_sort.cu (batch_offsets: host int64 [batch + 1])
+constexpr int kSortOffsets = 64;  // batch offsets per launch
+struct SortOffsets {
+  int64_t v[kSortOffsets];
+};
 cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const float2 *vis, const float *weight,
-                              bool host_inputs);
+                              const int64_t *batch_offsets, bool host_inputs);
 cudaError_t vis_cells(wst_plan_s *p, int32_t *plane, int32_t *i0, int32_t *j0, int64_t n_bound);
 int64_t scan_tmp_words(int64_t n);
 

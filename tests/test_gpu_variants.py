@@ -78,3 +78,34 @@ def test_correction_is_composite_simpson(wst, n, kernel, W, length):
     prod = img[0, n // 2].real.double().cpu().numpy()  # corr_{n/2} corr_a
     got = 1.0 / (prod * want[n // 2])
     assert np.all(np.abs(got - want) <= 3 * 2.0 ** -24 * np.abs(want) * 1.01 + 1e-12 * total)
+
+
+# ------------------------------------------------------------------------------------------
+# sort: visibilities of uneven images over the blocks
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("counts", [[1], [31, 0, 33], [0, 1, 31, 33, 0, 5000, 2, 0, 70_000, 64], [1] * 130])
+def test_sort_of_uneven_images(wst, counts):
+    """Placement, counts and each image's w range (from the data) against the oracle, where
+    a block's share of the visibilities spans several images, empty ones among them."""
+    n, fov, n_w = 256, 0.1, 5
+    total = sum(counts)
+    u, v, w = synth.disk_uvw(total, 0.53 * n / fov, 150.0, np.random.default_rng(total))
+    vis = synth.random_visibilities(total, np.random.default_rng(1))
+    vis[::97] = np.nan
+    off = [0] + [int(x) for x in np.cumsum(counts)]
+    plan = wst.Plan(wst.Config(n=n, fov=fov, n_w=n_w, batch=len(counts)))
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis), None, off)
+    k = torch.empty(total, dtype=torch.int32, device="cuda")
+    i0, j0 = torch.empty_like(k), torch.empty_like(k)
+    wst.wst_vis_cells(plan.handle, k, i0, j0)
+    kept = dropped = bad = 0
+    for a, b in zip(off[:-1], off[1:]):
+        lo, hi = oracle.resolve_w_range(w[a:b], 0.0, 0.0)
+        ko, io, jo, st = oracle.locate(OracleConfig(n, fov, n_w, lo, hi), u[a:b], v[a:b], w[a:b], vis[a:b])
+        np.testing.assert_array_equal(k[a:b].cpu().numpy(), ko)
+        np.testing.assert_array_equal(i0[a:b].cpu().numpy(), io)
+        np.testing.assert_array_equal(j0[a:b].cpu().numpy(), jo)
+        kept, dropped, bad = kept + int((st == 0).sum()), dropped + int((st == 1).sum()), bad + int((st == 2).sum())
+    s = plan.stats()
+    assert (s["n_kept"], s["n_dropped"], s["n_nonfinite"]) == (kept, dropped, bad)
