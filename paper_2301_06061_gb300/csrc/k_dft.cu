@@ -1,8 +1,8 @@
 // Direct transforms: the exact dirty image at chosen pixels (the conjugate of Eq. 1,
 // summed over visibilities) and Eq. 1 itself for a point-source sky.  Phases are
-// formed in float-float (u l + v m + w (n-1) with l, m, n-1 carried as float-float)
-// and reduced modulo one cycle before an FP32 sincospi, so a phase of thousands of
-// cycles keeps about 1e-9 cycle accuracy.
+// formed from float-float l, m, n - 1 and reduced modulo one cycle before an FP32
+// sincospi (phase_frac), so a phase of thousands of cycles keeps the accuracy of one
+// below a cycle.
 #include "dft_core.cuh"
 
 namespace wst {
@@ -26,12 +26,13 @@ cudaError_t dft_pixels(int64_t n_vis, const float *u, const float *v, const floa
   if (e != cudaSuccess || n_pix == 0) return e;
   const int64_t pix_blocks = (n_pix + kDftPix - 1) / kDftPix;
   int64_t vis_blocks = (n_vis + kDftThreads - 1) / kDftThreads;
-  // about 4 CTAs per SM in total, at least one visibility block per pixel group
+  // about 16 CTAs per SM in total (eight rounds of the resident two: a short last round),
+  // at least one visibility block per pixel group
   int dev = 0, sms = 0;
   e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  int64_t target = ((int64_t)sms * 4 + pix_blocks - 1) / pix_blocks;
+  int64_t target = ((int64_t)sms * 16 + pix_blocks - 1) / pix_blocks;
   if (vis_blocks > target) vis_blocks = target;
   if (vis_blocks < 1) vis_blocks = 1;
   for (int64_t y0 = 0; y0 < pix_blocks; y0 += 65535) {
@@ -70,7 +71,7 @@ k_predict(int64_t n_vis, const float *__restrict__ u, const float *__restrict__ 
     const int cnt = (int)((n_src - s0) < kSrcTile ? (n_src - s0) : kSrcTile);
     if (in)
       for (int i = 0; i < cnt; ++i) {
-        const float2 e = cis_cycles_ff(ff_neg(phase_ff(uf, vf, wf, sl[i], sm_[i], st[i])));
+        const float2 e = cis_cycles(-phase_frac(uf, vf, wf, sl[i], sm_[i], st[i]));
         acc.x = fmaf(sf[i], e.x, acc.x);
         acc.y = fmaf(sf[i], e.y, acc.y);
       }

@@ -109,3 +109,40 @@ def test_sort_of_uneven_images(wst, counts):
         kept, dropped, bad = kept + int((st == 0).sum()), dropped + int((st == 1).sum()), bad + int((st == 2).sum())
     s = plan.stats()
     assert (s["n_kept"], s["n_dropped"], s["n_nonfinite"]) == (kept, dropped, bad)
+
+
+# ------------------------------------------------------------------------------------------
+# direct transforms
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("n_vis,n_pix", [(1, 1), (255, 8), (257, 9), (3001, 17), (40_000, 7)])
+def test_direct_transforms_against_fp64(wst, n_vis, n_pix):
+    """wst_dft and wst_predict_points on a field reaching outside the unit sphere, with (u, v,
+    w) from below one to thousands of cycles of phase.  Per visibility the phase is rounded
+    to FP32 twice at magnitude <= 1 (2^-24 cycle each) and sincospi errs by 2^-22 at most; a
+    thread adds n_vis/256 terms and the reduction 20 more, each rounding by 2^-24 of a
+    partial sum; the output's magnitude bound is sum |w V|."""
+    n, fov = 4096, 1.9
+    rng = np.random.default_rng(n_vis)
+    scale = 10.0 ** rng.uniform(-2, 3.5, (3, n_vis))
+    u, v, w = (scale * rng.uniform(-1, 1, (3, n_vis))).astype(np.float32)
+    vis = synth.random_visibilities(n_vis, rng)
+    wt = rng.uniform(0.5, 1.5, n_vis).astype(np.float32)
+    pa, pb = rng.integers(0, n, (2, n_pix)).astype(np.int32)
+    pa[0], pb[0] = n // 2, n // 2  # the phase centre
+    if n_pix > 1:
+        pa[1], pb[1] = 0, 0  # outside the unit sphere
+    out = torch.full((n_pix,), float("nan"), dtype=torch.complex64, device="cuda")
+    wst.wst_dft(dev(u), dev(v), dev(w), dev(vis), n, fov, dev(pa), dev(pb), out, dev(wt))
+    ref = oracle.dft_pixels(u, v, w, vis, n, fov, pa, pb, wt)
+    per_vis = 2 * np.pi * 2 * 2.0 ** -24 + 2.0 ** -22
+    tol = (per_vis + 2.0 ** -24 * (n_vis / 256 + 21)) * np.abs(wt * vis).sum()
+    assert np.abs(out.cpu().numpy() - ref).max() <= tol
+    if n_pix > 1:
+        assert out[1] == 0
+    l, m = rng.uniform(-0.6, 0.6, (2, n_pix))
+    flux = rng.uniform(0.1, 1.0, n_pix)
+    got = torch.empty(n_vis, dtype=torch.complex64, device="cuda")
+    wst.wst_predict_points(dev(u), dev(v), dev(w), dev(l), dev(m), dev(flux), got)
+    err = np.abs(got.cpu().numpy() - oracle.predict_points(u, v, w, l, m, flux)).max()
+    assert err <= (per_vis + 2.0 ** -24 * (n_pix + 1)) * flux.sum()
