@@ -40,7 +40,11 @@
 // per visibility-row (the bins count a visibility-row once per bin it reaches,
 // 1 + (W - 1)/64 bins on average) go straight to float atomics.  On the benchmark
 // workload the image error against the FP64 oracle equals that of all-float
-// accumulation.  Images narrower than kFixedMinN (8192) keep float atomics throughout.
+// accumulation.  Rows shorter than kBinnedMinN (8192) have one bin, the whole row, and its
+// sum over the W buckets is formed here: shared float atomics are compare-and-swap loops,
+// and integer ones took this kernel from 1.74 to 1.30 ms at 4096^2 x 32 planes (4.08M
+// visibilities), from 16.2 to 14.0 ms on 64 images of 2048^2 x 16 (37.7M) and the 256^2
+// one from 26 to 20 us, at the same error against FP64.
 #include "fft_core.cuh"
 
 namespace wst {
@@ -97,10 +101,10 @@ __device__ __forceinline__ void x_taps(const KernelParams &kp, float gx, float q
 }
 
 constexpr int kFixedBinCap = 8192;
-// Short rows (N < kFixedMinN) carry few visibility-rows each: the bound's extra barriers
-// cost more than the float atomics they would save, so they keep float accumulation.
+// rows whose bound comes from column bins (k_row_bounds); the others' is the sum of their W
+// buckets' magnitudes, loaded with the offsets
 template <int N>
-constexpr bool kFixedRows = N >= kFixedMinN;
+constexpr bool kBinnedRows = bins_per_row(N) > 1;
 
 // one tap into the planar row: float atomics, or (FIXED) the tap already in units of the
 // row's quantum (the record's value was scaled by 1/delta once), converted and added as
@@ -259,7 +263,7 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const 
                                              const uint32_t *__restrict__ off, int64_t b0, int q, bool nonempty,
                                              const KernelParams &kp, float2 *__restrict__ orow,
                                              const float2 *twt, int jt, const float2 *__restrict__ rowbound,
-                                             float gmax, RecHead *stg, int stg_stride, PEND &pd) {
+                                             const float *__restrict__ binmag, float *mag, float gmax, RecHead *stg, int stg_stride, PEND &pd) {
   using C = RowCfg<N>;
   constexpr int EPT = C::EPT, TPR = C::TPR;
   constexpr int NST = num_stages(N, EPT);
@@ -272,8 +276,11 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const 
   // the row's largest bin sum and total of the bin sums (k_row_bounds), broadcast
   float2 mb = make_float2(0.0f, 0.0f);
   if (nonempty) {
-    for (int i = jt; i <= d_lo + 1; i += TPR) bnd[i] = off[(b0 + q - d_lo + i) * kColBlocks];
-    if constexpr (kFixedRows<N>) mb = __ldg(rowbound + b0 + q);
+    for (int i = jt; i <= d_lo + 1; i += TPR) {
+      bnd[i] = off[(b0 + q - d_lo + i) * kColBlocks];
+      if constexpr (!kBinnedRows<N>) mag[i] = i <= d_lo ? __ldg(binmag + b0 + q - d_lo + i) : 0.0f;
+    }
+    if constexpr (kBinnedRows<N>) mb = __ldg(rowbound + b0 + q);
   }
   // two groups of the previous row's outputs go out while the offsets load (more, or one
   // more after the first record heads are requested, measured slower)
@@ -283,15 +290,26 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const 
   __syncthreads();
   // the same decision and quantum in every thread of the row
   const uint32_t cnt = nonempty ? bnd[d_lo + 1] - bnd[0] : 0u;
+  if constexpr (!kBinnedRows<N>) {
+    if (nonempty)
+      for (int i = 0; i <= d_lo; ++i) mb.x += mag[i];
+  }
   const float mmax = mb.x, mtot = mb.y;
   const float bound = mmax * (gmax * gmax);
-  // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row
-  const float n_eff = mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
-  const bool fixed = kFixedRows<N> && nonempty && cnt < (1u << 30) && bound >= 0x1p-90f && bound <= 0x1p+100f &&
+  // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row (one
+  // bin: the row's visibilities)
+  const float n_eff = !kBinnedRows<N> ? (float)cnt
+                      : mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
+  const bool fixed = nonempty && cnt < (1u << 30) && bound >= 0x1p-90f && bound <= 0x1p+100f &&
                      n_eff <= (float)kFixedBinCap;
   // a bin of fewer than ~64 mean contributions may hold a single tap above B/8: such rows
-  // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range
-  const float unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
+  // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range.  A
+  // whole row as one bin spreads over more cells: there the quantum follows the count, so
+  // that it stays near 2^-26 of the mean magnitude (below the rounding of a float sum)
+  // while a cell may still hold 8 to 32 mean contributions in phase, or half the row
+  float unit;
+  if constexpr (kBinnedRows<N>) unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
+  else unit = n_eff < 16.0f ? 0x1p-30f : n_eff < 64.0f ? 0x1p-32f : n_eff < 256.0f ? 0x1p-33f : 0x1p-34f;
   bool fx = fixed;
   int ovf = 0;
   if (nonempty) {
@@ -299,9 +317,8 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const 
       ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, pd);
     else grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, pd);
   }
-  bool redo = false;  // a tap or a partial sum left the int32 range: accumulate in float
-  if constexpr (kFixedRows<N>) redo = __syncthreads_or(ovf < 0);
-  else __syncthreads();
+  // a tap or a partial sum left the int32 range: accumulate in float (every row of the CTA)
+  const bool redo = __syncthreads_or(ovf < 0);
   if (redo) {
     zero_row<N>(srow, jt);
     __syncthreads();
@@ -373,12 +390,13 @@ __global__ void __launch_bounds__(RowCfg<N>::THREADS)
 k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, int p0, int np,
             KernelParams kp, float2 *__restrict__ out, uint8_t *__restrict__ occ,
             unsigned long long *__restrict__ counter, Tw tw, const float2 *__restrict__ rowbound,
-            unsigned long long *__restrict__ rows_done) {
+            const float *__restrict__ binmag, unsigned long long *__restrict__ rows_done) {
   using C = RowCfg<N>;
   constexpr int TPR = C::TPR, RPC = C::RPC;
   extern __shared__ __align__(16) float2 sm_rows[];
   __shared__ long long s_item;
   __shared__ uint32_t s_bnd[RPC][kMaxSupport + 2];
+  __shared__ float s_mag[RPC][kMaxSupport + 2];
   __shared__ uint32_t s_gmax;  // largest |kernel value| (FP32 bits)
   const int rl = threadIdx.x / TPR, jt = threadIdx.x % TPR;
   float2 *srow = sm_rows + rl * C::PADL;
@@ -450,7 +468,7 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
         const long long item = base + (e >> 1);
         const int pl = (int)(item / N), q = (int)(item % N);
         grid_one_row<N, FFT, WT>(srow, s_bnd[0], rec, off, (int64_t)(p0 + pl) * N, q, e & 1, kp,
-                                 out + ((int64_t)pl * N + q) * N, twt, jt, rowbound, gmax, stg, stg_stride, pd);
+                                 out + ((int64_t)pl * N + q) * N, twt, jt, rowbound, binmag, s_mag[0], gmax, stg, stg_stride, pd);
       }
     }
     pd.write_all(jt);  // the CTA's last row
@@ -471,7 +489,7 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
       float2 *orow = valid && (!FFT || !empty) ? out + ((int64_t)pl * N + q) * N : nullptr;
       NoPending none;
       grid_one_row<N, FFT, WT>(srow, s_bnd[rl], rec, off, (int64_t)(p0 + pl) * N, q, !empty, kp, orow, twt, jt,
-                               rowbound, gmax, stg, stg_stride, none);
+                               rowbound, binmag, s_mag[rl], gmax, stg, stg_stride, none);
     }
   }
 }
@@ -639,7 +657,7 @@ static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) 
   e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), p->stream);
   if (e != cudaSuccess) return e;
   kern<<<grid, C::THREADS, smem, p->stream>>>(p->W_.records, p->W_.offsets, p0, np, kernel_params(p), out,
-                                             p->W_.occ, counter, tw_half(p), p->W_.rowbound,
+                                             p->W_.occ, counter, tw_half(p), p->W_.rowbound, p->W_.binmag,
                                              FFT ? p->W_.counters + CNT_ROWS : nullptr);
   return cudaGetLastError();
 }

@@ -484,7 +484,7 @@ __global__ void k_scatter(const float2 *__restrict__ vis, const float *__restric
         vre = val[h].x * wt[h];
         vim = (ki[h].y ? -val[h].y : val[h].y) * wt[h];  // mirrored: conj
       }
-      if (binmag) {  // the whole warp: the first bin by runs, the second (rare) directly
+      {  // the whole warp: the first bin by runs, the second (rare) directly
         const float mag = fmaxf(fabsf(vre), fabsf(vim));
         const int i0 = (int)(ki[h].z >> 18);
         const int bl = min(i0 >> kBinShift, nb - 1), bh = min((i0 + W - 1) >> kBinShift, nb - 1);
@@ -556,7 +556,11 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
     k_sort_init<<<1, 256, 0, s>>>(p->batch_off + i0, a, cnt, i0 == 0 ? ws.counters : nullptr, ws.wminmax, p->batch);
     p->launches += 1;
   }
-  if ((e = cudaMemsetAsync(ws.offsets, 0, sizeof(uint32_t) * nb1, s))) return e;
+  // offsets and, after them in the workspace, the magnitude bins
+  const int nb = bins_per_row(p->n);
+  const int64_t n_bins = p->n_buckets / kColBlocks * nb;
+  const size_t clear = (size_t)((char *)(ws.binmag + n_bins) - (char *)ws.offsets);
+  if ((e = cudaMemsetAsync(ws.offsets, 0, clear, s))) return e;
   const bool fold = (p->cfg.flags & WST_FLAG_WFOLD) != 0;
   int sms = 0;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device))) return e;
@@ -590,16 +594,12 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
   if ((e = cudaGetLastError())) return e;
   if ((e = scan_exclusive(ws.offsets, nb1, ws.scan_tmp, s, p->launches))) return e;
   if ((e = cudaMemcpyAsync(ws.cursor, ws.offsets, sizeof(uint32_t) * nb1, cudaMemcpyDeviceToDevice, s))) return e;
-  const int nb = bins_per_row(p->n);
-  float *binmag = p->n >= kFixedMinN ? ws.binmag : nullptr;  // only long rows use the bound
-  if (binmag && (e = cudaMemsetAsync(binmag, 0, sizeof(float) * (size_t)(p->n_buckets / kColBlocks) * nb, s)))
-    return e;
   k_scatter<<<grid_for(p->n_vis, 256, 152 * 16), 256, 0, s>>>(vis, weight, ws.keyinfo, ws.cursor, p->n_vis,
-                                                              ws.records, binmag, nb, p->W, stash);
+                                                              ws.records, ws.binmag, nb, p->W, stash);
   p->launches += 1;
-  if (binmag) {
+  if (nb > 1) {
     const int64_t n_rows = p->n_buckets / kColBlocks;
-    k_row_bounds<<<grid_for(n_rows * 32, 256, 152 * 8), 256, 0, s>>>(binmag, ws.offsets, n_rows, p->n, nb, p->W,
+    k_row_bounds<<<grid_for(n_rows * 32, 256, 152 * 8), 256, 0, s>>>(ws.binmag, ws.offsets, n_rows, p->n, nb, p->W,
                                                                      ws.rowbound);
     p->launches += 1;
   }

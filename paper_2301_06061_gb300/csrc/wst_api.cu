@@ -57,6 +57,8 @@ Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
   off += align_up((size_t)n_vis * sizeof(Record));
   L.offsets = off;
   off += align_up((size_t)(p->n_buckets + 1) * sizeof(uint32_t));
+  L.binmag = off;  // directly after the offsets: one memset clears both
+  off += align_up((size_t)(p->n_buckets / kColBlocks) * bins_per_row(p->n) * sizeof(float));
   L.cursor = off;
   off += align_up((size_t)(p->n_buckets + 1) * sizeof(uint32_t));
   L.scan_tmp = off;
@@ -67,10 +69,8 @@ Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
   off += align_up((size_t)2 * p->batch * sizeof(uint32_t));
   L.occ = off;
   off += align_up((size_t)p->n_planes * p->n);
-  L.binmag = off;
-  if (p->n >= kFixedMinN) off += align_up((size_t)(p->n_buckets / kColBlocks) * bins_per_row(p->n) * sizeof(float));
   L.rowbound = off;
-  if (p->n >= kFixedMinN) off += align_up((size_t)(p->n_buckets / kColBlocks) * sizeof(float2));
+  if (bins_per_row(p->n) > 1) off += align_up((size_t)(p->n_buckets / kColBlocks) * sizeof(float2));
   L.comp = off;
   if (p->chunk < p->n_planes) off += align_up((size_t)p->batch * p->n_img * p->n_img * sizeof(float2));
   L.total = off;
