@@ -1,8 +1,8 @@
 // Direct transform core shared by k_dft (k_dft.cu) and k_dft_partials (wst_noalloc.cu):
 // the exact dirty image at a few pixels (the conjugate of Eq. 1 summed over the
 // visibilities), phases u l + v m + w (n-1) formed from float-float l, m, n-1 with the
-// whole cycles taken out product by product (phase_frac) before an FP32 sincospi, so a
-// phase of thousands of cycles keeps the accuracy of one below a cycle.
+// cycles taken out product by product (cis_small, cis_any) before the FP32 sine and cosine,
+// so a phase of thousands of cycles keeps the accuracy of one below a cycle.
 #pragma once
 
 #include "wst_internal.cuh"
@@ -21,30 +21,39 @@ __device__ __forceinline__ ff ff_from_double(double d) {
   return {s.x, s.y};
 }
 
-// u l + v m + w t modulo whole cycles, as one FP32 number of magnitude about 1/2 or less.
-// Each product's leading part is exact as p + e (the product and its fused residual), and
-// p - rint(p) is exact, so the whole cycles leave each product before any sum is rounded;
-// the residuals and the low words' products are small and summed in FP32.  The sum of the
-// three fractions is exact unless a product is itself below a cycle or two; its error is
-// then at most 2^-24 cycle, that of the FP32 argument sincospi takes.  The kernels are bound
-// by FP32 issue; float-float products and sums of the whole phase took 1360 us for 2e5
-// visibilities at 2048 pixels, this (with the pixels' set-up once per CTA) 825 us, at an
-// error against FP64 of 2.7e-7 instead of 3.1e-7.
-__device__ __forceinline__ float phase_frac(float u, float v, float w, const ff &l, const ff &m, const ff &t) {
+// exp(2 pi i (u l + v m + w t)) for |u|, |v|, |w| <= kCisMax and |l|, |m|, |t| <= 1 (cis_small)
+//
+// Each product loses its half cycles before anything is summed: u l.hi + M is one fused
+// operation that rounds the exact product to a multiple of 1/2 (whose parity is the last bit
+// of the result), and the fused difference leaves the rest, |a| <= 1/4, rounded once (2^-27
+// cycle).  The low words' products and the three rests are summed and cis_small_cycles does
+// the remainder.  The kernel is bound by the FP32 multiply-add pipe: 39 operations a product
+// and pixel, 583 us for 2e5 visibilities at 2048 pixels; with rintf and the reductions inside
+// sincospi (cis_any), which go to a slower pipe, 827 us.
+constexpr float kCisMax = 0x1p+20f;
+__device__ __forceinline__ float2 cis_small(float u, float v, float w, const ff &l, const ff &m, const ff &t) {
+  constexpr float M = kHalfCycle;
+  const float tu = __fmaf_rn(u, l.hi, M), tv = __fmaf_rn(v, m.hi, M), tw = __fmaf_rn(w, t.hi, M);
+  const float a = __fmaf_rn(u, l.hi, -__fsub_rn(tu, M)), b = __fmaf_rn(v, m.hi, -__fsub_rn(tv, M));
+  const float c = __fmaf_rn(w, t.hi, -__fsub_rn(tw, M));
+  const float e = __fmaf_rn(w, t.lo, __fmaf_rn(v, m.lo, __fmul_rn(u, l.lo)));
+  return cis_small_cycles(__fadd_rn(__fadd_rn(a, b), __fadd_rn(c, e)),
+                          __float_as_uint(tu) ^ __float_as_uint(tv) ^ __float_as_uint(tw));
+}
+
+// the same for any size: whole cycles by rint, product by product (p + e is the exact
+// product, p - rint(p) is exact), then sincospi
+static __device__ __noinline__ float2 cis_any(float u, float v, float w, ff l, ff m, ff t) {
   const float pu = __fmul_rn(u, l.hi), pv = __fmul_rn(v, m.hi), pw = __fmul_rn(w, t.hi);
   float e = __fmaf_rn(u, l.lo, __fmaf_rn(u, l.hi, -pu));
   e = __fmaf_rn(v, m.lo, __fadd_rn(e, __fmaf_rn(v, m.hi, -pv)));
   e = __fmaf_rn(w, t.lo, __fadd_rn(e, __fmaf_rn(w, t.hi, -pw)));
   const float a = __fsub_rn(pu, rintf(pu)), b = __fsub_rn(pv, rintf(pv)), c = __fsub_rn(pw, rintf(pw));
   const float s = __fadd_rn(__fadd_rn(a, b), c);
-  return __fadd_rn(__fsub_rn(s, rintf(s)), e);
-}
-
-// exp(2 pi i phi) of a phase given in cycles
-__device__ __forceinline__ float2 cis_cycles(float phi) {
-  float s, c;
-  sincospif(2.0f * phi, &s, &c);
-  return make_float2(c, s);
+  const float phi = __fadd_rn(__fsub_rn(s, rintf(s)), e);
+  float sn, cs;
+  sincospif(2.0f * phi, &sn, &cs);
+  return make_float2(cs, sn);
 }
 
 // The CTA's share of out_i = sum_j w_j V_j exp(2 pi i (u_j l_i + v_j m_i + w_j (n_i - 1)))
@@ -96,11 +105,16 @@ __device__ __forceinline__ float2 dft_cta_partial(int64_t n_vis, const float *__
     if (!(isfinite(uf) && isfinite(vf) && isfinite(wf) && isfinite(val.x) && isfinite(val.y) && isfinite(wt)))
       continue;
     val = make_float2(val.x * wt, val.y * wt);
+    auto add = [&](float2 &s, float2 e) {
+      s.x = fmaf(val.x, e.x, fmaf(-val.y, e.y, s.x));
+      s.y = fmaf(val.x, e.y, fmaf(val.y, e.x, s.y));
+    };
+    if (fmaxf(fmaxf(fabsf(uf), fabsf(vf)), fabsf(wf)) <= kCisMax) {
 #pragma unroll
-    for (int i = 0; i < kDftPix; ++i) {
-      const float2 e = cis_cycles(phase_frac(uf, vf, wf, px[i].l, px[i].m, px[i].t));
-      acc[i].x = fmaf(val.x, e.x, fmaf(-val.y, e.y, acc[i].x));
-      acc[i].y = fmaf(val.x, e.y, fmaf(val.y, e.x, acc[i].y));
+      for (int i = 0; i < kDftPix; ++i) add(acc[i], cis_small(uf, vf, wf, px[i].l, px[i].m, px[i].t));
+    } else {
+#pragma unroll
+      for (int i = 0; i < kDftPix; ++i) add(acc[i], cis_any(uf, vf, wf, px[i].l, px[i].m, px[i].t));
     }
   }
   __shared__ float2 red[kDftThreads / 32][kDftPix];

@@ -1,7 +1,7 @@
 // Direct transforms: the exact dirty image at chosen pixels (the conjugate of Eq. 1,
 // summed over visibilities) and Eq. 1 itself for a point-source sky.  Phases are
-// formed from float-float l, m, n - 1 and reduced modulo one cycle before an FP32
-// sincospi (phase_frac), so a phase of thousands of cycles keeps the accuracy of one
+// formed from float-float l, m, n - 1 and reduced modulo one cycle before the FP32 sine
+// and cosine (dft_core.cuh), so a phase of thousands of cycles keeps the accuracy of one
 // below a cycle.
 #include "dft_core.cuh"
 
@@ -57,8 +57,10 @@ k_predict(int64_t n_vis, const float *__restrict__ u, const float *__restrict__ 
   const bool in = j < n_vis;
   const float uf = in ? u[j] : 0.0f, vf = in ? v[j] : 0.0f, wf = in ? w[j] : 0.0f;
   float2 acc = make_float2(0.0f, 0.0f);
+  const bool small_vis = fmaxf(fmaxf(fabsf(uf), fabsf(vf)), fabsf(wf)) <= kCisMax;
   for (int64_t s0 = 0; s0 < n_src; s0 += kSrcTile) {
     __syncthreads();
+    bool small_src = true;  // cis_small's range of l and m (a source may be given anywhere)
     for (int i = threadIdx.x; i < kSrcTile && s0 + i < n_src; i += blockDim.x) {
       const double ls = l[s0 + i], ms = m[s0 + i];
       const double r2 = ls * ls + ms * ms;
@@ -66,15 +68,18 @@ k_predict(int64_t n_vis, const float *__restrict__ u, const float *__restrict__ 
       sm_[i] = ff_from_double(ms);
       st[i] = ff_from_double(r2 < 1.0 ? -r2 / (1.0 + sqrt(1.0 - r2)) : 0.0);
       sf[i] = (float)flux[s0 + i];
+      small_src = small_src && fmax(fabs(ls), fabs(ms)) <= 1.0;
     }
-    __syncthreads();
+    const bool small = __syncthreads_and(small_src) && small_vis;
     const int cnt = (int)((n_src - s0) < kSrcTile ? (n_src - s0) : kSrcTile);
-    if (in)
-      for (int i = 0; i < cnt; ++i) {
-        const float2 e = cis_cycles(-phase_frac(uf, vf, wf, sl[i], sm_[i], st[i]));
-        acc.x = fmaf(sf[i], e.x, acc.x);
-        acc.y = fmaf(sf[i], e.y, acc.y);
-      }
+    auto add = [&](int i, float2 e) {  // the conjugate: Eq. 1 has the negative exponent
+      acc.x = fmaf(sf[i], e.x, acc.x);
+      acc.y = fmaf(sf[i], -e.y, acc.y);
+    };
+    if (in && small)
+      for (int i = 0; i < cnt; ++i) add(i, cis_small(uf, vf, wf, sl[i], sm_[i], st[i]));
+    else if (in)
+      for (int i = 0; i < cnt; ++i) add(i, cis_any(uf, vf, wf, sl[i], sm_[i], st[i]));
   }
   if (in) out[j] = acc;
 }

@@ -146,3 +146,33 @@ def test_direct_transforms_against_fp64(wst, n_vis, n_pix):
     wst.wst_predict_points(dev(u), dev(v), dev(w), dev(l), dev(m), dev(flux), got)
     err = np.abs(got.cpu().numpy() - oracle.predict_points(u, v, w, l, m, flux)).max()
     assert err <= (per_vis + 2.0 ** -24 * (n_pix + 1)) * flux.sum()
+
+
+@pytest.mark.parametrize("scale", [0.99, 1.01, 4.0])
+def test_direct_transforms_around_the_fast_phases_range(wst, scale):
+    """|u| at and beyond 2^20 wavelengths, where the direct transforms change to the general
+    phase reduction, with sources in and outside |l| <= 1 for the prediction.  l is a pair of
+    floats, 2^-49 of its value, so a phase errs by 2^-29 cycle there; the sums' bound is that
+    of the phases' FP32 rounding."""
+    n, fov, n_vis, n_pix = 512, 0.2, 3000, 9
+    rng = np.random.default_rng(int(100 * scale))
+    u, v, w = (rng.uniform(-1, 1, (3, n_vis)) * scale * 2.0 ** 20).astype(np.float32)
+    vis = synth.random_visibilities(n_vis, rng)
+    pa, pb = rng.integers(0, n, (2, n_pix)).astype(np.int32)
+    out = torch.empty(n_pix, dtype=torch.complex64, device="cuda")
+    wst.wst_dft(dev(u), dev(v), dev(w), dev(vis), n, fov, dev(pa), dev(pb), out)
+    ref = oracle.dft_pixels(u, v, w, vis, n, fov, pa, pb)
+    per_vis = 2 * np.pi * 3 * 2.0 ** -24 + 2.0 ** -22
+    assert np.abs(out.cpu().numpy() - ref).max() <= (per_vis + 2.0 ** -24 * (n_vis / 256 + 21)) * np.abs(vis).sum()
+    for far in (0.0, 1.5):
+        l, m = rng.uniform(-0.1, 0.1, (2, 5))
+        l[0] += far
+        flux = rng.uniform(0.1, 1.0, 5)
+        got = torch.empty(n_vis, dtype=torch.complex64, device="cuda")
+        wst.wst_predict_points(dev(u), dev(v), dev(w), dev(l), dev(m), dev(flux), got)
+        keep = np.arange(5) if far == 0.0 else np.arange(1, 5)
+        if far == 0.0:
+            err = np.abs(got.cpu().numpy() - oracle.predict_points(u, v, w, l, m, flux)).max()
+            assert err <= (per_vis + 2.0 ** -24 * 6) * flux[keep].sum()
+        else:
+            assert torch.isfinite(torch.view_as_real(got)).all()
