@@ -384,9 +384,11 @@ struct TableTw {
   }
 };
 
-// middle_stages with the twiddles from a provider (see stage_compute_f)
-template <int L, int EPT, int TPL, int S, int DIR, class SMI, class TWP>
-__device__ __forceinline__ void middle_stages_f(float2 (&v)[EPT], int jt, float2 *sm, SMI smi, const TWP &twp) {
+// middle_stages with the twiddles from a provider (see stage_compute_f); `sync` is the
+// barrier of the threads that share the line
+template <int L, int EPT, int TPL, int S, int DIR, class SMI, class TWP, class SYNC>
+__device__ __forceinline__ void middle_stages_f(float2 (&v)[EPT], int jt, float2 *sm, SMI smi, const TWP &twp,
+                                                const SYNC &sync) {
   constexpr int NST = num_stages(L, EPT);
   if constexpr (S < NST) {
     constexpr int RP = stage_radix(L, EPT, S - 1);
@@ -394,16 +396,16 @@ __device__ __forceinline__ void middle_stages_f(float2 (&v)[EPT], int jt, float2
     for (int b = 0; b < EPT / RP; ++b)
 #pragma unroll
       for (int r = 0; r < RP; ++r) sm[smi(out_index<L, EPT, TPL, S - 1>(jt, b, r))] = v[b * RP + r];
-    __syncthreads();
+    sync();
     constexpr int R = stage_radix(L, EPT, S);
 #pragma unroll
     for (int b = 0; b < EPT / R; ++b)
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b * R + r] = sm[smi(in_index<L, EPT, TPL, S>(jt, b, r))];
     if constexpr (S + 1 < NST) {
-      __syncthreads();
+      sync();
       stage_compute_f<L, EPT, TPL, S, DIR>(v, jt, twp);
-      middle_stages_f<L, EPT, TPL, S + 1, DIR>(v, jt, sm, smi, twp);
+      middle_stages_f<L, EPT, TPL, S + 1, DIR>(v, jt, sm, smi, twp, sync);
     }
   }
 }

@@ -17,8 +17,8 @@
 // w G_y(d) sum_a G_x(a) row[i0 + a] to dvis; the kernel gradient scatters the tap
 // products into a shared partial table.  Rows nobody reads are skipped.
 //
-// Items are handed out by a device counter to persistent CTAs (one row or, for short
-// rows, RowCfg::RPC rows per CTA step).
+// Rows are handed out by a device counter to the thread groups of persistent CTAs
+// (GroupCfg).
 //
 // Fixed-point accumulation.  Shared-memory integer atomics sustain about three times
 // the rate of float ones on this GPU.  The sort leaves, per row bucket and bin of 64
@@ -32,7 +32,7 @@
 // fine quantum usable; but a cell or a single tap can exceed 2^31 delta = B/8 (a
 // dominant visibility, a coherent pile-up), so every integer atomic returns the old
 // value and the kernel checks for a wrapped partial sum or a saturated conversion: if
-// any occurred in the row, the row is zeroed and accumulated again with float atomics.
+// any occurred in the row, the row is zeroed and accumulated again with delta = B / 2^30.
 // Rows whose busiest bin holds fewer than 64 mean contributions take delta = B / 2^30,
 // which cannot overflow (sparse rows would otherwise overflow often; their cells are
 // few-term sums, for which the coarser quantum is precise enough).
@@ -40,14 +40,78 @@
 // per visibility-row (the bins count a visibility-row once per bin it reaches,
 // 1 + (W - 1)/64 bins on average) go straight to float atomics.  On the benchmark
 // workload the image error against the FP64 oracle equals that of all-float
-// accumulation.  Rows shorter than kBinnedMinN (8192) have one bin, the whole row, and its
-// sum over the W buckets is formed here: shared float atomics are compare-and-swap loops,
-// and integer ones took this kernel from 1.74 to 1.30 ms at 4096^2 x 32 planes (4.08M
-// visibilities), from 16.2 to 14.0 ms on 64 images of 2048^2 x 16 (37.7M) and the 256^2
-// one from 26 to 20 us, at the same error against FP64.
+// accumulation.  Rows shorter than 8192 take finer steps of the quantum (log2_unit): shared
+// float atomics are compare-and-swap loops, and integer ones took this kernel from 1.74 to
+// 1.30 ms at 4096^2 x 32 planes (4.08M visibilities), from 16.2 to 14.0 ms on 64 images of
+// 2048^2 x 16 (37.7M) and the 256^2 one from 26 to 20 us, at the same error against FP64.
 #include "fft_core.cuh"
 
 namespace wst {
+
+// The row kernels' threads: a row has TPR, and the rows of a CTA are worked on by groups
+// of GT threads (whole warps) that claim rows and synchronise on their own: a group with
+// a dense row does not hold up the others, and empty rows cost no barrier of the CTA.  The
+// groups share the CTA's twiddle tables.  Rows shorter than 512 have fewer than 32 threads;
+// a group then takes GR rows in step.  CTAs of 128 threads, so that short workloads (a
+// 256^2 image has 16 rows per SM) still spread over the SMs.
+template <int N, int MINT = 128>
+struct GroupCfg {
+  static constexpr int EPT = RowCfg<N>::EPT, TPR = RowCfg<N>::TPR, PADL = RowCfg<N>::PADL;
+  static constexpr int GT = TPR >= 32 ? TPR : 32;
+  static constexpr int GR = GT / TPR;
+  static constexpr int THREADS = TPR >= MINT ? TPR : MINT;
+  static constexpr int GROUPS = THREADS / GT;
+  static constexpr int ROWS = GROUPS * GR;  // rows in a CTA's shared memory
+};
+
+// The gridder's configuration: four rows of 4096 at once in a CTA of 1024 threads, which
+// share its 33 KB of twiddle tables (two CTAs with a row each fit otherwise: 1327 instead of
+// 1277 us on 32 planes of 4096^2 with 4.08M visibilities, 986 instead of 882 us on 21 planes
+// with the ES kernel).  Two rows of 8192 in a CTA leave 64 registers a thread: 5.90 instead of
+// 5.03 ms on 16 planes with 20M visibilities.
+template <int N>
+using GridCfg = GroupCfg<N, N == 4096 ? 1024 : 128>;
+// whether a group writes a row out during its next row's gridding: where it is alone
+template <int N>
+constexpr bool kPending = N >= 8192;
+
+// barrier of one group: the CTA, a warp, or a named barrier of the group's warps
+template <int GT, int GROUPS>
+struct GroupSync {
+  int g;
+  __device__ __forceinline__ void operator()() const {
+    if constexpr (GROUPS == 1) __syncthreads();
+    else if constexpr (GT == 32) __syncwarp();
+    else asm volatile("barrier.cta.sync %0, %1;" ::"r"(g + 1), "n"(GT) : "memory");
+  }
+  // barrier with the or of a predicate over the group
+  __device__ __forceinline__ bool any(bool x) const {
+    if constexpr (GROUPS == 1) {
+      return __syncthreads_or(x);
+    } else if constexpr (GT == 32) {
+      const bool r = __any_sync(0xFFFFFFFFu, x);
+      __syncwarp();
+      return r;
+    } else {
+      uint32_t r;
+      asm volatile(
+          "{\n .reg .pred p, q;\n setp.ne.u32 q, %1, 0;\n barrier.cta.red.or.pred p, %2, %3, q;\n"
+          " selp.u32 %0, 1, 0, p;\n}\n"
+          : "=r"(r)
+          : "r"((uint32_t)x), "r"(g + 1), "n"(GT)
+          : "memory");
+      return r != 0;
+    }
+  }
+};
+
+// Rows are handed out in batches: the first ones to each group by its index, the others by
+// a device counter, claimed ahead of time.  A batch is at most kRowBatch rows (one lane of
+// the group's first warp looks at each; eight keep the end of a long row stream balanced)
+// and few enough that every group gets several.
+constexpr int kRowBatch = 8;
+// threads per SM that the short rows' registers are limited for
+constexpr int kRowThreadsPerSm = 768;
 
 template <int N>
 __device__ __forceinline__ void zero_row(float2 *srow, int jt) {
@@ -96,15 +160,45 @@ __device__ __forceinline__ void x_taps(const KernelParams &kp, float gx, float q
     }
   } else {
 #pragma unroll
-    for (int a = 0; a < WT; ++a) g[a] = kernel_eval(kp, (float)a - kp.half + gx);
+    for (int a = 0; a < WT; ++a) g[a] = kernel_tap(kp, (float)a - kp.half + gx);
+  }
+}
+
+// f(a, G(a - W/2 + g_x)) for every tap a: the unrolled x_taps where the support has an
+// instance of its own (and not EVAL), else each tap evaluated
+template <int WT, bool EVAL, class F>
+__device__ __forceinline__ void for_taps(const KernelParams &kp, float gx, float q, const F &f) {
+  if constexpr (WT > 0 && !EVAL) {
+    float g[WT];
+    x_taps<WT>(kp, gx, q, g);
+#pragma unroll
+    for (int a = 0; a < WT; ++a) f(a, g[a]);
+  } else {
+    const int W = WT > 0 ? WT : kp.support;
+#pragma unroll
+    for (int a = 0; a < W; ++a) f(a, kernel_tap(kp, (float)a - kp.half + gx));
   }
 }
 
 constexpr int kFixedBinCap = 8192;
 // rows whose bound comes from column bins (k_row_bounds); the others' is the sum of their W
-// buckets' magnitudes, loaded with the offsets
+// buckets' magnitudes
 template <int N>
 constexpr bool kBinnedRows = bins_per_row(N) > 1;
+
+// log2(delta / B) of a row shorter than 8192, n_eff the mean contributions in its busiest bin
+// (one bin: all of the row).  The rounding of a tap stays near 2^-28 of the mean magnitude
+// while the bins are sparse, that of a float sum of a few taps, and a cell may hold, before
+// the row is accumulated again, the whole bin of fewer than 16, above that 8 or more mean
+// contributions in phase at weight 1 (taps average a tenth of it).  With 2^-34 of a whole
+// row's magnitude for every count above 256 the error against FP64 at 4096^2 (4.08M
+// visibilities) was 8.7e-6, with this 5.1e-6, with float atomics 5.6e-6.
+__device__ __forceinline__ int log2_unit(float n_eff) {
+  if (n_eff < 16.0f) return -30;
+  if (n_eff < 64.0f) return -32;
+  if (n_eff < 256.0f) return -34;
+  return n_eff < 1024.0f ? -35 : n_eff < 4096.0f ? -36 : -37;
+}
 
 // one tap into the planar row: float atomics, or (FIXED) the tap already in units of the
 // row's quantum (the record's value was scaled by 1/delta once), converted and added as
@@ -132,6 +226,12 @@ __device__ __forceinline__ void add_tap(float *sre, float *sim, int c, float re,
 // fixes the support at compile time.
 __device__ __forceinline__ void cp_async16_rg(uint32_t dst, const void *src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// 4- or 8-byte asynchronous copy
+template <int BYTES>
+__device__ __forceinline__ void cp_async_small(uint32_t dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(BYTES) : "memory");
 }
 
 // The previous row's transformed values, written out while this row is gridded: two
@@ -189,7 +289,7 @@ struct NoPending {
 
 // With FIXED, qscale = 1/delta and gmax the largest |kernel value|: a record whose scaled
 // value times gmax comes within 0.2% of 2^31 (a margin for the rounding of the taps)
-// could saturate a conversion, and sends the row to float atomics like a wrapped sum.
+// could saturate a conversion, and sends the row through again like a wrapped sum.
 template <int N, int WT, bool FIXED, class PEND>
 __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__restrict__ rec,
                                         const uint32_t *bnd, int d_lo, const KernelParams &kp, int jt,
@@ -197,73 +297,51 @@ __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__
   constexpr int TPR = RowCfg<N>::TPR;
   int ovf = 0;
   const uint32_t s_end = bnd[d_lo + 1];
-  if constexpr (WT > 0) {
-    const float q = exp2f(-2.0f * kp.l2c);
-    // this thread's record heads are copied into its own three shared slots two records
-    // ahead (cp.async), so two loads are in flight while a record is gridded
-    const uint32_t slot0 = (uint32_t)__cvta_generic_to_shared(stg);
-    const uint32_t sstep = (uint32_t)(stg_stride * sizeof(RecHead));
-    uint32_t s = bnd[0] + jt;
-    if (s < s_end) cp_async16_rg(slot0, rec + s);
+  const float q = exp2f(-2.0f * kp.l2c);
+  // this thread's record heads are copied into its own three shared slots two records
+  // ahead (cp.async), so two loads are in flight while a record is gridded
+  const uint32_t slot0 = (uint32_t)__cvta_generic_to_shared(stg);
+  const uint32_t sstep = (uint32_t)(stg_stride * sizeof(RecHead));
+  uint32_t s = bnd[0] + jt;
+  if (s < s_end) cp_async16_rg(slot0, rec + s);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  if (s + TPR < s_end) cp_async16_rg(slot0 + sstep, rec + s + TPR);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  int i = 0;  // the thread's records come in increasing order, so do their buckets
+  int cur = 0, nxt = 2;  // slot of this record, slot of the one two ahead
+  for (; s < s_end; s += TPR) {
+    if (s + 2 * TPR < s_end) cp_async16_rg(slot0 + nxt * sstep, rec + s + 2 * TPR);
     asm volatile("cp.async.commit_group;" ::: "memory");
-    if (s + TPR < s_end) cp_async16_rg(slot0 + sstep, rec + s + TPR);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-    int i = 0;  // the thread's records come in increasing order, so do their buckets
-    int cur = 0, nxt = 2;  // slot of this record, slot of the one two ahead
-    for (; s < s_end; s += TPR) {
-      if (s + 2 * TPR < s_end) cp_async16_rg(slot0 + nxt * sstep, rec + s + 2 * TPR);
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      asm volatile("cp.async.wait_group 2;" ::: "memory");
-      const RecHead r = stg[cur * stg_stride];
-      cur = cur == 2 ? 0 : cur + 1;
-      nxt = nxt == 2 ? 0 : nxt + 1;
-      while (i < d_lo && bnd[i + 1] <= s) ++i;  // the last row starting at or before the record
-      // the record's row offset keeps y in [-W/2, W/2): no range test
-      const float y = (float)(d_lo - i) - kp.half + rec_gy(r);
-      const float gy = kp.kind == WST_KERNEL_GAUSS ? exp2f(-y * y * kp.l2c) : kernel_eval(kp, y);
-      float g[WT];
-      x_taps<WT>(kp, rec_gx(r), q, g);
-      const int i0 = rec_i0(r);
-      const float gq = FIXED ? gy * qscale : gy;
-      const float vre = r.vre * gq, vim = r.vim * gq;
-      if (FIXED && fmaxf(fabsf(vre), fabsf(vim)) * gmax >= 0x1.ffp30f) ovf = -1;
-#pragma unroll
-      for (int a = 0; a < WT; ++a) add_tap<FIXED>(sre, sim, i0 + a, vre * g[a], vim * g[a], ovf);
-      pd.write_one(jt);
-    }
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-  } else {
-    const int W = kp.support;
-    for (uint32_t s = bnd[0] + jt; s < s_end; s += TPR) {
-      int i = d_lo;
-      while (s < bnd[i]) --i;
-      const RecHead r = rec_head(rec, s);
-      const float gy = kernel_eval(kp, (float)(d_lo - i) - kp.half + rec_gy(r));
-      const float gx = rec_gx(r);
-      const int i0 = rec_i0(r);
-      const float gq = FIXED ? gy * qscale : gy;
-      const float vre = r.vre * gq, vim = r.vim * gq;
-      if (FIXED && fmaxf(fabsf(vre), fabsf(vim)) * gmax >= 0x1.ffp30f) ovf = -1;
-      for (int a = 0; a < W; ++a) {
-        const float g = kernel_eval(kp, (float)a - kp.half + gx);
-        add_tap<FIXED>(sre, sim, i0 + a, vre * g, vim * g, ovf);
-      }
-      pd.write_one(jt);
-    }
+    asm volatile("cp.async.wait_group 2;" ::: "memory");
+    const RecHead r = stg[cur * stg_stride];
+    cur = cur == 2 ? 0 : cur + 1;
+    nxt = nxt == 2 ? 0 : nxt + 1;
+    while (i < d_lo && bnd[i + 1] <= s) ++i;  // the last row starting at or before the record
+    // the record's row offset keeps y in [-W/2, W/2): no range test
+    const float y = (float)(d_lo - i) - kp.half + rec_gy(r);
+    const float gy = WT > 0 && kp.kind == WST_KERNEL_GAUSS ? exp2f(-y * y * kp.l2c) : kernel_tap(kp, y);
+    const int i0 = rec_i0(r);
+    const float gq = FIXED ? gy * qscale : gy;
+    const float vre = r.vre * gq, vim = r.vim * gq;
+    if (FIXED && fmaxf(fabsf(vre), fabsf(vim)) * gmax >= 0x1.ffp30f) ovf = -1;
+    for_taps<WT, false>(kp, rec_gx(r), q, [&](int a, float g) { add_tap<FIXED>(sre, sim, i0 + a, vre * g, vim * g, ovf); });
+    pd.write_one(jt);
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
   return ovf;
 }
 
-// One non-empty row q of a plane: accumulate, transform (FFT) and write it (with a
-// PendingRow, during the next row's gridding: pd holds the row before this one on entry
-// and this row on return).  Every thread of the row group calls it; it ends with the row
-// buffer free again.
-template <int N, bool FFT, int WT, class PEND>
-__device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const Record *__restrict__ rec,
-                                             const uint32_t *__restrict__ off, int64_t b0, int q, bool nonempty,
-                                             const KernelParams &kp, float2 *__restrict__ orow,
-                                             const float2 *twt, int jt, const float2 *__restrict__ rowbound,
-                                             const float *__restrict__ binmag, float *mag, float gmax, RecHead *stg, int stg_stride, PEND &pd) {
+// One row q of a plane: accumulate, transform (FFT) and write it (with a PendingRow, during
+// the next row's gridding: pd holds the row before this one on entry and this row on
+// return).  bnd[0 .. d_lo + 1]: where the rows j0 = q - d_lo ... q start, and the end; mb:
+// the row's largest bin sum and the total of its bin sums.  Every thread of the row group
+// calls it; it ends with the row buffer free again.
+template <int N, bool FFT, int WT, class PEND, class SYNC>
+__device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, int d_lo, float2 mb,
+                                             const Record *__restrict__ rec, int q, bool nonempty,
+                                             const KernelParams &kp, float2 *__restrict__ orow, const float2 *twt,
+                                             int jt, float gmax, RecHead *stg, int stg_stride, PEND &pd,
+                                             const SYNC &sync) {
   using C = RowCfg<N>;
   constexpr int EPT = C::EPT, TPR = C::TPR;
   constexpr int NST = num_stages(N, EPT);
@@ -272,66 +350,55 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const 
   auto smi = [](int i) { return i + i / EPT; };
   const int W = WT > 0 ? WT : kp.support;
   float *sre = reinterpret_cast<float *>(srow), *sim = sre + N;  // planar accumulation
-  const int d_lo = min(q, W - 1);
-  // the row's largest bin sum and total of the bin sums (k_row_bounds), broadcast
-  float2 mb = make_float2(0.0f, 0.0f);
-  if (nonempty) {
-    for (int i = jt; i <= d_lo + 1; i += TPR) {
-      bnd[i] = off[(b0 + q - d_lo + i) * kColBlocks];
-      if constexpr (!kBinnedRows<N>) mag[i] = i <= d_lo ? __ldg(binmag + b0 + q - d_lo + i) : 0.0f;
-    }
-    if constexpr (kBinnedRows<N>) mb = __ldg(rowbound + b0 + q);
-  }
-  // two groups of the previous row's outputs go out while the offsets load (more, or one
+  // two groups of the previous row's outputs go out before the row is zeroed (more, or one
   // more after the first record heads are requested, measured slower)
   pd.write_one(jt);
   pd.write_one(jt);
   zero_row<N>(srow, jt);
-  __syncthreads();
+  sync();
   // the same decision and quantum in every thread of the row
   const uint32_t cnt = nonempty ? bnd[d_lo + 1] - bnd[0] : 0u;
-  if constexpr (!kBinnedRows<N>) {
-    if (nonempty)
-      for (int i = 0; i <= d_lo; ++i) mb.x += mag[i];
-  }
   const float mmax = mb.x, mtot = mb.y;
   const float bound = mmax * (gmax * gmax);
   // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row (one
   // bin: the row's visibilities)
   const float n_eff = !kBinnedRows<N> ? (float)cnt
                       : mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
-  const bool fixed = nonempty && cnt < (1u << 30) && bound >= 0x1p-90f && bound <= 0x1p+100f &&
+  const bool fixed = nonempty && cnt < (1u << 30) && bound >= 0x1p-87f && bound <= 0x1p+100f &&
                      n_eff <= (float)kFixedBinCap;
   // a bin of fewer than ~64 mean contributions may hold a single tap above B/8: such rows
-  // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range.  A
-  // whole row as one bin spreads over more cells: there the quantum follows the count, so
-  // that it stays near 2^-26 of the mean magnitude (below the rounding of a float sum)
-  // while a cell may still hold 8 to 32 mean contributions in phase, or half the row
+  // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range
   float unit;
-  if constexpr (kBinnedRows<N>) unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
-  else unit = n_eff < 16.0f ? 0x1p-30f : n_eff < 64.0f ? 0x1p-32f : n_eff < 256.0f ? 0x1p-33f : 0x1p-34f;
-  bool fx = fixed;
+  if constexpr (N >= 8192) unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
+  else unit = __int_as_float((127 + log2_unit(n_eff)) << 23);
   int ovf = 0;
   if (nonempty) {
     if (fixed)
       ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, pd);
     else grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, pd);
   }
-  // a tap or a partial sum left the int32 range: accumulate in float (every row of the CTA)
-  const bool redo = __syncthreads_or(ovf < 0);
-  if (redo) {
+  // a tap or a partial sum left the int32 range: once more with delta = B / 2^30, which holds
+  // any row.  (Such a row has a cell of 1/64 of its busiest bin's magnitude or more, whose
+  // rounding in float would be as coarse.  Float atomics here are compare-and-swap loops that
+  // retry for every lane on the same cell, and these are the rows with many on one cell: with
+  // them a 2048^2 image of 1M visibilities on slow tracks spent 600 us in a few rows.)
+  if (sync.any(ovf < 0)) {
     zero_row<N>(srow, jt);
-    __syncthreads();
-    if (nonempty) grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, pd);
-    fx = false;
-    __syncthreads();
+    sync();
+    if (nonempty && fixed) {
+      unit = 0x1p-30f;
+      grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, pd);
+    } else if (nonempty) {
+      grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, pd);
+    }
+    sync();
   }
   pd.write_all(jt);  // the previous row is out before this one's transform takes its place
-  const float delta = fx ? bound * unit : 1.0f;
+  const float delta = fixed ? bound * unit : 1.0f;
   const int *ire = reinterpret_cast<const int *>(sre), *iim = reinterpret_cast<const int *>(sim);
   if constexpr (FFT) {
     float2 v[EPT];
-    if (fx) {
+    if (fixed) {
 #pragma unroll
       for (int b = 0; b < EPT / R0; ++b)
 #pragma unroll
@@ -350,10 +417,10 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const 
           v[b * R0 + r] = make_float2(sg * sre[idx], sg * sim[idx]);
         }
     }
-    __syncthreads();  // natural-order reads done before the padded writes
+    sync();  // natural-order reads done before the padded writes
     const TableTw<N, EPT, TPR, 1> twp{twt, jt};
     stage_compute_f<N, EPT, TPR, 0, 1>(v, jt, twp);
-    middle_stages_f<N, EPT, TPR, 1, 1>(v, jt, srow, smi, twp);
+    middle_stages_f<N, EPT, TPR, 1, 1>(v, jt, srow, smi, twp, sync);
     stage_compute_f<N, EPT, TPR, NST - 1, 1>(v, jt, twp);
     if constexpr (std::is_same_v<PEND, PendingRow<N>>) {
       // kept for the next row's gridding (assigned on every path, so that the old values
@@ -371,125 +438,147 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, uint32_t *bnd, const 
     }
   } else {
     if (orow) {
-      if (fx)
+      if (fixed)
         for (int i = jt; i < N; i += TPR)
           orow[i] = make_float2(delta * __int2float_rn(ire[i]), delta * __int2float_rn(iim[i]));
       else
         for (int i = jt; i < N; i += TPR) orow[i] = make_float2(sre[i], sim[i]);
     }
   }
-  __syncthreads();  // the row buffer is reused by the next row
+  sync();  // the row buffer is reused by the next row
 }
 
-// rows handed out per counter fetch (one row per CTA step); warp 0 scans a batch, one
-// lane per row.  Eight rows keep the end of the kernel's row stream balanced.
-constexpr int kRowBatch = 8;
-
 template <int N, bool FFT, int WT>
-__global__ void __launch_bounds__(RowCfg<N>::THREADS)
+__global__ void __launch_bounds__(GridCfg<N>::THREADS,
+                                  N >= 4096 ? 1 : kRowThreadsPerSm / GridCfg<N>::THREADS)
 k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, int p0, int np,
             KernelParams kp, float2 *__restrict__ out, uint8_t *__restrict__ occ,
             unsigned long long *__restrict__ counter, Tw tw, const float2 *__restrict__ rowbound,
-            const float *__restrict__ binmag, unsigned long long *__restrict__ rows_done) {
-  using C = RowCfg<N>;
-  constexpr int TPR = C::TPR, RPC = C::RPC;
+            const float *__restrict__ binmag, unsigned long long *__restrict__ rows_done, int batch) {
+  using C = GridCfg<N>;
+  constexpr int TPR = C::TPR, GT = C::GT, GR = C::GR, GROUPS = C::GROUPS;
   extern __shared__ __align__(16) float2 sm_rows[];
-  __shared__ long long s_item;
-  __shared__ uint32_t s_bnd[RPC][kMaxSupport + 2];
-  __shared__ float s_mag[RPC][kMaxSupport + 2];
-  __shared__ uint32_t s_gmax;  // largest |kernel value| (FP32 bits)
-  const int rl = threadIdx.x / TPR, jt = threadIdx.x % TPR;
+  const int g = threadIdx.x / GT, gt = threadIdx.x % GT;   // group, thread of the group
+  const int rl = threadIdx.x / TPR, jt = threadIdx.x % TPR;  // row of the CTA, thread of the row
+  const GroupSync<GT, GROUPS> sync{g};
   float2 *srow = sm_rows + rl * C::PADL;
-  float2 *twt = sm_rows + RPC * C::PADL;  // twiddle tables (visible after the first barrier)
+  float2 *twt = sm_rows + C::ROWS * C::PADL;  // twiddle tables (visible after the first barrier)
   // three record-head slots per thread after the tables
   RecHead *stg = reinterpret_cast<RecHead *>(twt + (FFT ? line_table_size<N, C::EPT, TPR>() : 0)) + threadIdx.x;
   const int stg_stride = C::THREADS;
   if constexpr (FFT) fill_line_tables<N, C::EPT, TPR>(twt, tw);
   // G^2 of the fixed-point bound (G = 1 for the Gaussian and the ES kernel, the largest
   // |sample| of a table: linear interpolation stays below it)
-  if (threadIdx.x == 0) s_gmax = __float_as_uint(1.0f);
-  if (kp.kind == WST_KERNEL_TABLE) {
-    __syncthreads();
-    float gm = 0.0f;
-    for (int i = threadIdx.x; i < kp.table_len; i += blockDim.x) gm = fmaxf(gm, fabsf(__ldg(kp.table + i)));
-    if (threadIdx.x == 0) s_gmax = 0u;
-    __syncthreads();
-    atomicMax(&s_gmax, __float_as_uint(gm));
-  }
+  const float gmax = kp.kind == WST_KERNEL_TABLE ? __ldg(kp.table_max) : 1.0f;
   __syncthreads();
-  const float gmax = __uint_as_float(s_gmax);
   const long long total = (long long)np * N;
   const int W = WT > 0 ? WT : kp.support;
-  auto row_empty = [&](long long item) {
-    const int64_t b0 = (int64_t)(p0 + item / N) * N;
-    const int q = (int)(item % N);
-    return off[(b0 + max(0, q - W + 1)) * kColBlocks] == off[(b0 + q + 1) * kColBlocks];
-  };
-  if constexpr (RPC == 1) {
-    // batches of kRowBatch rows: warp 0 finds the non-empty ones (and fills occ), the
-    // CTA then grids and transforms only those; the next batch is fetched meanwhile
-    __shared__ int s_list[kRowBatch], s_cnt;
-    unsigned long long next = 0;
-    // the transforming path writes each row during the next row's gridding
-    std::conditional_t<FFT, PendingRow<N>, NoPending> pd;
-    if constexpr (FFT) {
+  const long long group0 = (long long)blockIdx.x * GROUPS + g, ngroups = (long long)gridDim.x * GROUPS;
+  if constexpr (GR == 1) {
+    // batches of rows (a power of two, so that a batch lies in one plane).  The bucket
+    // offsets its rows need, q0 - W + 1 ... q0 + batch, and the rows' bounds are copied
+    // (cp.async) while the batch before it is worked on; the group's first warp then lists
+    // the non-empty rows (and fills occ), and the group grids and transforms only those.
+    __shared__ long long s_item[GROUPS];
+    __shared__ int s_list[GROUPS][kRowBatch], s_cnt[GROUPS];
+    __shared__ uint32_t s_off[GROUPS][2][kRowBatch + kMaxSupport + 1];
+    __shared__ __align__(8) float2 s_rb[GROUPS][2][kRowBatch];
+    const uint32_t off_sm = (uint32_t)__cvta_generic_to_shared(&s_off[g][0][0]);
+    const uint32_t rb_sm = (uint32_t)__cvta_generic_to_shared(&s_rb[g][0][0]);
+    auto fetch = [&](long long base, int buf) {  // by the first warp
+      if (base < total) {
+        const int64_t b0 = (int64_t)(p0 + base / N) * N;
+        const int q0 = (int)(base % N);
+        const int j = q0 - (W - 1) + gt;  // entry gt: where row j starts (unused below the plane)
+        if (gt < W + batch && j >= 0)
+          cp_async_small<4>(off_sm + (uint32_t)(buf * (kRowBatch + kMaxSupport + 1) + gt) * 4u,
+                            off + (b0 + j) * kColBlocks);
+        if (gt < batch) cp_async_small<8>(rb_sm + (uint32_t)(buf * kRowBatch + gt) * 8u, rowbound + b0 + q0 + gt);
+      }
+    };
+    // the transforming path of long rows writes each row during the next row's gridding
+    std::conditional_t<FFT && kPending<N>, PendingRow<N>, NoPending> pd;
+    if constexpr (FFT && kPending<N>) {
       pd.next = PendingRow<N>::NCH;
       pd.orow = nullptr;
     }
-    if (threadIdx.x == 0) next = atomicAdd(counter, (unsigned long long)kRowBatch);
-    while (true) {
-      if (threadIdx.x == 0) {
-        s_item = (long long)next;
-        next = atomicAdd(counter, (unsigned long long)kRowBatch);
-      }
-      __syncthreads();
-      const long long base = s_item;
-      if (base >= total) break;
-      if (threadIdx.x < 32) {
-        const long long item = base + threadIdx.x;
-        const bool valid = (int)threadIdx.x < kRowBatch && item < total;
-        const bool nonempty = valid && !row_empty(item);
-        if (valid) occ[item] = nonempty ? 1 : 0;
+    long long next = group0 * batch;  // first warp: the next batch, its data under way
+    long long after = (ngroups + group0) * batch;  // lane 0: the one after it
+    if (gt < 32) fetch(next, 0);
+    for (int buf = 0;; buf ^= 1) {
+      if (gt < 32) {
+        const long long base = next;
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        __syncwarp();
+        next = __shfl_sync(0xFFFFFFFFu, after, 0);
+        if (gt == 0) after = 2 * ngroups * batch + (long long)atomicAdd(counter, (unsigned long long)batch);
+        fetch(next, buf ^ 1);
+        const bool valid = gt < batch && base + gt < total;
+        const int skip = max(0, W - 1 - ((int)(base % N) + gt));  // rows below the plane
+        const bool nonempty = valid && s_off[g][buf][gt + skip] != s_off[g][buf][gt + W];
+        if (valid) occ[base + gt] = nonempty ? 1 : 0;
         // plain gridding hands the planes to the caller: it also lists the empty rows,
         // which get zeros; the column pass reads only occupied rows of transformed planes
         const bool listed = FFT ? nonempty : valid;
         const unsigned m = __ballot_sync(0xFFFFFFFFu, listed);
-        if (listed) s_list[__popc(m & ((1u << threadIdx.x) - 1u))] = threadIdx.x * 2 + (nonempty ? 1 : 0);
-        if (threadIdx.x == 0) s_cnt = __popc(m);
+        if (listed) s_list[g][__popc(m & ((1u << gt) - 1u))] = gt * 2 + (nonempty ? 1 : 0);
+        if (gt == 0) {
+          s_cnt[g] = __popc(m);
+          s_item[g] = base;
+        }
         if (rows_done) {  // the occupied rows of the batch, for the caller's statistics
           const unsigned occupied = __ballot_sync(0xFFFFFFFFu, nonempty);
-          if (threadIdx.x == 0 && occupied) atomicAdd(rows_done, (unsigned long long)__popc(occupied));
+          if (gt == 0 && occupied) atomicAdd(rows_done, (unsigned long long)__popc(occupied));
         }
       }
-      __syncthreads();
-      const int cnt = s_cnt;
-      for (int k = 0; k < cnt; ++k) {
-        const int e = s_list[k];
-        const long long item = base + (e >> 1);
-        const int pl = (int)(item / N), q = (int)(item % N);
-        grid_one_row<N, FFT, WT>(srow, s_bnd[0], rec, off, (int64_t)(p0 + pl) * N, q, e & 1, kp,
-                                 out + ((int64_t)pl * N + q) * N, twt, jt, rowbound, binmag, s_mag[0], gmax, stg, stg_stride, pd);
-      }
-    }
-    pd.write_all(jt);  // the CTA's last row
-  } else {
-    while (true) {
-      if (threadIdx.x == 0) s_item = (long long)atomicAdd(counter, (unsigned long long)RPC);
-      __syncthreads();
-      const long long base = s_item;
-      __syncthreads();
+      sync();
+      const long long base = s_item[g];
       if (base >= total) break;
-      const long long item = base + rl;
+      const int cnt = s_cnt[g];
+      for (int k = 0; k < cnt; ++k) {
+        const int e = s_list[g][k], r = e >> 1;
+        const long long item = base + r;
+        const int pl = (int)(item / N), q = (int)(item % N);
+        const int d_lo = min(q, W - 1);
+        grid_one_row<N, FFT, WT>(srow, &s_off[g][buf][r + W - 1 - d_lo], d_lo, s_rb[g][buf][r], rec, q, e & 1, kp,
+                                 out + ((int64_t)pl * N + q) * N, twt, jt, gmax, stg, stg_stride, pd, sync);
+      }
+      if (cnt == 0) sync();  // s_item, s_cnt and the list are read before they are written again
+    }
+    pd.write_all(jt);  // the group's last row
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  } else {
+    __shared__ uint32_t s_bnd[C::ROWS][kMaxSupport + 2];
+    __shared__ float s_mag[C::ROWS][kMaxSupport + 2];
+    static_assert(!kBinnedRows<N>, "one bin per row");
+    long long next = group0 * GR;
+    while (true) {
+      const long long base = __shfl_sync(0xFFFFFFFFu, next, 0);  // a group is one warp here
+      if (base >= total) break;
+      if (gt == 0) next = ngroups * GR + (long long)atomicAdd(counter, (unsigned long long)GR);
+      const long long item = base + rl % GR;
       const bool valid = item < total;
       const int pl = valid ? (int)(item / N) : 0;
       const int q = valid ? (int)(item % N) : 0;
-      const bool empty = !valid || row_empty(item);
+      const int64_t b0 = (int64_t)(p0 + pl) * N;
+      const int d_lo = min(q, W - 1);
+      for (int i = jt; i <= d_lo + 1; i += TPR) {
+        s_bnd[rl][i] = off[(b0 + q - d_lo + i) * kColBlocks];
+        s_mag[rl][i] = i <= d_lo ? __ldg(binmag + b0 + q - d_lo + i) : 0.0f;
+      }
+      __syncwarp();
+      const bool empty = !valid || s_bnd[rl][0] == s_bnd[rl][d_lo + 1];
       if (valid && jt == 0) occ[item] = empty ? 0 : 1;
       if (rows_done && valid && jt == 0 && !empty) atomicAdd(rows_done, 1ull);
-      float2 *orow = valid && (!FFT || !empty) ? out + ((int64_t)pl * N + q) * N : nullptr;
-      NoPending none;
-      grid_one_row<N, FFT, WT>(srow, s_bnd[rl], rec, off, (int64_t)(p0 + pl) * N, q, !empty, kp, orow, twt, jt,
-                               rowbound, binmag, s_mag[rl], gmax, stg, stg_stride, none);
+      if (!FFT || !__all_sync(0xFFFFFFFFu, empty)) {
+        float2 mb = make_float2(0.0f, 0.0f);
+        for (int i = 0; i <= d_lo; ++i) mb.x += s_mag[rl][i];
+        float2 *orow = valid && (!FFT || !empty) ? out + ((int64_t)pl * N + q) * N : nullptr;
+        NoPending none;
+        grid_one_row<N, FFT, WT>(srow, s_bnd[rl], d_lo, mb, rec, q, !empty, kp, orow, twt, jt, gmax, stg, stg_stride,
+                                 none, sync);
+      }
+      __syncwarp();
     }
   }
 }
@@ -497,56 +586,86 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
 // -------------------------------------------------------------------------------------
 // adjoint: row FFT^H of the adjoint plane + degridding / kernel gradient
 // -------------------------------------------------------------------------------------
-template <int N, bool KGRAD>
-__global__ void __launch_bounds__(RowCfg<N>::THREADS)
+// x[t] added to at[t][offset] for every t with at[t] set (shared memory).  A shared float
+// atomic is a compare-and-swap loop of its own, and a run of them a serial chain of round
+// trips; here the first attempts of all T go out together and only what lost a race (another
+// lane or an equal address in the same run) is added the usual way.
+template <int T>
+__device__ __forceinline__ void add_all(float *const (&at)[T], const float (&x)[T], int offset) {
+  uint32_t old[T], got[T];
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (at[t]) old[t] = __float_as_uint(*(volatile float *)(at[t] + offset));
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (at[t])
+      got[t] = atomicCAS(reinterpret_cast<uint32_t *>(at[t] + offset), old[t],
+                         __float_as_uint(__uint_as_float(old[t]) + x[t]));
+#pragma unroll
+  for (int t = 0; t < T; ++t)
+    if (at[t] && got[t] != old[t]) atomicAdd(at[t] + offset, x[t]);
+}
+
+// Rows are shared out as in k_grid_rows.  Degridding adds a record's row sum to its place in
+// sorted order (vacc, one 8-byte vector reduction; adjacent lanes hold adjacent records, so a
+// warp's reductions fall on whole sectors) and k_unsort hands the sums back in the caller's
+// order.  Two scalar reductions per record and row at the caller's index, the taps each
+// evaluated on their own and the records of each bucket shared out separately took 5.64 ms
+// for 10M visibilities on 16 planes of 8192^2.
+template <int N, int WT, bool KGRAD>
+__global__ void __launch_bounds__(GroupCfg<N, KGRAD ? 256 : 128>::THREADS,
+                                  N >= 16384 || (KGRAD && N == 8192) ? 1 : KGRAD || N == 8192 ? 2 : N == 4096 ? 3
+                                  : 1024 / GroupCfg<N>::THREADS)
 k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec,
                const uint32_t *__restrict__ off, int p0, int np, KernelParams kp,
-               float2 *__restrict__ dvis, float *__restrict__ dtab,
-               unsigned long long *__restrict__ counter, Tw tw) {
-  using C = RowCfg<N>;
-  constexpr int EPT = C::EPT, TPR = C::TPR, RPC = C::RPC;
+               float2 *__restrict__ vacc, float *__restrict__ dtab,
+               unsigned long long *__restrict__ counter, Tw tw, int batch, bool dvis_order) {
+  using C = GroupCfg<N, KGRAD ? 256 : 128>;
+  constexpr int EPT = C::EPT, TPR = C::TPR, GT = C::GT, GR = C::GR, GROUPS = C::GROUPS;
   constexpr int NST = num_stages(N, EPT);
   constexpr int R0 = stage_radix(N, EPT, 0);
   constexpr int RL = stage_radix(N, EPT, NST - 1);
   extern __shared__ __align__(16) float2 sm_rows[];
-  __shared__ long long s_item;
-  float2 *twt = sm_rows + RPC * C::PADL;  // twiddle tables (visible after the first barrier)
+  __shared__ long long s_item[GROUPS];
+  __shared__ int s_list[GROUPS][kRowBatch], s_cnt[GROUPS];
+  __shared__ uint32_t s_bnd[C::ROWS][kMaxSupport + 2];
+  float2 *twt = sm_rows + C::ROWS * C::PADL;  // twiddle tables (visible after the first barrier)
   fill_line_tables<N, C::EPT, TPR>(twt, tw);
   float *ptab = reinterpret_cast<float *>(twt + line_table_size<N, C::EPT, C::TPR>());  // KGRAD partial table
+  const int g = threadIdx.x / GT, gt = threadIdx.x % GT;
   const int rl = threadIdx.x / TPR, jt = threadIdx.x % TPR;
+  const GroupSync<GT, GROUPS> sync{g};
   float2 *srow = sm_rows + rl * C::PADL;
+  uint32_t *bnd = s_bnd[rl];
   auto smi = [](int i) { return i + i / EPT; };
   const long long total = (long long)np * N;
-  const int W = kp.support;
+  const int W = WT > 0 ? WT : kp.support;
   if (KGRAD) {
     for (int i = threadIdx.x; i < kp.table_len; i += blockDim.x) ptab[i] = 0.0f;
   }
-  while (true) {
-    if (threadIdx.x == 0) s_item = (long long)atomicAdd(counter, (unsigned long long)RPC);
-    __syncthreads();
-    const long long base = s_item;
-    __syncthreads();
-    if (base >= total) break;
-    const long long item = base + rl;
-    const bool valid = item < total;
-    const int pl = valid ? (int)(item / N) : 0;
-    const int q = valid ? (int)(item % N) : 0;
+  __syncthreads();
+  auto row_empty = [&](long long item) {
+    const int64_t b0 = (int64_t)(p0 + item / N) * N;
+    const int q = (int)(item % N);
+    return off[(b0 + max(0, q - W + 1)) * kColBlocks] == off[(b0 + q + 1) * kColBlocks];
+  };
+  auto do_row = [&](long long item, bool nonempty) {
+    const int pl = (int)(item / N), q = (int)(item % N);
     const int64_t b0 = (int64_t)(p0 + pl) * N;
-    const bool empty = !valid || off[(b0 + max(0, q - W + 1)) * kColBlocks] == off[(b0 + q + 1) * kColBlocks];
-    if constexpr (RPC == 1) {
-      if (empty) continue;  // nobody reads this row
-    }
+    const int d_lo = min(q, W - 1);
     const float2 *grow = planes + ((int64_t)pl * N + q) * N;
     float2 v[EPT];
 #pragma unroll
     for (int b = 0; b < EPT / R0; ++b)
 #pragma unroll
-      for (int r = 0; r < R0; ++r) v[b * R0 + r] = grow[in_index<N, EPT, TPR, 0>(jt, b, r)];
+      for (int r = 0; r < R0; ++r)
+        v[b * R0 + r] = nonempty ? __ldcs(grow + in_index<N, EPT, TPR, 0>(jt, b, r)) : make_float2(0.0f, 0.0f);
+    for (int i = jt; i <= d_lo + 1; i += TPR) bnd[i] = nonempty ? off[(b0 + q - d_lo + i) * kColBlocks] : 0u;
     const TableTw<N, EPT, TPR, -1> twp{twt, jt};
     stage_compute_f<N, EPT, TPR, 0, -1>(v, jt, twp);
-    middle_stages_f<N, EPT, TPR, 1, -1>(v, jt, srow, smi, twp);
+    middle_stages_f<N, EPT, TPR, 1, -1>(v, jt, srow, smi, twp, sync);
     stage_compute_f<N, EPT, TPR, NST - 1, -1>(v, jt, twp);
-    __syncthreads();  // every padded read done before the natural-order writes
+    sync();  // every padded read done before the natural-order writes
 #pragma unroll
     for (int b = 0; b < EPT / RL; ++b)
 #pragma unroll
@@ -556,62 +675,121 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
         if ((idx + q) & 1) x = make_float2(-x.x, -x.y);
         srow[idx] = x;
       }
-    __syncthreads();
-    if (valid && !empty) {
-      for (int d = 0; d < W && q - d >= 0; ++d) {
-        const uint32_t s0 = off[(b0 + q - d) * kColBlocks], s1 = off[(b0 + q - d + 1) * kColBlocks];
-        const float ty = (float)d - kp.half;
-        for (uint32_t s = s0 + jt; s < s1; s += TPR) {
-          const RecHead rc = rec_head(rec, s);
-          const float targ_y = ty + rec_gy(rc);
-          const float gy = kernel_eval(kp, targ_y);
-          const float gx0 = rec_gx(rc);
-          const float2 *cell = srow + rec_i0(rc);
-          if (!KGRAD) {
-            float are = 0.0f, aim = 0.0f;
-            for (int a = 0; a < W; ++a) {
-              const float g = kernel_eval(kp, (float)a - kp.half + gx0);
-              are = fmaf(g, cell[a].x, are);
-              aim = fmaf(g, cell[a].y, aim);
-            }
-            const uint2 tail = __ldg(reinterpret_cast<const uint2 *>(rec + s) + 2);  // index, weight
-            const float wt = __uint_as_float(tail.y) * gy;
-            const uint32_t j = tail.x;
-            atomicAdd(&dvis[j].x, wt * are);
-            atomicAdd(&dvis[j].y, wt * aim);
-          } else {
-            // c_a = Re(conj(gh[q, i0 + a]) (w V)); x-profile tap a gets c_a G_y(d), the
-            // y-profile tap d gets sum_a c_a G_x(a); each is split over the two table
-            // samples bracketing the tap's argument
-            float sum_cx = 0.0f;
-            for (int a = 0; a < W; ++a) {
-              const float targ = (float)a - kp.half + gx0;
+    sync();
+    // the row's records are one contiguous range, split evenly over its threads (one head
+    // in flight); bnd[i] is where row j0 = q - d_lo + i starts
+    const uint32_t s_end = bnd[d_lo + 1];
+    uint32_t s = bnd[0] + jt;
+    RecHead nxt{};
+    if (s < s_end) nxt = rec_head(rec, s);
+    int i = 0;
+    for (; s < s_end; s += TPR) {
+      const RecHead rc = nxt;
+      if (s + TPR < s_end) nxt = rec_head(rec, s + TPR);
+      while (i < d_lo && bnd[i + 1] <= s) ++i;
+      const float targ_y = (float)(d_lo - i) - kp.half + rec_gy(rc);
+      const float gy = kernel_tap(kp, targ_y);
+      const float gx0 = rec_gx(rc);
+      const float2 *cell = srow + rec_i0(rc);
+      if constexpr (!KGRAD) {
+        float are = 0.0f, aim = 0.0f;
+        // the taps one by one, as the table gradient takes them: the image's corners enter with
+        // the grid correction's 1e3 to 1e5 and cancel here, which magnifies any other rounding
+        for_taps<WT, true>(kp, gx0, 0.0f, [&](int a, float gx) {
+          const float2 c = cell[a];
+          are = fmaf(gx, c.x, are);
+          aim = fmaf(gx, c.y, aim);
+        });
+        const float wt = __uint_as_float(__ldg(reinterpret_cast<const uint32_t *>(rec + s) + 5)) * gy;
+        const uint32_t at = dvis_order ? __ldg(&rec[s].index) : s;
+        asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(vacc + at), "f"(wt * are), "f"(wt * aim)
+                     : "memory");
+      } else {
+        // c_a = Re(conj(gh[q, i0 + a]) (w V)); x-profile tap a gets c_a G_y(d), the
+        // y-profile tap d gets sum_a c_a G_x(a); each is split over the two table
+        // samples bracketing the tap's argument
+        float sum_cx = 0.0f;
+        constexpr int T = WT > 0 ? WT : 4;  // taps at a time
+        auto split = [&](float targ, float x, float *&at, float &lo, float &hi) {
+          const float pos = (targ + kp.half) * kp.table_scale;
+          int k = (int)floorf(pos);
+          k = max(0, min(k, kp.table_len - 2));
+          const float f = pos - (float)k;
+          at = ptab + k;
+          lo = x * (1.0f - f);
+          hi = x * f;
+          return fmaf(f, __ldg(kp.table + k + 1) - __ldg(kp.table + k), __ldg(kp.table + k));  // G(targ)
+        };
+        for (int a0 = 0; a0 < W; a0 += T) {
+          float *at[T];
+          float lo[T], hi[T];
+#pragma unroll
+          for (int t = 0; t < T; ++t) {
+            const int a = a0 + t;
+            if (WT > 0 || a < W) {
               const float2 c = cell[a];
               const float cr = c.x * rc.vre + c.y * rc.vim;
-              sum_cx = fmaf(cr, kernel_eval(kp, targ), sum_cx);
-              const float pos = (targ + kp.half) * kp.table_scale;
-              int i = (int)floorf(pos);
-              i = max(0, min(i, kp.table_len - 2));
-              const float f = pos - (float)i;
-              atomicAdd(&ptab[i], cr * gy * (1.0f - f));
-              atomicAdd(&ptab[i + 1], cr * gy * f);
+              sum_cx = fmaf(cr, split((float)a - kp.half + gx0, cr * gy, at[t], lo[t], hi[t]), sum_cx);
+            } else {
+              at[t] = nullptr;
             }
-            const float pos = (targ_y + kp.half) * kp.table_scale;
-            int i = (int)floorf(pos);
-            i = max(0, min(i, kp.table_len - 2));
-            const float f = pos - (float)i;
-            atomicAdd(&ptab[i], sum_cx * (1.0f - f));
-            atomicAdd(&ptab[i + 1], sum_cx * f);
           }
+          add_all<T>(at, lo, 0);
+          add_all<T>(at, hi, 1);
         }
+        float *at[1];
+        float lo[1], hi[1];
+        split(targ_y, sum_cx, at[0], lo[0], hi[0]);
+        add_all<1>(at, lo, 0);
+        add_all<1>(at, hi, 1);
       }
     }
-    __syncthreads();
+    sync();  // the row buffer is reused by the next row
+  };
+  const long long group0 = (long long)blockIdx.x * GROUPS + g, ngroups = (long long)gridDim.x * GROUPS;
+  long long next = group0 * (GR == 1 ? batch : GR);
+  if constexpr (GR == 1) {
+    while (true) {
+      if (gt == 0) {
+        s_item[g] = next;
+        next = ngroups * batch + (long long)atomicAdd(counter, (unsigned long long)batch);
+      }
+      sync();
+      const long long base = s_item[g];
+      if (base >= total) break;
+      if (gt < 32) {  // the rows of the batch that somebody reads
+        const bool listed = gt < batch && base + gt < total && !row_empty(base + gt);
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, listed);
+        if (listed) s_list[g][__popc(m & ((1u << gt) - 1u))] = gt;
+        if (gt == 0) s_cnt[g] = __popc(m);
+      }
+      sync();
+      const int cnt = s_cnt[g];
+      for (int k = 0; k < cnt; ++k) do_row(base + s_list[g][k], true);
+    }
+  } else {
+    while (true) {
+      const long long base = __shfl_sync(0xFFFFFFFFu, next, 0);  // a group is one warp here
+      if (base >= total) break;
+      if (gt == 0) next = ngroups * GR + (long long)atomicAdd(counter, (unsigned long long)GR);
+      const long long item = base + rl % GR;
+      const bool nonempty = item < total && !row_empty(item);
+      if (__any_sync(0xFFFFFFFFu, nonempty)) do_row(item < total ? item : base, nonempty);
+    }
   }
   if (KGRAD) {
     __syncthreads();
     for (int i = threadIdx.x; i < kp.table_len; i += blockDim.x)
       if (ptab[i] != 0.0f) atomicAdd(&dtab[i], ptab[i]);
+  }
+}
+
+// the sums of the sorted records back in the caller's order
+__global__ void k_unsort(const float2 *__restrict__ vacc, const Record *__restrict__ rec,
+                         const uint32_t *__restrict__ n_kept, float2 *__restrict__ dvis) {
+  const uint32_t n = *n_kept;
+  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
+    dvis[__ldcs(&rec[s].index)] = __ldcs(vacc + s);
   }
 }
 
@@ -626,57 +804,66 @@ static Tw tw_half(const wst_plan_s *p) {
   return t;
 }
 
-template <class K>
-static cudaError_t persistent_grid(wst_plan_s *p, K kern, int threads, size_t smem, int &grid) {
+// the grid of a persistent row kernel: every resident CTA, no more than there are rows for;
+// and the rows of a batch, so that each group gets eight batches or more of a long stream
+template <class C, class K>
+static cudaError_t persistent_grid(wst_plan_s *p, K kern, size_t smem, int64_t rows, int &grid, int &batch) {
   // always raised to the request: the 48 KB default counts the kernel's static shared
   // memory too, so a dynamic request just under 48 KB can already exceed it
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   int per_sm = 0, sms = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::THREADS, smem);
   if (e != cudaSuccess) return e;
   e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
   if (e != cudaSuccess) return e;
-  grid = (per_sm > 0 ? per_sm : 1) * sms;
+  const int64_t resident = (int64_t)(per_sm > 0 ? per_sm : 1) * sms, need = (rows + C::ROWS - 1) / C::ROWS;
+  grid = (int)(resident < need ? resident : need);
+  const int64_t b = rows / ((int64_t)grid * C::GROUPS * 8);
+  for (batch = 1; 2 * batch <= b && 2 * batch <= kRowBatch;) batch *= 2;
   return cudaSuccess;
 }
 
 template <int N, bool FFT>
 static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) {
-  using C = RowCfg<N>;
+  using C = GridCfg<N>;
   // the imaging path has the common supports unrolled
-  auto kern = !FFT ? k_grid_rows<N, FFT, 0>
-              : p->cfg.support == 7 ? k_grid_rows<N, FFT, 7>
-              : p->cfg.support == 8 ? k_grid_rows<N, FFT, 8> : k_grid_rows<N, FFT, 0>;
-  const size_t smem = sizeof(float2) * (C::RPC * C::PADL + (FFT ? line_table_size<N, C::EPT, C::TPR>() : 0)) +
+  auto kern = k_grid_rows<N, FFT, 0>;
+  if constexpr (FFT) {
+    if (p->cfg.support == 7) kern = k_grid_rows<N, FFT, 7>;
+    else if (p->cfg.support == 8) kern = k_grid_rows<N, FFT, 8>;
+  }
+  const size_t smem = sizeof(float2) * (C::ROWS * C::PADL + (FFT ? line_table_size<N, C::EPT, C::TPR>() : 0)) +
                       3 * C::THREADS * sizeof(RecHead);
-  int grid = 0;
-  cudaError_t e = persistent_grid(p, kern, C::THREADS, smem, grid);
+  int grid = 0, batch = 0;
+  cudaError_t e = persistent_grid<C>(p, kern, smem, (int64_t)np * N, grid, batch);
   if (e != cudaSuccess) return e;
   unsigned long long *counter = p->W_.counters + CNT_WORK;
   e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), p->stream);
   if (e != cudaSuccess) return e;
   kern<<<grid, C::THREADS, smem, p->stream>>>(p->W_.records, p->W_.offsets, p0, np, kernel_params(p), out,
                                              p->W_.occ, counter, tw_half(p), p->W_.rowbound, p->W_.binmag,
-                                             FFT ? p->W_.counters + CNT_ROWS : nullptr);
+                                             FFT ? p->W_.counters + CNT_ROWS : nullptr, batch);
   return cudaGetLastError();
 }
 
 template <int N, bool KGRAD>
-static cudaError_t launch_rows_adjoint(wst_plan_s *p, int p0, int np, const float2 *planes, float2 *dvis,
-                                       float *dtab) {
-  using C = RowCfg<N>;
-  auto kern = k_rows_adjoint<N, KGRAD>;
-  const size_t smem = sizeof(float2) * (C::RPC * C::PADL + line_table_size<N, C::EPT, C::TPR>()) +
+static cudaError_t launch_rows_adjoint(wst_plan_s *p, int p0, int np, const float2 *planes, float2 *dvis, float *dtab) {
+  using C = GroupCfg<N, KGRAD ? 256 : 128>;
+  auto kern = k_rows_adjoint<N, 0, KGRAD>;
+  if (p->cfg.support == 8) kern = k_rows_adjoint<N, 8, KGRAD>;
+  if constexpr (!KGRAD)
+    if (p->cfg.support == 7) kern = k_rows_adjoint<N, 7, KGRAD>;
+  const size_t smem = sizeof(float2) * (C::ROWS * C::PADL + line_table_size<N, C::EPT, C::TPR>()) +
                       (KGRAD ? sizeof(float) * p->cfg.ktable_len : 0);
-  int grid = 0;
-  cudaError_t e = persistent_grid(p, kern, C::THREADS, smem, grid);
+  int grid = 0, batch = 0;
+  cudaError_t e = persistent_grid<C>(p, kern, smem, (int64_t)np * N, grid, batch);
   if (e != cudaSuccess) return e;
   unsigned long long *counter = p->W_.counters + CNT_WORK;
   e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), p->stream);
   if (e != cudaSuccess) return e;
   kern<<<grid, C::THREADS, smem, p->stream>>>(planes, p->W_.records, p->W_.offsets, p0, np, kernel_params(p),
-                                             dvis, dtab, counter, tw_half(p));
+                                             dvis ? dvis : p->W_.vacc, dtab, counter, tw_half(p), batch, dvis != nullptr);
   return cudaGetLastError();
 }
 
@@ -722,6 +909,33 @@ cudaError_t rows_adjoint(wst_plan_s *p, int p0, int p1, const float2 *planes, fl
     WST_N_SWITCH(p->n, CALL_D)
 #undef CALL_D
   }
+}
+
+// occ of a chunk's rows, as k_grid_rows leaves it, for the adjoint column pass
+__global__ void k_row_occ(const uint32_t *__restrict__ off, int64_t b0, int64_t rows, int n, int W,
+                          uint8_t *__restrict__ occ) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= rows) return;
+  const int64_t b = b0 + i;
+  occ[i] = off[(b - min((int)(i % n), W - 1)) * kColBlocks] != off[(b + 1) * kColBlocks];
+}
+
+cudaError_t row_occupancy(wst_plan_s *p, int p0, int p1) {
+  const int64_t rows = (int64_t)(p1 - p0) * p->n;
+  if (rows <= 0) return cudaSuccess;
+  k_row_occ<<<(unsigned)((rows + 255) / 256), 256, 0, p->stream>>>(p->W_.offsets, (int64_t)p0 * p->n, rows, p->n, p->W,
+                                                                   p->W_.occ);
+  p->launches += 1;
+  return cudaGetLastError();
+}
+
+cudaError_t unsort_sums(wst_plan_s *p, float2 *dvis) {
+  if (p->n_vis <= 0) return cudaSuccess;
+  const int64_t blocks = (p->n_vis + 255) / 256;
+  k_unsort<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, p->stream>>>(
+      p->W_.vacc, p->W_.records, p->W_.offsets + p->n_buckets, dvis);
+  p->launches += 1;
+  return cudaGetLastError();
 }
 
 }  // namespace wst

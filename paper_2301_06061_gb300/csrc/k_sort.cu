@@ -502,30 +502,49 @@ __global__ void k_scatter(const float2 *__restrict__ vis, const float *__restric
 }
 
 // Per grid row q of every (image, plane): over the column bins b, the largest and the
-// total of M_b = sum of bin b of the buckets j0 = q - W + 1 ... q (one warp per row; rows
-// no visibility reaches get zeros).  The fused row kernel takes its fixed-point quantum
-// from them.
-__global__ void k_row_bounds(const float *__restrict__ binmag, const uint32_t *__restrict__ offsets,
-                             int64_t n_rows, int n, int nb, int W, float2 *__restrict__ rowbound) {
+// total of M_b = sum of bin b of the buckets j0 = q - W + 1 ... q (rows no visibility reaches
+// get zeros).  The fused row kernel takes its fixed-point quantum from them.  A warp takes
+// kBoundRows consecutive rows, a lane a bin: the rows share their buckets, so each bin is
+// read (kBoundRows + W - 1) / kBoundRows times instead of W.
+constexpr int kBoundRows = 8;
+template <int WMAX>
+__global__ void __launch_bounds__(256)
+k_row_bounds(const float *__restrict__ binmag, const uint32_t *__restrict__ offsets, int64_t n_rows, int n, int nb,
+             int W, float2 *__restrict__ rowbound) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < n_rows; r += warps) {
-    const int q = (int)(r % n);
-    const int d_lo = min(q, W - 1);
-    float mmax = 0.0f, mtot = 0.0f;
-    if (offsets[(r - d_lo) * kColBlocks] != offsets[(r + 1) * kColBlocks]) {
+  for (int64_t r0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * kBoundRows; r0 < n_rows;
+       r0 += warps * kBoundRows) {  // n is a multiple of kBoundRows: the rows are one plane's
+    const int q0 = (int)(r0 % n);
+    float mmax[kBoundRows] = {}, mtot[kBoundRows] = {};
+    if (offsets[(r0 - min(q0, W - 1)) * kColBlocks] != offsets[(r0 + kBoundRows) * kColBlocks]) {
       for (int b = lane; b < nb; b += 32) {
-        float m = 0.0f;
-        for (int d = 0; d <= d_lo; ++d) m += binmag[(size_t)(r - d) * nb + b];
-        mmax = fmaxf(mmax, m);
-        mtot += m;
+        float x[kBoundRows + WMAX - 1];  // bin b of rows r0 - (WMAX - 1) ... r0 + kBoundRows - 1
+#pragma unroll
+        for (int k = 0; k < kBoundRows + WMAX - 1; ++k) {
+          const int d = k - (WMAX - 1);
+          x[k] = (d > -W && q0 + d >= 0) ? __ldg(binmag + (r0 + d) * nb + b) : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < kBoundRows; ++k) {
+          float m = 0.0f;
+#pragma unroll
+          for (int d = 0; d < WMAX; ++d)
+            if (d < W) m += x[k + WMAX - 1 - d];
+          mmax[k] = fmaxf(mmax[k], m);
+          mtot[k] += m;
+        }
       }
-      for (int o = 16; o > 0; o >>= 1) {
-        mmax = fmaxf(mmax, __shfl_xor_sync(0xFFFFFFFFu, mmax, o));
-        mtot += __shfl_xor_sync(0xFFFFFFFFu, mtot, o);
-      }
+#pragma unroll
+      for (int k = 0; k < kBoundRows; ++k)
+        for (int o = 16; o > 0; o >>= 1) {
+          mmax[k] = fmaxf(mmax[k], __shfl_xor_sync(0xFFFFFFFFu, mmax[k], o));
+          mtot[k] += __shfl_xor_sync(0xFFFFFFFFu, mtot[k], o);
+        }
     }
-    if (lane == 0) rowbound[r] = make_float2(mmax, mtot);
+#pragma unroll
+    for (int k = 0; k < kBoundRows; ++k)
+      if (lane == k) rowbound[r0 + k] = make_float2(mmax[k], mtot[k]);
   }
 }
 
@@ -599,8 +618,9 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
   p->launches += 1;
   if (nb > 1) {
     const int64_t n_rows = p->n_buckets / kColBlocks;
-    k_row_bounds<<<grid_for(n_rows * 32, 256, 152 * 8), 256, 0, s>>>(ws.binmag, ws.offsets, n_rows, p->n, nb, p->W,
-                                                                     ws.rowbound);
+    const auto bounds = p->W <= 8 ? k_row_bounds<8> : k_row_bounds<kMaxSupport>;
+    bounds<<<grid_for(n_rows * (32 / kBoundRows), 256, 152 * 8), 256, 0, s>>>(ws.binmag, ws.offsets, n_rows, p->n, nb,
+                                                                              p->W, ws.rowbound);
     p->launches += 1;
   }
   return cudaGetLastError();

@@ -20,6 +20,7 @@ KernelParams kernel_params(const wst_plan_s *p) {
   k.table_len = p->cfg.ktable_len;
   k.table_scale = (k.kind == WST_KERNEL_TABLE) ? (float)((double)(p->cfg.ktable_len - 1) / p->W) : 0.0f;
   k.tap_table = p->ktap;
+  k.table_max = p->kmax;
   k.per_cell = p->ktap ? (p->cfg.ktable_len - 1) / p->W : 0;
   return k;
 }
@@ -108,8 +109,20 @@ __global__ void k_kernel_nodes(double *nodes, int P, int kind, int W, double par
 }
 
 __global__ void __launch_bounds__(kCorrThreads) k_correction(float *corr, int n, const double *__restrict__ nodes,
-                                                             int P, int W) {
+                                                             int P, int W, const float *__restrict__ tab,
+                                                             float *__restrict__ tab_max) {
   const int k = blockIdx.x;  // nu = k / n, 0 <= k <= n/2
+  if (k > n / 2) {  // a table's last block: its largest |sample|, for the gridder's bound
+    __shared__ uint32_t s_max;
+    if (threadIdx.x == 0) s_max = 0u;
+    __syncthreads();
+    float m = 0.0f;
+    for (int i = threadIdx.x; i <= P; i += kCorrThreads) m = fmaxf(m, fabsf(__ldg(tab + i)));
+    atomicMax(&s_max, __float_as_uint(m));
+    __syncthreads();
+    if (threadIdx.x == 0) *tab_max = __uint_as_float(s_max);
+    return;
+  }
   const double turn = (double)k * (double)W / ((double)n * (double)P);  // 2 nu h/2: half turns per node
   double acc = 0.0, s, c, ds, dc;
   sincospi(turn * (double)threadIdx.x, &s, &c);
@@ -145,7 +158,8 @@ cudaError_t build_tables(wst_plan_s *p) {
 cudaError_t build_correction(wst_plan_s *p) {
   const int P = node_panels(p);
   k_kernel_nodes<<<(P + 256) / 256, 256, 0, p->stream>>>(p->knodes, P, p->cfg.kernel, p->W, p->cfg.kparam, p->ktable);
-  k_correction<<<p->n / 2 + 1, kCorrThreads, 0, p->stream>>>(p->corr, p->n, p->knodes, P, p->W);
+  k_correction<<<p->n / 2 + 1 + (p->ktable ? 1 : 0), kCorrThreads, 0, p->stream>>>(p->corr, p->n, p->knodes, P, p->W,
+                                                                                   p->ktable, p->kmax);
   p->launches += 2;
   return cudaGetLastError();
 }

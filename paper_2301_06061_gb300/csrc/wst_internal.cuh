@@ -18,11 +18,10 @@ constexpr int kColBlocks = 1;    // sub-buckets per row (by tap-start column; a 
 constexpr uint32_t kDropKey = 0xFFFFFFFFu;
 // Column bins of the fixed-point gridder's bound: for every row bucket (image, plane, j0)
 // the sort sums max(|Re|, |Im|) of the weighted values whose W taps reach each bin of
-// kBinCols columns.  Rows shorter than kBinnedMinN carry few enough visibilities for one
-// bin, the whole row: a bound of at most a few thousand contributions needs no finer one
-// (k_rowgrid.cu), and 8192-cell bins cost memory, atomics and a pass of their own.
+// kBinCols columns.  The shortest rows have one bin, the whole row: their calls are bound by
+// launches, and a bound over a few bins would cost one more (k_row_bounds).
 constexpr int kBinCols = 64, kBinShift = 6;
-constexpr int kBinnedMinN = 8192;
+constexpr int kBinnedMinN = 512;
 __host__ __device__ constexpr int bins_per_row(int n) { return n >= kBinnedMinN ? n / kBinCols : 1; }
 
 // counters[] slots in the workspace
@@ -78,6 +77,7 @@ struct KernelParams {
   float table_scale;   // (L-1)/W
   const float2 *tap_table;  // TABLE with L - 1 = W * per_cell: [per_cell][W] pairs (T[a pc + i], T[a pc + i + 1])
   int per_cell;
+  const float *table_max;   // TABLE: the largest |sample|
 };
 
 struct Workspace {
@@ -94,6 +94,7 @@ struct Workspace {
   float2 *rowbound;    // binned rows only: (largest bin sum, total of the bin sums) over the W buckets
   float2 *planes;      // chunk of planes
   float2 *comp;        // Kahan compensation image [batch][N*N]
+  float2 *vacc;        // per sorted record: the degridded sum before its weight
   size_t bytes;
 };
 
@@ -117,6 +118,7 @@ struct wst_plan_s {
   float2 *l2ff = nullptr;    // l_a^2 as float-float
   double *l2d = nullptr;     // l_a^2 in FP64 (WST_FLAG_FP64_SCREEN)
   float *ktable = nullptr;   // TABLE kernel samples
+  float *kmax = nullptr;     // TABLE: the largest |sample| (k_correction)
   float2 *ktap = nullptr;    // TABLE samples in tap-major pairs (see KernelParams::tap_table)
   double *wrange = nullptr;  // per image: w_lo, scale = n_w/(w_hi-w_lo), dw, w_hi
   float4 *wrange_ff = nullptr;  // per image: w_lo and scale as float-float pairs
@@ -253,8 +255,9 @@ __device__ __forceinline__ float2 cis_cycles_d(double phi) {
 // ------------------------------------------------------------------------------------
 // convolution kernel G (section 2, Eq. 3)
 // ------------------------------------------------------------------------------------
-__device__ __forceinline__ float kernel_eval(const KernelParams &k, float x) {
-  if (x < -k.half || x > k.half) return 0.0f;
+// G at a tap's position: x = a - W/2 + g, 0 <= a < W, g in [0, 1), is within [-W/2, W/2] (the
+// rounded sum cannot pass W/2)
+__device__ __forceinline__ float kernel_tap(const KernelParams &k, float x) {
   if (k.kind == WST_KERNEL_GAUSS) return expf(-x * x * k.inv2s2);
   if (k.kind == WST_KERNEL_ES) {
     float z = x * k.two_over_w;
@@ -335,12 +338,18 @@ int64_t scan_tmp_words(int64_t n);
 
 // k_rowgrid.cu
 cudaError_t grid_rows(wst_plan_s *p, int p0, int p1, float2 *out, bool fft);
+// adjoint rows.  dtab: the table gradient is added to it; else degridding, the sums added to
+// dvis in the caller's order or (dvis null) to W_.vacc in sorted order (unsort_sums hands
+// them over once every plane has been through)
 cudaError_t rows_adjoint(wst_plan_s *p, int p0, int p1, const float2 *planes, float2 *dvis, float *dtab);
+cudaError_t row_occupancy(wst_plan_s *p, int p0, int p1);  // W_.occ of planes [p0, p1)
+cudaError_t unsort_sums(wst_plan_s *p, float2 *dvis);
 
 // k_fft.cu
 cudaError_t fft_rows(wst_plan_s *p, float2 *planes, int nplanes, int dir, bool presign,
                      bool postsign);
-// occ (nullable): per (plane of the call, row) 0 if the row is known to be zero
+// occ (nullable): per (plane of the call, row) 0 if the row is known to be zero (forward) or
+// not to be read afterwards (twiddle_first)
 cudaError_t fft_cols_a(wst_plan_s *p, float2 *planes, int nplanes, int dir, bool twiddle_first,
                        const uint8_t *occ);
 // forward: accumulate planes [p0,p1) (stored at planes[0..]) into image (+comp); range_start
