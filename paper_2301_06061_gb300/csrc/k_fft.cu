@@ -232,8 +232,8 @@ k_cols_a(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict__ 
     for (int r = 0; r < R0; ++r) {
       const int i = in_index<LB, EPT, TPL, 0>(jt, b, r);
       // rows the gridder left empty are zero: do not read them
-      float2 x = (occ && !occ[(size_t)blockIdx.z * n + a + A * i]) ? make_float2(0.0f, 0.0f)
-                                                                     : base[(size_t)i * rstride];
+      float2 x = (!TW_FIRST && occ && !occ[(size_t)blockIdx.z * n + a + A * i]) ? make_float2(0.0f, 0.0f)
+                                                                                  : base[(size_t)i * rstride];
       if (TW_FIRST) x = cmul(x, twiddle(tw, a * i, DIR));
       v[b * R0 + r] = x;
     }
@@ -250,6 +250,8 @@ k_cols_a(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict__ 
       const int c = out_index<LB, EPT, TPL, NST - 1>(jt, b, r);
       float2 x = v[b * RL + r];
       if (!TW_FIRST) x = cmul(x, twiddle(tw, a * c, DIR));
+      // adjoint: rows no visibility reaches are not read, so not written
+      if (TW_FIRST && occ && !occ[(size_t)blockIdx.z * n + a + A * c]) continue;
       base[(size_t)c * rstride] = x;
     }
 }
@@ -273,7 +275,9 @@ __device__ __forceinline__ void cp_async_wait() {
 // keeps two CTAs per SM with the deeper ring.  A warp covers 32 columns at one line
 // position: shared-memory accesses are conflict-free without padding and twiddles are
 // warp-uniform.  The factors w_N^{a c} of a tile come from a shared table filled with the
-// tile (three in rotation), each factor evaluated by sincospi.
+// tile (three in rotation), each factor evaluated by sincospi.  The adjoint (TW_FIRST) reads
+// every row but writes only those a visibility reaches, the ones the row pass reads; their
+// flags are in a shared table of the tile too.
 template <int LB, int DIR, bool TW_FIRST>
 __global__ void __launch_bounds__(LB / 16 * 32, 512 / (LB / 16 * 32))
 k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict__ occ, int nplanes) {
@@ -285,6 +289,7 @@ k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict_
   static_assert(PIECES % THREADS == 0, "pieces");
   __shared__ __align__(16) float2 stage[3][LB * CB];
   __shared__ float2 s_tw[3][LB];    // w_N^{DIR a c}, c < LB, of the tiles in flight
+  __shared__ uint8_t s_out[TW_FIRST ? 3 : 1][TW_FIRST ? LB : 1];  // adjoint: output rows' flags
   const int A = n / LB;
   const int lg_bands = 31 - __clz(n / CB), lg_A = 31 - __clz(A);
   const int total = nplanes << (lg_bands + lg_A);
@@ -299,8 +304,16 @@ k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict_
 #pragma unroll
     for (int k = 0; k < PPT; ++k) {
       const int i = (threadIdx.x + k * THREADS) / (CB / 2);
-      f[k] = (t >= total || !occ) ? 1u : (uint32_t)occ[(size_t)z * n + a + A * i];
+      f[k] = (TW_FIRST || t >= total || !occ) ? 1u : (uint32_t)occ[(size_t)z * n + a + A * i];
     }
+  };
+  // the flag of output row threadIdx.x of a tile, loaded a tile ahead like the inputs'
+  auto load_out = [&](int t) -> uint32_t {
+    const int a = (t >> lg_bands) & (A - 1), z = t >> (lg_bands + lg_A);
+    return (!TW_FIRST || !occ || t >= total || threadIdx.x >= LB) ? 1u : (uint32_t)occ[(size_t)z * n + a + A * (int)threadIdx.x];
+  };
+  auto put_out = [&](int slot, uint32_t f) {
+    if (TW_FIRST && threadIdx.x < LB) s_out[slot][threadIdx.x] = (uint8_t)f;
   };
   auto issue = [&](int t, float2 *buf, const uint32_t (&f)[PPT]) {
     const int band = t & ((1 << lg_bands) - 1);
@@ -330,12 +343,13 @@ k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict_
   // tiles it and it + 1 in flight before the loop; tile it + 2 is issued after the first
   // barrier of tile it, into the slot of tile it - 1
   load_flags(t, f0);
-  if (t < total) { issue(t, stage[0], f0); fill_tw(t, s_tw[0]); }
+  if (t < total) { issue(t, stage[0], f0); fill_tw(t, s_tw[0]); put_out(0, load_out(t)); }
   cp_async_commit();
   load_flags(t + G, f0);
-  if (t + G < total) { issue(t + G, stage[1], f0); fill_tw(t + G, s_tw[1]); }
+  if (t + G < total) { issue(t + G, stage[1], f0); fill_tw(t + G, s_tw[1]); put_out(TW_FIRST ? 1 : 0, load_out(t + G)); }
   cp_async_commit();
   load_flags(t + 2 * G, f1);
+  uint32_t fo = load_out(t + 2 * G);
   for (int it = 0; t < total; ++it, t += G) {
     const int band = t & ((1 << lg_bands) - 1);
     const int a = (t >> lg_bands) & (A - 1), z = t >> (lg_bands + lg_A);
@@ -345,9 +359,11 @@ k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict_
     if (t + 2 * G < total) {
       issue(t + 2 * G, stage[(it + 2) % 3], f1);
       fill_tw(t + 2 * G, s_tw[(it + 2) % 3]);
+      put_out(TW_FIRST ? (it + 2) % 3 : 0, fo);
     }
     cp_async_commit();
     load_flags(t + 3 * G, f1);
+    fo = load_out(t + 3 * G);
     float2 *buf = stage[it % 3];
     float2 v[EPT];
 #pragma unroll
@@ -375,6 +391,7 @@ k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict_
         const int c = jt + b * TPL + 16 * r;
         float2 x = v[b * R1 + r];
         if (!TW_FIRST) x = cmul(x, tws[c]);
+        if (TW_FIRST && !s_out[it % 3][c]) continue;
         __stcs(&dst[(size_t)c * rstride], x);
       }
   }
@@ -532,15 +549,27 @@ __device__ __forceinline__ void flush_pixel(float2 *im, float2 *cp, size_t o, fl
   }
 }
 
+// The images of a call are independent: blockIdx.z takes ipz of them each, so that small
+// images in one call still fill the SMs (one block per tile walked all images before).
+// Narrows [p0, p1) to the block's planes and returns how many planes before them it skips.
+__device__ __forceinline__ int image_split(int &p0, int &p1, int n_w, int ipz) {
+  const int first = p0, ia = p0 / n_w + (int)blockIdx.z * ipz;
+  p0 = max(p0, ia * n_w);
+  p1 = min(p1, (ia + ipz) * n_w);
+  return p0 - first;
+}
+
 template <int LA, bool FP64S, bool CROP>
 __global__ void __launch_bounds__(ColCfg<LA>::THREADS, ColCfg<LA>::THREADS >= 32 ? 512 / ColCfg<LA>::THREADS : 1)
 k_cols_b_acc(const float2 *__restrict__ planes, int p0, int p1, int n_w, Tw tw,
              int n, ScreenCtx sc, float2 *__restrict__ image, float2 *__restrict__ comp, int flags,
-             int n_img_arg, int crop_arg) {
+             int n_img_arg, int crop_arg, int ipz) {
   // an image smaller than the grid (CROP) is its central n_img x n_img from grid index
   // crop; otherwise both are compile-time facts, which keeps the registers of the
   // plain kernel free for the transform
   const int n_img = CROP ? n_img_arg : n, crop = CROP ? crop_arg : 0;
+  planes += (size_t)image_split(p0, p1, n_w, ipz) * n * n;
+  if (p0 >= p1) return;
   using C = ColCfg<LA>;
   constexpr int EPT = C::EPT, TPL = C::TPL;
   constexpr int NST = num_stages(LA, EPT);
@@ -654,8 +683,10 @@ template <int LA, bool FP64S, bool CROP>
 __global__ void __launch_bounds__(LA / 16 * kCB, LA == 128 ? 3 : 6)
 k_cols_b16(const float2 *__restrict__ planes, int p0, int p1, int n_w, Tw tw,
            int n, ScreenCtx sc, float2 *__restrict__ image, float2 *__restrict__ comp, int flags,
-           int n_img_arg, int crop_arg) {
+           int n_img_arg, int crop_arg, int ipz) {
   const int n_img = CROP ? n_img_arg : n, crop = CROP ? crop_arg : 0;  // as in k_cols_b_acc
+  planes += (size_t)image_split(p0, p1, n_w, ipz) * n * n;
+  if (p0 >= p1) return;
   constexpr int EPT = 16, TPL = LA / EPT, THREADS = TPL * kCB, R1 = LA / 16;
   static_assert(num_stages(LA, EPT) == 2 && stage_radix(LA, EPT, 1) == R1, "two stages");
   __shared__ __align__(16) float2 stage_buf[2][LA * kCB];
@@ -807,11 +838,13 @@ template <int LA, bool FP64S, bool CROP>
 __global__ void __launch_bounds__(LA / 16 * kCB, LA == 128 ? 3 : 6)
 k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, Tw tw, int n, ScreenCtx sc,
              float2 *__restrict__ image, float2 *__restrict__ comp, int flags, int n_img_arg, int crop_arg,
-             unsigned long long *__restrict__ err, unsigned long long wait_ns, int first_lo, int last_hi) {
+             unsigned long long *__restrict__ err, unsigned long long wait_ns, int first_lo, int last_hi, int ipz) {
   // an image starts its sum in this call if its first plane is at or after first_lo (p0,
   // or below every plane when the call starts the requested range) and finishes it if its
   // last plane is before last_hi (p1, or above every plane when the call ends the range)
   const int n_img = CROP ? n_img_arg : n, crop = CROP ? crop_arg : 0;  // as in k_cols_b_acc
+  const int z0 = image_split(p0, p1, n_w, ipz);  // the block's first plane in the tensor map
+  if (p0 >= p1) return;
   constexpr int EPT = 16, TPL = LA / EPT, THREADS = TPL * kCB, R1 = LA / 16;
   static_assert(num_stages(LA, EPT) == 2 && stage_radix(LA, EPT, 1) == R1, "two stages");
   constexpr uint32_t kTileBytes = LA * kCB * sizeof(float2);
@@ -860,7 +893,7 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
   int issued = 0;  // thread 0: planes (indices within the call) whose tile copy is issued
   auto issue = [&](int q) {
     const int slot = q % kColsBRing;
-    tma_load_tile3d(ring0 + (uint32_t)slot * kTileBytes, &tmap, 2 * col0, LA * c, q, mbar0 + 8u * slot, kTileBytes);
+    tma_load_tile3d(ring0 + (uint32_t)slot * kTileBytes, &tmap, 2 * col0, LA * c, z0 + q, mbar0 + 8u * slot, kTileBytes);
   };
   if (threadIdx.x == 0)
     for (; issued < kColsBRing && issued < nplanes; ++issued) issue(issued);
@@ -993,25 +1026,82 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
 // ---------------------------------------------------------------------------------
 // pass CB^H (adjoint): image tile -> planes; sign, correction and conjugate screen fused
 // ---------------------------------------------------------------------------------
+// stages S .. last of a length-LA line: exchange `turn` goes through buffer turn mod 2 (a
+// buffer's readers have passed the next exchange's barrier before it is written again)
+template <int LA, int S, class SMI>
+__device__ __forceinline__ void bh_stages(float2 (&v)[ColCfg<LA>::EPT], int jt, float2 (*sm)[LA * ColCfg<LA>::PADW],
+                                          int turn, SMI smi, const float2 *twid, int tstride) {
+  constexpr int EPT = ColCfg<LA>::EPT, TPL = ColCfg<LA>::TPL;
+  if constexpr (S < num_stages(LA, EPT)) {
+    constexpr int RP = stage_radix(LA, EPT, S - 1), R = stage_radix(LA, EPT, S);
+    float2 *buf = sm[turn & 1];
+#pragma unroll
+    for (int b = 0; b < EPT / RP; ++b)
+#pragma unroll
+      for (int r = 0; r < RP; ++r) buf[smi(out_index<LA, EPT, TPL, S - 1>(jt, b, r))] = v[b * RP + r];
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < EPT / R; ++b)
+#pragma unroll
+      for (int r = 0; r < R; ++r) v[b * R + r] = buf[smi(in_index<LA, EPT, TPL, S>(jt, b, r))];
+#pragma unroll
+    for (int b = 0; b < EPT / R; ++b) {
+#pragma unroll
+      for (int r = 1; r < R; ++r)
+        v[b * R + r] = cmul(v[b * R + r], twid[(stage_tw_offset<LA, EPT, S>() + b * (R - 1) + r - 1) * tstride]);
+      dft<R, -1>(&v[b * R]);
+    }
+    bh_stages<LA, S + 1>(v, jt, sm, turn + 1, smi, twid, tstride);
+  }
+}
+
 // An image smaller than the grid (oversampled grid: the image is the central n_img x
 // n_img from grid index crop) enters zero-padded: the adjoint of the forward crop.
+//
+// Bound by the plane writes, if there are warps enough to cover the exchange: the image
+// tile and the running screens are in registers, the steps in thread-private shared slots,
+// the stage twiddles in a shared table (one row per line position), and the exchanges
+// alternate between two buffers, one barrier each.  With the steps and twiddle loads in
+// the way (141 registers: 8 warps per SM at LA = 128, four barriers per plane) 16 planes of
+// 8192^2 took 4.14 ms.  The arithmetic is that of the plain stages in the same order: the
+// grid correction multiplies the corners by up to 1e5 here and they cancel in the
+// degridded values, which would show any other rounding.
+template <int LA>
+struct BhCfg {
+  static constexpr int CTAS = 768 / ColCfg<LA>::THREADS > 24 ? 24 : 768 / ColCfg<LA>::THREADS;  // resident per SM
+};
 template <int LA, bool FP64S>
-__global__ void __launch_bounds__(ColCfg<LA>::THREADS)
+__global__ void __launch_bounds__(ColCfg<LA>::THREADS, BhCfg<LA>::CTAS)
 k_cols_bh(const float2 *__restrict__ dimage, int p0, int p1, int n_w, Tw tw,
-          int n, ScreenCtx sc, int correct, float2 *__restrict__ planes, int n_img, int crop) {
+          int n, ScreenCtx sc, int correct, float2 *__restrict__ planes, int n_img, int crop, int ppz) {
   using C = ColCfg<LA>;
-  constexpr int EPT = C::EPT, TPL = C::TPL;
+  constexpr int EPT = C::EPT, TPL = C::TPL, THREADS = C::THREADS;
   constexpr int NST = num_stages(LA, EPT);
   constexpr int RL = stage_radix(LA, EPT, NST - 1);
   constexpr int R0 = stage_radix(LA, EPT, 0);
-  __shared__ float2 sm[LA * C::PADW];
+  constexpr int NTW = total_tw_count<LA, EPT>() > 0 ? total_tw_count<LA, EPT>() : 1;
+  __shared__ float2 sm[2][LA * C::PADW];
+  __shared__ float2 s_step[EPT][THREADS];  // conj of each input's per-plane screen step
+  __shared__ float2 s_twid[NTW][TPL];
   const int B = n / LA;
   const int col = threadIdx.x % kCB, jt = threadIdx.x / kCB;
   const int c = blockIdx.y;
   const int kp = blockIdx.x * kCB + col;
+  const int first = p0;  // plane at planes[0]
+  p0 += (int)blockIdx.z * ppz;
+  p1 = min(p1, p0 + ppz);
   auto smi = [col](int i) { return i * C::PADW + col; };
+  if constexpr (NST > 1) {
+    if (threadIdx.x < TPL) {
+      float2 t[NTW];
+      all_twiddles<LA, EPT, TPL, -1>(t, threadIdx.x, tw, B);
+#pragma unroll
+      for (int i = 0; i < NTW; ++i) s_twid[i][threadIdx.x] = t[i];
+    }
+    __syncthreads();
+  }
   // inputs of the first stage: element d <-> image row kq = c + B d
-  float2 dv[EPT], scr[EPT], stp[EPT];
+  float2 dv[EPT], scr[EPT];
   int img_loaded = -1, pstart = p0;
   for (int P = p0; P < p1; ++P) {
     const int img = P / n_w;
@@ -1019,48 +1109,44 @@ k_cols_bh(const float2 *__restrict__ dimage, int p0, int p1, int n_w, Tw tw,
       const float2 *im = dimage + (size_t)img * n_img * n_img;
       const bool col_in = kp >= crop && kp < crop + n_img;
 #pragma unroll
-      for (int b = 0; b < EPT / R0; ++b)
-#pragma unroll
-        for (int r = 0; r < R0; ++r) {
-          const int kq = c + B * in_index<LA, EPT, TPL, 0>(jt, b, r);
-          dv[b * R0 + r] = (col_in && kq >= crop && kq < crop + n_img)
-                               ? im[(size_t)(kq - crop) * n_img + (kp - crop)]
-                               : make_float2(0.0f, 0.0f);
-        }
+      for (int e = 0; e < EPT; ++e) {
+        const int kq = c + B * in_index<LA, EPT, TPL, 0>(jt, e / R0, e % R0);
+        dv[e] = (col_in && kq >= crop && kq < crop + n_img) ? im[(size_t)(kq - crop) * n_img + (kp - crop)]
+                                                            : make_float2(0.0f, 0.0f);
+      }
       img_loaded = img;
       pstart = P;
     }
     if ((P - pstart) % kAnchor == 0) {
 #pragma unroll
-      for (int b = 0; b < EPT / R0; ++b)
-#pragma unroll
-        for (int r = 0; r < R0; ++r) {
-          const int kq = c + B * in_index<LA, EPT, TPL, 0>(jt, b, r);
-          float f = ((kq + kp) & 1) ? -1.0f : 1.0f;
-          if (correct) f *= sc.corr[kp] * sc.corr[kq];
-          float2 a, st;
-          screen_anchor<FP64S>(sc, kp, kq, P, img, f, a, st);
-          scr[b * R0 + r] = make_float2(a.x, -a.y);  // conjugate screen
-          stp[b * R0 + r] = make_float2(st.x, -st.y);
+      for (int e = 0; e < EPT; ++e) {
+        const int kq = c + B * in_index<LA, EPT, TPL, 0>(jt, e / R0, e % R0);
+        float f = ((kq + kp) & 1) ? -1.0f : 1.0f;
+        if (correct) f *= sc.corr[kp] * sc.corr[kq];
+        float2 a, st;
+        if (P == pstart) {
+          screen_anchor<FP64S, true>(sc, kp, kq, P, img, f, a, st);
+          s_step[e][threadIdx.x] = make_float2(st.x, -st.y);
+        } else {
+          screen_anchor<FP64S, false>(sc, kp, kq, P, img, f, a, st);
         }
+        scr[e] = make_float2(a.x, -a.y);  // conjugate screen
+      }
     }
     float2 v[EPT];
 #pragma unroll
     for (int e = 0; e < EPT; ++e) {
       v[e] = cmul(dv[e], scr[e]);
-      scr[e] = cmul(scr[e], stp[e]);
+      scr[e] = cmul(scr[e], s_step[e][threadIdx.x]);
     }
-    stage_compute<LA, EPT, TPL, 0, -1>(v, jt, tw, B);
-    if constexpr (NST > 1) {
-      middle_stages<LA, EPT, TPL, 1, -1>(v, jt, sm, smi, tw, B);
-      stage_compute<LA, EPT, TPL, NST - 1, -1>(v, jt, tw, B);
-    }
-    float2 *base = planes + (size_t)(P - p0) * n * n + (size_t)(LA * c) * n + kp;
+#pragma unroll
+    for (int b = 0; b < EPT / R0; ++b) dft<R0, -1>(&v[b * R0]);
+    if constexpr (NST > 1) bh_stages<LA, 1>(v, jt, sm, (P - p0) * (NST - 1), smi, &s_twid[0][jt], TPL);
+    float2 *base = planes + (size_t)(P - first) * n * n + (size_t)(LA * c) * n + kp;
 #pragma unroll
     for (int b = 0; b < EPT / RL; ++b)
 #pragma unroll
-      for (int r = 0; r < RL; ++r) base[(size_t)out_index<LA, EPT, TPL, NST - 1>(jt, b, r) * n] = v[b * RL + r];
-    if constexpr (NST > 1) __syncthreads();
+      for (int r = 0; r < RL; ++r) __stcs(base + (size_t)out_index<LA, EPT, TPL, NST - 1>(jt, b, r) * n, v[b * RL + r]);
   }
 }
 
@@ -1230,32 +1316,41 @@ static bool plane_tile_map(CUtensorMap *m, const float2 *planes, int n, int npla
 
 template <int LA, bool FP64S, bool CROP>
 static void launch_cols_b_variant(wst_plan_s *p, const float2 *planes, int p0, int p1, float2 *image,
-                                  float2 *comp, int flags) {
-  // the grid's column bands that hold image columns, every row block
+                                  float2 *comp, int flags, int sms) {
+  // the grid's column bands that hold image columns, every row block; and, where these are
+  // fewer than about eight per resident CTA slot, the images split over blockIdx.z
   dim3 grd((p->crop + p->n_img + kCB - 1) / kCB - p->crop / kCB, p->n / LA);
-  if constexpr (LA == 64 || LA == 128) {
+  const int imgs = (p1 - 1) / p->n_w - p0 / p->n_w + 1, tiles = (int)(grd.x * grd.y);
+  const int want = (sms * 8 * (384 / LA) + tiles - 1) / tiles;
+  const int ipz = (imgs + want - 1) / want;
+  grd.z = (imgs + ipz - 1) / ipz;
+  if constexpr (LA >= 64) {
     CUtensorMap map;
-    if (plane_tile_map(&map, planes, p->n, p1 - p0, LA))
+    if (plane_tile_map(&map, planes, p->n, p1 - p0, LA)) {
       k_cols_b_tma<LA, FP64S, CROP><<<grd, LA / 16 * kCB, 0, p->stream>>>(
           map, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), image, comp, flags, p->n_img, p->crop,
           p->W_.counters + CNT_ERROR, p->wait_ns, (flags & ACC_RANGE_START) ? -1 : p0,
-          (flags & ACC_RANGE_END) ? 0x7FFFFFFF : p1);
-    else
-      k_cols_b16<LA, FP64S, CROP><<<grd, LA / 16 * kCB, 0, p->stream>>>(
-          planes, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), image, comp, flags, p->n_img, p->crop);
+          (flags & ACC_RANGE_END) ? 0x7FFFFFFF : p1, ipz);
+      return;
+    }
+    k_cols_b16<LA, FP64S, CROP><<<grd, LA / 16 * kCB, 0, p->stream>>>(
+        planes, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), image, comp, flags, p->n_img, p->crop, ipz);
   } else
     k_cols_b_acc<LA, FP64S, CROP><<<grd, ColCfg<LA>::THREADS, 0, p->stream>>>(
-        planes, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), image, comp, flags, p->n_img, p->crop);
+        planes, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), image, comp, flags, p->n_img, p->crop, ipz);
 }
 
 template <int LA>
 static cudaError_t launch_cols_b(wst_plan_s *p, const float2 *planes, int p0, int p1, float2 *image,
                                  float2 *comp, int flags) {
   const bool fp64 = fp64_screen(p), crop = p->crop != 0;
-  if (fp64 && crop) launch_cols_b_variant<LA, true, true>(p, planes, p0, p1, image, comp, flags);
-  else if (fp64) launch_cols_b_variant<LA, true, false>(p, planes, p0, p1, image, comp, flags);
-  else if (crop) launch_cols_b_variant<LA, false, true>(p, planes, p0, p1, image, comp, flags);
-  else launch_cols_b_variant<LA, false, false>(p, planes, p0, p1, image, comp, flags);
+  int sms = 0;
+  const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+  if (e != cudaSuccess) return e;
+  if (fp64 && crop) launch_cols_b_variant<LA, true, true>(p, planes, p0, p1, image, comp, flags, sms);
+  else if (fp64) launch_cols_b_variant<LA, true, false>(p, planes, p0, p1, image, comp, flags, sms);
+  else if (crop) launch_cols_b_variant<LA, false, true>(p, planes, p0, p1, image, comp, flags, sms);
+  else launch_cols_b_variant<LA, false, false>(p, planes, p0, p1, image, comp, flags, sms);
   return cudaGetLastError();
 }
 
@@ -1280,16 +1375,29 @@ cudaError_t fft_cols_b_accumulate(wst_plan_s *p, const float2 *planes, int p0, i
   return cudaErrorInvalidValue;
 }
 
+template <int LA, bool FP64S>
+static void launch_cols_bh_variant(wst_plan_s *p, const float2 *dimage, int p0, int p1, float2 *planes, int correct,
+                                   int sms) {
+  // every tile; the runs of kAnchor planes split over blockIdx.z where the tiles alone leave
+  // resident slots empty, as many runs to a block as that takes
+  dim3 grd(p->n / kCB, p->n / LA);
+  const int tiles = (int)(grd.x * grd.y), slots = sms * BhCfg<LA>::CTAS, np = p1 - p0;
+  int z = slots / tiles, runs = (np + kAnchor - 1) / kAnchor;
+  if (p->batch > 1 || z < 1) z = 1;  // (an image's first plane starts a run)
+  const int ppz = (runs + z - 1) / z * kAnchor;
+  grd.z = (np + ppz - 1) / ppz;
+  k_cols_bh<LA, FP64S><<<grd, ColCfg<LA>::THREADS, 0, p->stream>>>(
+      dimage, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), correct, planes, p->n_img, p->crop, ppz);
+}
+
 template <int LA>
 static cudaError_t launch_cols_bh(wst_plan_s *p, const float2 *dimage, int p0, int p1, float2 *planes,
                                   bool correct) {
-  dim3 grd(p->n / kCB, p->n / LA);
-  if (fp64_screen(p))
-    k_cols_bh<LA, true><<<grd, ColCfg<LA>::THREADS, 0, p->stream>>>(
-        dimage, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), correct ? 1 : 0, planes, p->n_img, p->crop);
-  else
-    k_cols_bh<LA, false><<<grd, ColCfg<LA>::THREADS, 0, p->stream>>>(
-        dimage, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), correct ? 1 : 0, planes, p->n_img, p->crop);
+  int sms = 0;
+  const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+  if (e != cudaSuccess) return e;
+  if (fp64_screen(p)) launch_cols_bh_variant<LA, true>(p, dimage, p0, p1, planes, correct ? 1 : 0, sms);
+  else launch_cols_bh_variant<LA, false>(p, dimage, p0, p1, planes, correct ? 1 : 0, sms);
   return cudaGetLastError();
 }
 

@@ -507,7 +507,8 @@ wst_status wst_degrid(wst_plan p, const void *dimage, void *dvis, uint32_t flags
   for (int p0 = 0; p0 < p->n_planes; p0 += p->chunk) {
     const int p1 = (p0 + p->chunk < p->n_planes) ? p0 + p->chunk : p->n_planes;
     WST_CUDA(p, fft_cols_bh_from_image(p, (const float2 *)dimage, p0, p1, planes, correct), "cols B^H");
-    WST_CUDA(p, fft_cols_a(p, planes, p1 - p0, -1, true, nullptr), "cols A^H");
+    WST_CUDA(p, row_occupancy(p, p0, p1), "row occupancy");
+    WST_CUDA(p, fft_cols_a(p, planes, p1 - p0, -1, true, p->W_.occ), "cols A^H");
     WST_CUDA(p, rows_adjoint(p, p0, p1, planes, sorted ? nullptr : (float2 *)dvis, nullptr),
              "rows^H + degrid");
   }
@@ -527,7 +528,8 @@ wst_status wst_kernel_grad(wst_plan p, const void *dimage, float *dtable, uint32
   for (int p0 = 0; p0 < p->n_planes; p0 += p->chunk) {
     const int p1 = (p0 + p->chunk < p->n_planes) ? p0 + p->chunk : p->n_planes;
     WST_CUDA(p, fft_cols_bh_from_image(p, (const float2 *)dimage, p0, p1, planes, false), "cols B^H");
-    WST_CUDA(p, fft_cols_a(p, planes, p1 - p0, -1, true, nullptr), "cols A^H");
+    WST_CUDA(p, row_occupancy(p, p0, p1), "row occupancy");
+    WST_CUDA(p, fft_cols_a(p, planes, p1 - p0, -1, true, p->W_.occ), "cols A^H");
     WST_CUDA(p, rows_adjoint(p, p0, p1, planes, nullptr, dtable), "rows^H + kernel gradient");
   }
   return WST_OK;
