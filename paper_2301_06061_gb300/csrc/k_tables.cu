@@ -71,12 +71,12 @@ __global__ void k_l2(float2 *l2ff, double *l2d, int n, double dl) {
 // them), and k_correction sums c_j cos(2 pi nu j h/2) for each nu >= 0; -nu has the same.
 //
 // Bound: the FP64 pipe (2 FMA per clock and SM).  Each thread takes every 128th node and
-// advances its cosine by a rotation, 4 multiply-adds per node instead of a cospi (the
-// rotation's error after the longest run, 65536/128 steps, stays near 1e-13 of Ghat(0),
-// far below the FP32 result).  A block per nu with the kernel evaluated and three cospi
-// taken in every panel took 1106 us for an 8193-sample table at n = 512, on every
-// wst_plan_set_kernel_table, that is on every training step;
-// that step as a whole went from 1492 to 422 us.
+// advances its cosine by the Chebyshev recurrence, one multiply-add per node beside the sum's
+// (its error grows with the square of the steps: 512 of them, for the longest table, leave
+// 3e-11 of Ghat(0), far below the FP32 result).  By rotations, 4 multiply-adds per node, the
+// 8193-sample table at n = 512 took 29 us, now 15; with a block per nu, the kernel evaluated
+// and three cospi taken in every panel, 1106 us, on every wst_plan_set_kernel_table, that is
+// on every training step.
 constexpr int kNodePanels = 256;   // panels per cell, analytic kernels
 constexpr int kCorrThreads = 128;
 
@@ -124,14 +124,14 @@ __global__ void __launch_bounds__(kCorrThreads) k_correction(float *corr, int n,
     return;
   }
   const double turn = (double)k * (double)W / ((double)n * (double)P);  // 2 nu h/2: half turns per node
-  double acc = 0.0, s, c, ds, dc;
-  sincospi(turn * (double)threadIdx.x, &s, &c);
-  sincospi(turn * (double)kCorrThreads, &ds, &dc);
+  // c_{m+1} = 2 cos(d) c_m - c_{m-1} from node to node of this thread
+  double acc = 0.0, c = cospi(turn * (double)threadIdx.x), before = cospi(turn * ((double)threadIdx.x - kCorrThreads));
+  const double twice = 2.0 * cospi(turn * (double)kCorrThreads);
   for (int j = threadIdx.x; j <= P; j += kCorrThreads) {
     acc = fma(__ldg(nodes + j), c, acc);
-    const double cn = fma(c, dc, -s * ds);
-    s = fma(s, dc, c * ds);
-    c = cn;
+    const double next = fma(twice, c, -before);
+    before = c;
+    c = next;
   }
   __shared__ double red[kCorrThreads];
   red[threadIdx.x] = acc;
