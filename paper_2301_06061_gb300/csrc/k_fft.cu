@@ -373,7 +373,7 @@ k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict_
       if (TW_FIRST) x = cmul(x, tws[i]);
       v[r] = x;
     }
-    dft<16, DIR>(v);
+    dft<16, DIR, (LB < 128)>(v);
     __syncthreads();  // every stage-0 read of the slot done before the exchange in place
 #pragma unroll
     for (int r = 0; r < 16; ++r) buf[(16 * jt + r) * CB + col] = v[r];
@@ -382,7 +382,7 @@ k_cols_a16(float2 *__restrict__ planes, Tw tw, int n, const uint8_t *__restrict_
     for (int b = 0; b < 16 / R1; ++b)
 #pragma unroll
       for (int r = 0; r < R1; ++r) v[b * R1 + r] = buf[(jt + b * TPL + 16 * r) * CB + col];
-    stage_compute_pre<LB, EPT, 1, DIR>(v, twr);
+    stage_compute_pre<LB, EPT, 1, DIR, (LB < 128)>(v, twr);
     float2 *dst = planes + (size_t)z * n * n + (size_t)a * n + band * CB + col;
 #pragma unroll
     for (int b = 0; b < 16 / R1; ++b)
@@ -480,8 +480,8 @@ __device__ __forceinline__ void screen_from_t(float2 t2, float2 w, float2 dw, fl
   if (STEP) stp = make_float2(0.0f, 0.0f);
   if (isnan(t2.x)) return;
   const ff t = {t2.x, t2.y};
-  scr = cis_cycles_ff(ff_mul({w.x, w.y}, t));
-  if (STEP) stp = cis_cycles_ff(ff_mul({dw.x, dw.y}, t));
+  scr = cis_cycles_poly(ff_mul({w.x, w.y}, t));
+  if (STEP) stp = cis_cycles_poly(ff_mul({dw.x, dw.y}, t));
   scr.x *= scale;
   scr.y *= scale;
 }
@@ -921,7 +921,7 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
         } else {
           bool valid;
           const ff t = n_minus_one_ff(s_l2p[col], s_l2q[out_line(e)], valid);
-          st = valid ? cis_cycles_ff(ff_mul({dwI.x, dwI.y}, t)) : make_float2(0.0f, 0.0f);
+          st = valid ? cis_cycles_poly(ff_mul({dwI.x, dwI.y}, t)) : make_float2(0.0f, 0.0f);
         }
         s_cstep[e][threadIdx.x] = make_float2(st.x, -st.y);
       }
@@ -983,7 +983,7 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
           } else {
             bool valid;
             const ff t = n_minus_one_ff(s_l2p[col], s_l2q[out_line(e)], valid);
-            a = valid ? cis_cycles_ff(ff_mul({wP.x, wP.y}, t)) : make_float2(0.0f, 0.0f);
+            a = valid ? cis_cycles_poly(ff_mul({wP.x, wP.y}, t)) : make_float2(0.0f, 0.0f);
             a.x *= sg;
             a.y *= sg;
           }

@@ -245,6 +245,10 @@ __device__ __forceinline__ float2 cis_small_cycles(float s, uint32_t parity) {
   const float cs = __fmaf_rn(z, pc, 1.0f);
   return make_float2(__uint_as_float(__float_as_uint(cs) ^ sign), __uint_as_float(__float_as_uint(sn) ^ sign));
 }
+// cis_cycles_ff by the polynomials
+__device__ __forceinline__ float2 cis_cycles_poly(ff phi) {
+  return cis_small_cycles(__fadd_rn(__fsub_rn(phi.hi, rintf(phi.hi)), phi.lo), 0u);
+}
 __device__ __forceinline__ float2 cis_cycles_d(double phi) {
   double r = phi - rint(phi);
   float s, c;
