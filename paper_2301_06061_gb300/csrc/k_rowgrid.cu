@@ -838,9 +838,7 @@ static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) 
   int grid = 0, batch = 0;
   cudaError_t e = persistent_grid<C>(p, kern, smem, (int64_t)np * N, grid, batch);
   if (e != cudaSuccess) return e;
-  unsigned long long *counter = p->W_.counters + CNT_WORK;
-  e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), p->stream);
-  if (e != cudaSuccess) return e;
+  unsigned long long *counter = p->W_.counters + CNT_WORK;  // cleared by the caller
   kern<<<grid, C::THREADS, smem, p->stream>>>(p->W_.records, p->W_.offsets, p0, np, kernel_params(p), out,
                                              p->W_.occ, counter, tw_half(p), p->W_.rowbound, p->W_.binmag,
                                              FFT ? p->W_.counters + CNT_ROWS : nullptr, batch);
@@ -859,9 +857,7 @@ static cudaError_t launch_rows_adjoint(wst_plan_s *p, int p0, int np, const floa
   int grid = 0, batch = 0;
   cudaError_t e = persistent_grid<C>(p, kern, smem, (int64_t)np * N, grid, batch);
   if (e != cudaSuccess) return e;
-  unsigned long long *counter = p->W_.counters + CNT_WORK;
-  e = cudaMemsetAsync(counter, 0, sizeof(unsigned long long), p->stream);
-  if (e != cudaSuccess) return e;
+  unsigned long long *counter = p->W_.counters + CNT_WORK;  // cleared by row_occupancy
   kern<<<grid, C::THREADS, smem, p->stream>>>(planes, p->W_.records, p->W_.offsets, p0, np, kernel_params(p),
                                              dvis ? dvis : p->W_.vacc, dtab, counter, tw_half(p), batch, dvis != nullptr);
   return cudaGetLastError();
@@ -911,10 +907,12 @@ cudaError_t rows_adjoint(wst_plan_s *p, int p0, int p1, const float2 *planes, fl
   }
 }
 
-// occ of a chunk's rows, as k_grid_rows leaves it, for the adjoint column pass
+// occ of a chunk's rows, as k_grid_rows leaves it, for the adjoint column pass; the work
+// counter of the row pass after it is cleared on the way
 __global__ void k_row_occ(const uint32_t *__restrict__ off, int64_t b0, int64_t rows, int n, int W,
-                          uint8_t *__restrict__ occ) {
+                          uint8_t *__restrict__ occ, unsigned long long *__restrict__ work) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *work = 0ull;
   if (i >= rows) return;
   const int64_t b = b0 + i;
   occ[i] = off[(b - min((int)(i % n), W - 1)) * kColBlocks] != off[(b + 1) * kColBlocks];
@@ -924,7 +922,7 @@ cudaError_t row_occupancy(wst_plan_s *p, int p0, int p1) {
   const int64_t rows = (int64_t)(p1 - p0) * p->n;
   if (rows <= 0) return cudaSuccess;
   k_row_occ<<<(unsigned)((rows + 255) / 256), 256, 0, p->stream>>>(p->W_.offsets, (int64_t)p0 * p->n, rows, p->n, p->W,
-                                                                   p->W_.occ);
+                                                                   p->W_.occ, p->W_.counters + CNT_WORK);
   p->launches += 1;
   return cudaGetLastError();
 }

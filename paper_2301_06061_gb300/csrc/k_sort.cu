@@ -49,9 +49,15 @@ __device__ __forceinline__ int image_of(const int64_t *__restrict__ boff, int ba
 }
 
 // batch offsets (64 per launch, passed as kernel arguments: no host synchronisation), and
-// with the first of them the counters and every image's w-range words
-__global__ void k_sort_init(int64_t *boff, SortOffsets a, int count, unsigned long long *counters, uint32_t *wminmax,
-                            int batch) {
+// with the first of them the counters, every image's w-range words and, up to kInitClear
+// bytes, the cleared bucket counts and bins (beyond that a memset's bandwidth counts for more
+// than its launch)
+constexpr size_t kInitClear = 4 << 20;
+__global__ void __launch_bounds__(256) k_sort_init(int64_t *boff, SortOffsets a, int count, unsigned long long *counters,
+                                                   uint32_t *wminmax, int batch, uint4 *clear, uint32_t n_clear) {
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_clear; i += gridDim.x * blockDim.x)
+    clear[i] = make_uint4(0u, 0u, 0u, 0u);
+  if (blockIdx.x > 0) return;
   const int i = threadIdx.x;
   if (i < count) boff[i] = a.v[i];
   if (!counters) return;
@@ -359,7 +365,8 @@ __global__ void k_scan_reduce(const uint32_t *data, int64_t n, uint32_t *block_s
   }
 }
 
-__global__ void k_scan_apply(uint32_t *data, int64_t n, const uint32_t *block_offsets) {
+// (copy: a second destination, or null)
+__global__ void k_scan_apply(uint32_t *data, int64_t n, const uint32_t *block_offsets, uint32_t *copy) {
   const int64_t base = (int64_t)blockIdx.x * kScanBlock + threadIdx.x * kScanItems;
   uint32_t v[kScanItems];
   uint32_t s = 0;
@@ -372,7 +379,10 @@ __global__ void k_scan_apply(uint32_t *data, int64_t n, const uint32_t *block_of
   uint32_t run = block_exclusive_scan(s, &total) + (block_offsets ? block_offsets[blockIdx.x] : 0u);
 #pragma unroll
   for (int i = 0; i < kScanItems; ++i) {
-    if (base + i < n) data[base + i] = run;
+    if (base + i < n) {
+      data[base + i] = run;
+      if (copy) copy[base + i] = run;
+    }
     run += v[i];
   }
 }
@@ -389,17 +399,17 @@ int64_t scan_tmp_words(int64_t n) {
 }
 
 static cudaError_t scan_exclusive(uint32_t *data, int64_t n, uint32_t *tmp, cudaStream_t s,
-                                  int64_t &launches) {
+                                  int64_t &launches, uint32_t *copy) {
   const int64_t nb = scan_blocks(n);
   if (nb <= 1) {
-    k_scan_apply<<<1, kScanThreads, 0, s>>>(data, n, nullptr);
+    k_scan_apply<<<1, kScanThreads, 0, s>>>(data, n, nullptr, copy);
     launches += 1;
     return cudaGetLastError();
   }
   k_scan_reduce<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, tmp);
-  cudaError_t e = scan_exclusive(tmp, nb, tmp + nb + 64, s, launches);
+  cudaError_t e = scan_exclusive(tmp, nb, tmp + nb + 64, s, launches, nullptr);
   if (e != cudaSuccess) return e;
-  k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, tmp);
+  k_scan_apply<<<(unsigned)nb, kScanThreads, 0, s>>>(data, n, tmp, copy);
   launches += 2;
   return cudaGetLastError();
 }
@@ -568,18 +578,22 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
   Workspace &ws = p->W_;
   const int64_t nb1 = p->n_buckets + 1;
   cudaError_t e;
+  // offsets and, after them in the workspace, the magnitude bins; both start on 256-byte
+  // boundaries with padding up to the next array, so the clear may round up to 16 bytes
+  const int nb = bins_per_row(p->n);
+  const int64_t n_bins = p->n_buckets / kColBlocks * nb;
+  const size_t clear = (size_t)((char *)(ws.binmag + n_bins) - (char *)ws.offsets);
+  const uint32_t n_clear = clear <= kInitClear ? (uint32_t)((clear + 15) / 16) : 0u;
   for (int i0 = 0; i0 <= p->batch; i0 += kSortOffsets) {
     SortOffsets a;
     const int cnt = (p->batch + 1 - i0) < kSortOffsets ? (p->batch + 1 - i0) : kSortOffsets;
     for (int i = 0; i < cnt; ++i) a.v[i] = batch_offsets[i0 + i];
-    k_sort_init<<<1, 256, 0, s>>>(p->batch_off + i0, a, cnt, i0 == 0 ? ws.counters : nullptr, ws.wminmax, p->batch);
+    const unsigned blocks = i0 == 0 && n_clear ? (n_clear + 1023) / 1024 : 1u;
+    k_sort_init<<<blocks, 256, 0, s>>>(p->batch_off + i0, a, cnt, i0 == 0 ? ws.counters : nullptr, ws.wminmax, p->batch,
+                                       reinterpret_cast<uint4 *>(ws.offsets), i0 == 0 ? n_clear : 0u);
     p->launches += 1;
   }
-  // offsets and, after them in the workspace, the magnitude bins
-  const int nb = bins_per_row(p->n);
-  const int64_t n_bins = p->n_buckets / kColBlocks * nb;
-  const size_t clear = (size_t)((char *)(ws.binmag + n_bins) - (char *)ws.offsets);
-  if ((e = cudaMemsetAsync(ws.offsets, 0, clear, s))) return e;
+  if (!n_clear && (e = cudaMemsetAsync(ws.offsets, 0, clear, s))) return e;
   const bool fold = (p->cfg.flags & WST_FLAG_WFOLD) != 0;
   int sms = 0;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device))) return e;
@@ -589,8 +603,11 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
     if (coords.rows) k_wrange<true><<<grd, kWrangeThreads, 0, s>>>(coords, p->batch_off, p->batch, p->n_vis, ws.wminmax, fold);
     else k_wrange<false><<<grd, kWrangeThreads, 0, s>>>(coords, p->batch_off, p->batch, p->n_vis, ws.wminmax, fold);
     p->launches += 1;
+    if ((e = build_plane_centres(p))) return e;
+  } else if (s != p->centres_stream) {  // a configured range: built with the plan, and for each
+    if ((e = build_plane_centres(p))) return e;  // stream it moves to, in that stream's order
+    p->centres_stream = s;
   }
-  if ((e = build_plane_centres(p))) return e;
   SortGeom g;
   g.n = p->n;
   g.W = p->W;
@@ -611,8 +628,7 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
                                       ws.offsets, ws.keyinfo, ws.counters, stash, fold);
   p->launches += 1;
   if ((e = cudaGetLastError())) return e;
-  if ((e = scan_exclusive(ws.offsets, nb1, ws.scan_tmp, s, p->launches))) return e;
-  if ((e = cudaMemcpyAsync(ws.cursor, ws.offsets, sizeof(uint32_t) * nb1, cudaMemcpyDeviceToDevice, s))) return e;
+  if ((e = scan_exclusive(ws.offsets, nb1, ws.scan_tmp, s, p->launches, ws.cursor))) return e;
   k_scatter<<<grid_for(p->n_vis, 256, 152 * 16), 256, 0, s>>>(vis, weight, ws.keyinfo, ws.cursor, p->n_vis,
                                                               ws.records, ws.binmag, nb, p->W, stash);
   p->launches += 1;

@@ -232,6 +232,8 @@ wst_status wst_plan_create(const wst_config *cfg, void *cuda_stream, wst_plan *o
   }
   e = build_tables(p);
   if (e == cudaSuccess && c.kernel != WST_KERNEL_TABLE) e = build_correction(p);
+  if (e == cudaSuccess && c.w_min != c.w_max) e = build_plane_centres(p);  // else from each data set
+  p->centres_stream = p->stream;
   if (e != cudaSuccess) {
     destroy_tables(p);
     delete p;
@@ -414,6 +416,7 @@ wst_status wst_grid(wst_plan p, int32_t b, int32_t e, void *out) {
   wst_status st = check_ready(p);
   if (st) return st;
   if (b < 0 || e > p->n_planes || b > e || (!out && e > b)) return fail(p, WST_ERR_INVALID_ARG, "plane range or output");
+  WST_CUDA(p, cudaMemsetAsync(p->W_.counters + CNT_WORK, 0, sizeof(unsigned long long), p->stream), "memset");
   WST_CUDA(p, grid_rows(p, b, e, (float2 *)out, false), "grid");
   return WST_OK;
 }
@@ -462,9 +465,12 @@ static wst_status image_range(wst_plan_s *p, int b, int e, void *image_out, uint
   float2 *planes = p->W_.planes;
   p->n_chunks = 0;
   p->launches = 0;
-  WST_CUDA(p, cudaMemsetAsync(p->W_.counters + CNT_ROWS, 0, sizeof(unsigned long long), p->stream), "memset");
+  static_assert(CNT_ROWS == CNT_WORK + 1, "cleared together");
+  if (b == e) WST_CUDA(p, cudaMemsetAsync(p->W_.counters + CNT_ROWS, 0, sizeof(unsigned long long), p->stream), "memset");
   for (int p0 = b; p0 < e; p0 += p->chunk) {
     const int p1 = (p0 + p->chunk < e) ? p0 + p->chunk : e;
+    WST_CUDA(p, cudaMemsetAsync(p->W_.counters + CNT_WORK, 0, (p0 == b ? 2 : 1) * sizeof(unsigned long long), p->stream),
+             "memset");
     WST_CUDA(p, time_begin(p, p->ev_img, ST_GRID), "event");
     WST_CUDA(p, grid_rows(p, p0, p1, planes, true), "grid + rows");
     WST_CUDA(p, time_end(p, p->ev_img), "event");

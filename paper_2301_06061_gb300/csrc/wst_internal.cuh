@@ -126,6 +126,7 @@ struct wst_plan_s {
   double *wcentre_d = nullptr;  // per global plane: centre w_k (FP64)
   float2 *dwff = nullptr;    // per image: plane spacing dw as float-float
   bool table_set = false;
+  cudaStream_t centres_stream = nullptr;  // where the centres of a configured w range were built last
   // limit of the device-side waits for data (the row kernel's bulk copies), nanoseconds;
   // 0 = expire at once (failure-path testing, wst_plan_set_wait_limit)
   unsigned long long wait_ns = 2000000000ull;
@@ -341,12 +342,12 @@ cudaError_t vis_cells(wst_plan_s *p, int32_t *plane, int32_t *i0, int32_t *j0, i
 int64_t scan_tmp_words(int64_t n);
 
 // k_rowgrid.cu
-cudaError_t grid_rows(wst_plan_s *p, int p0, int p1, float2 *out, bool fft);
+cudaError_t grid_rows(wst_plan_s *p, int p0, int p1, float2 *out, bool fft);  // CNT_WORK zero before
 // adjoint rows.  dtab: the table gradient is added to it; else degridding, the sums added to
 // dvis in the caller's order or (dvis null) to W_.vacc in sorted order (unsort_sums hands
 // them over once every plane has been through)
 cudaError_t rows_adjoint(wst_plan_s *p, int p0, int p1, const float2 *planes, float2 *dvis, float *dtab);
-cudaError_t row_occupancy(wst_plan_s *p, int p0, int p1);  // W_.occ of planes [p0, p1)
+cudaError_t row_occupancy(wst_plan_s *p, int p0, int p1);  // W_.occ of planes [p0, p1); clears CNT_WORK
 cudaError_t unsort_sums(wst_plan_s *p, float2 *dvis);
 
 // k_fft.cu
