@@ -75,6 +75,10 @@ using GridCfg = GroupCfg<N, N == 4096 ? 1024 : 128>;
 template <int N>
 constexpr bool kPending = N >= 8192;
 
+// rows whose kernel copies the tap-major table to shared memory (smem_taps: if it fits)
+template <int N>
+constexpr bool kTapsShared = N == 8192;
+
 // barrier of one group: the CTA, a warp, or a named barrier of the group's warps
 template <int GT, int GROUPS>
 struct GroupSync {
@@ -124,8 +128,10 @@ __device__ __forceinline__ void zero_row(float2 *srow, int jt) {
 // q = exp(-2c), c = 1/(2 sigma^2); each exponential is a power of two, exp(-y c) =
 // 2^(-y c log2 e), with c log2 e rounded once from FP64 (the FP32 argument carries the
 // same rounding as with exp).
-template <int WT>
-__device__ __forceinline__ void x_taps(const KernelParams &kp, float gx, float q, float (&g)[WT]) {
+// taps: the tap-major table, in shared memory if SMT (else in device memory), or null.
+template <int WT, bool SMT>
+__device__ __forceinline__ void x_taps(const KernelParams &kp, const float *taps, float gx, float q, float (&g)[WT]) {
+  static_assert(WT <= kTapRow, "taps of a row");
   if (kp.kind == WST_KERNEL_GAUSS) {
     const float t = gx - kp.half;
     float ga = exp2f(-t * t * kp.l2c);
@@ -136,28 +142,24 @@ __device__ __forceinline__ void x_taps(const KernelParams &kp, float gx, float q
       ga *= ra;
       ra *= q;
     }
-  } else if (kp.tap_table) {
-    // tabulated kernel: all W taps share the sub-cell position, so their bracketing
-    // samples are one contiguous run of W pairs (tap-major table)
+  } else if (taps) {
+    // tabulated kernel: all W taps share the sub-cell position, so the samples that bracket
+    // them are two neighbouring rows of the tap-major table, four 16-byte loads.  The loads
+    // bound the gridder with a table (a warp's go to 32 different lines each): rows of 8192,
+    // one CTA per SM, have the memory to keep the table in shared memory
     const float pos = gx * (float)kp.per_cell;
     const int i = min((int)pos, kp.per_cell - 1);
     const float f = pos - (float)i;
-    const float2 *run = kp.tap_table + (size_t)i * WT;
-    if constexpr (WT % 2 == 0) {  // 16-byte aligned: two taps per load
-      const float4 *run4 = reinterpret_cast<const float4 *>(run);
+    const float4 *row = reinterpret_cast<const float4 *>(taps + (size_t)i * kTapRow);
+    float lo[kTapRow], hi[kTapRow];
 #pragma unroll
-      for (int a = 0; a < WT / 2; ++a) {
-        const float4 t = __ldg(run4 + a);
-        g[2 * a] = fmaf(f, t.y - t.x, t.x);
-        g[2 * a + 1] = fmaf(f, t.w - t.z, t.z);
-      }
-    } else {
-#pragma unroll
-      for (int a = 0; a < WT; ++a) {
-        const float2 t = __ldg(run + a);
-        g[a] = fmaf(f, t.y - t.x, t.x);
-      }
+    for (int k = 0; k < kTapRow / 4; ++k) {
+      const float4 x = SMT ? row[k] : __ldg(row + k), y = SMT ? row[kTapRow / 4 + k] : __ldg(row + kTapRow / 4 + k);
+      lo[4 * k] = x.x, lo[4 * k + 1] = x.y, lo[4 * k + 2] = x.z, lo[4 * k + 3] = x.w;
+      hi[4 * k] = y.x, hi[4 * k + 1] = y.y, hi[4 * k + 2] = y.z, hi[4 * k + 3] = y.w;
     }
+#pragma unroll
+    for (int a = 0; a < WT; ++a) g[a] = fmaf(f, hi[a] - lo[a], lo[a]);
   } else {
 #pragma unroll
     for (int a = 0; a < WT; ++a) g[a] = kernel_tap(kp, (float)a - kp.half + gx);
@@ -166,11 +168,11 @@ __device__ __forceinline__ void x_taps(const KernelParams &kp, float gx, float q
 
 // f(a, G(a - W/2 + g_x)) for every tap a: the unrolled x_taps where the support has an
 // instance of its own (and not EVAL), else each tap evaluated
-template <int WT, bool EVAL, class F>
-__device__ __forceinline__ void for_taps(const KernelParams &kp, float gx, float q, const F &f) {
+template <int WT, bool EVAL, bool SMT, class F>
+__device__ __forceinline__ void for_taps(const KernelParams &kp, const float *taps, float gx, float q, const F &f) {
   if constexpr (WT > 0 && !EVAL) {
     float g[WT];
-    x_taps<WT>(kp, gx, q, g);
+    x_taps<WT, SMT>(kp, taps, gx, q, g);
 #pragma unroll
     for (int a = 0; a < WT; ++a) f(a, g[a]);
   } else {
@@ -293,7 +295,7 @@ struct NoPending {
 template <int N, int WT, bool FIXED, class PEND>
 __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__restrict__ rec,
                                         const uint32_t *bnd, int d_lo, const KernelParams &kp, int jt,
-                                        float qscale, float gmax, RecHead *stg, int stg_stride, PEND &pd) {
+                                        float qscale, float gmax, RecHead *stg, int stg_stride, const float *taps, PEND &pd) {
   constexpr int TPR = RowCfg<N>::TPR;
   int ovf = 0;
   const uint32_t s_end = bnd[d_lo + 1];
@@ -324,7 +326,9 @@ __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__
     const float gq = FIXED ? gy * qscale : gy;
     const float vre = r.vre * gq, vim = r.vim * gq;
     if (FIXED && fmaxf(fabsf(vre), fabsf(vim)) * gmax >= 0x1.ffp30f) ovf = -1;
-    for_taps<WT, false>(kp, rec_gx(r), q, [&](int a, float g) { add_tap<FIXED>(sre, sim, i0 + a, vre * g, vim * g, ovf); });
+    for_taps<WT, false, kTapsShared<N>>(kp, taps, rec_gx(r), q, [&](int a, float g) {
+      add_tap<FIXED>(sre, sim, i0 + a, vre * g, vim * g, ovf);
+    });
     pd.write_one(jt);
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -340,7 +344,7 @@ template <int N, bool FFT, int WT, class PEND, class SYNC>
 __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, int d_lo, float2 mb,
                                              const Record *__restrict__ rec, int q, bool nonempty,
                                              const KernelParams &kp, float2 *__restrict__ orow, const float2 *twt,
-                                             int jt, float gmax, RecHead *stg, int stg_stride, PEND &pd,
+                                             int jt, float gmax, RecHead *stg, int stg_stride, const float *taps, PEND &pd,
                                              const SYNC &sync) {
   using C = RowCfg<N>;
   constexpr int EPT = C::EPT, TPR = C::TPR;
@@ -374,8 +378,8 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   int ovf = 0;
   if (nonempty) {
     if (fixed)
-      ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, pd);
-    else grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, pd);
+      ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps, pd);
+    else grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
   }
   // a tap or a partial sum left the int32 range: once more with delta = B / 2^30, which holds
   // any row.  (Such a row has a cell of 1/64 of its busiest bin's magnitude or more, whose
@@ -387,9 +391,9 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
     sync();
     if (nonempty && fixed) {
       unit = 0x1p-30f;
-      grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, pd);
+      grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps, pd);
     } else if (nonempty) {
-      grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, pd);
+      grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
     }
     sync();
   }
@@ -454,7 +458,7 @@ __global__ void __launch_bounds__(GridCfg<N>::THREADS,
 k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, int p0, int np,
             KernelParams kp, float2 *__restrict__ out, uint8_t *__restrict__ occ,
             unsigned long long *__restrict__ counter, Tw tw, const float2 *__restrict__ rowbound,
-            const float *__restrict__ binmag, unsigned long long *__restrict__ rows_done, int batch) {
+            const float *__restrict__ binmag, unsigned long long *__restrict__ rows_done, int batch, bool smem_taps) {
   using C = GridCfg<N>;
   constexpr int TPR = C::TPR, GT = C::GT, GR = C::GR, GROUPS = C::GROUPS;
   extern __shared__ __align__(16) float2 sm_rows[];
@@ -470,6 +474,15 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
   // G^2 of the fixed-point bound (G = 1 for the Gaussian and the ES kernel, the largest
   // |sample| of a table: linear interpolation stays below it)
   const float gmax = kp.kind == WST_KERNEL_TABLE ? __ldg(kp.table_max) : 1.0f;
+  const float *taps = kp.tap_table;
+  if constexpr (kTapsShared<N> && WT > 0) {
+    if (smem_taps) {
+      float4 *t = reinterpret_cast<float4 *>(stg - threadIdx.x + 3 * C::THREADS);
+      for (int i = threadIdx.x; i < (kp.per_cell + 1) * (kTapRow / 4); i += C::THREADS)
+        t[i] = __ldg(reinterpret_cast<const float4 *>(kp.tap_table) + i);
+      taps = reinterpret_cast<const float *>(t);
+    }
+  }
   __syncthreads();
   const long long total = (long long)np * N;
   const int W = WT > 0 ? WT : kp.support;
@@ -541,7 +554,7 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
         const int pl = (int)(item / N), q = (int)(item % N);
         const int d_lo = min(q, W - 1);
         grid_one_row<N, FFT, WT>(srow, &s_off[g][buf][r + W - 1 - d_lo], d_lo, s_rb[g][buf][r], rec, q, e & 1, kp,
-                                 out + ((int64_t)pl * N + q) * N, twt, jt, gmax, stg, stg_stride, pd, sync);
+                                 out + ((int64_t)pl * N + q) * N, twt, jt, gmax, stg, stg_stride, taps, pd, sync);
       }
       if (cnt == 0) sync();  // s_item, s_cnt and the list are read before they are written again
     }
@@ -576,7 +589,7 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
         float2 *orow = valid && (!FFT || !empty) ? out + ((int64_t)pl * N + q) * N : nullptr;
         NoPending none;
         grid_one_row<N, FFT, WT>(srow, s_bnd[rl], d_lo, mb, rec, q, !empty, kp, orow, twt, jt, gmax, stg, stg_stride,
-                                 none, sync);
+                                 taps, none, sync);
       }
       __syncwarp();
     }
@@ -695,7 +708,7 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
         float are = 0.0f, aim = 0.0f;
         // the taps one by one, as the table gradient takes them: the image's corners enter with
         // the grid correction's 1e3 to 1e5 and cancel here, which magnifies any other rounding
-        for_taps<WT, true>(kp, gx0, 0.0f, [&](int a, float gx) {
+        for_taps<WT, true, false>(kp, nullptr, gx0, 0.0f, [&](int a, float gx) {
           const float2 c = cell[a];
           are = fmaf(gx, c.x, are);
           aim = fmaf(gx, c.y, aim);
@@ -833,15 +846,24 @@ static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) 
     if (p->cfg.support == 7) kern = k_grid_rows<N, FFT, 7>;
     else if (p->cfg.support == 8) kern = k_grid_rows<N, FFT, 8>;
   }
-  const size_t smem = sizeof(float2) * (C::ROWS * C::PADL + (FFT ? line_table_size<N, C::EPT, C::TPR>() : 0)) +
-                      3 * C::THREADS * sizeof(RecHead);
+  size_t smem = sizeof(float2) * (C::ROWS * C::PADL + (FFT ? line_table_size<N, C::EPT, C::TPR>() : 0)) +
+                3 * C::THREADS * sizeof(RecHead);
+  bool smem_taps = false;
+  if (FFT && kTapsShared<N> && p->ktap) {
+    int most = 0;
+    const cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
+    if (e != cudaSuccess) return e;
+    const size_t tab = sizeof(float) * kTapRow * (kernel_params(p).per_cell + 1);
+    smem_taps = smem + tab + 1024 <= (size_t)most;  // 1 KB: the kernel's static shared memory
+    if (smem_taps) smem += tab;
+  }
   int grid = 0, batch = 0;
   cudaError_t e = persistent_grid<C>(p, kern, smem, (int64_t)np * N, grid, batch);
   if (e != cudaSuccess) return e;
   unsigned long long *counter = p->W_.counters + CNT_WORK;  // cleared by the caller
   kern<<<grid, C::THREADS, smem, p->stream>>>(p->W_.records, p->W_.offsets, p0, np, kernel_params(p), out,
                                              p->W_.occ, counter, tw_half(p), p->W_.rowbound, p->W_.binmag,
-                                             FFT ? p->W_.counters + CNT_ROWS : nullptr, batch);
+                                             FFT ? p->W_.counters + CNT_ROWS : nullptr, batch, smem_taps);
   return cudaGetLastError();
 }
 

@@ -25,20 +25,20 @@ KernelParams kernel_params(const wst_plan_s *p) {
   return k;
 }
 
-// Tap-major copy of a kernel table with L - 1 = W pc samples: entry [i][a] holds the two
-// samples that bracket tap a at sub-cell position i / pc, so the W taps of one
-// visibility (all at the same sub-cell offset) are one contiguous run of W pairs.
-__global__ void k_tap_table(const float *t, float2 *tap, int W, int pc) {
+// Tap-major copy of a kernel table with L - 1 = W pc samples: row i, 0 <= i <= pc, holds
+// every tap's sample at sub-cell position i / pc, so the samples that bracket the W taps of
+// one visibility (all at the same sub-cell offset) are two neighbouring rows.
+__global__ void k_tap_table(const float *t, float *tap, int W, int pc) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= W * pc) return;
-  const int i = idx / W, a = idx % W;
-  tap[idx] = make_float2(t[a * pc + i], t[a * pc + i + 1]);
+  if (idx >= kTapRow * (pc + 1)) return;
+  const int i = idx / kTapRow, a = idx % kTapRow;
+  tap[idx] = a < W ? t[a * pc + i] : 0.0f;
 }
 
 cudaError_t build_tap_table(wst_plan_s *p) {
   if (!p->ktap) return cudaSuccess;
   const int pc = (p->cfg.ktable_len - 1) / p->W;
-  k_tap_table<<<(p->W * pc + 255) / 256, 256, 0, p->stream>>>(p->ktable, p->ktap, p->W, pc);
+  k_tap_table<<<(kTapRow * (pc + 1) + 255) / 256, 256, 0, p->stream>>>(p->ktable, p->ktap, p->W, pc);
   p->launches += 1;
   return cudaGetLastError();
 }

@@ -223,7 +223,9 @@ wst_status wst_plan_create(const wst_config *cfg, void *cuda_stream, wst_plan *o
   ALLOC(p->batch_off, c.batch + 1);
   if (c.kernel == WST_KERNEL_TABLE) ALLOC(p->ktable, c.ktable_len);
   if (c.kernel == WST_KERNEL_TABLE) ALLOC(p->kmax, 1);
-  if (c.kernel == WST_KERNEL_TABLE && (c.ktable_len - 1) % c.support == 0) ALLOC(p->ktap, c.ktable_len - 1);
+  // the imaging kernel's unrolled supports take the tap-major table
+  if (c.kernel == WST_KERNEL_TABLE && (c.support == 7 || c.support == 8) && (c.ktable_len - 1) % c.support == 0)
+    ALLOC(p->ktap, kTapRow * ((c.ktable_len - 1) / c.support + 1));
 #undef ALLOC
   if (e != cudaSuccess) {
     destroy_tables(p);

@@ -64,6 +64,8 @@ __device__ __forceinline__ float rec_gy(const RecHead &r) {
   return (float)(r.ypack & 0xFFFFFFu) * (1.0f / 16777216.0f);
 }
 
+constexpr int kTapRow = 8;  // taps of a row of the tap-major table (16-byte loads)
+
 struct KernelParams {
   int kind;        // WST_KERNEL_*
   int support;     // W
@@ -75,7 +77,7 @@ struct KernelParams {
   const float *table;  // TABLE: device samples
   int table_len;
   float table_scale;   // (L-1)/W
-  const float2 *tap_table;  // TABLE with L - 1 = W * per_cell: [per_cell][W] pairs (T[a pc + i], T[a pc + i + 1])
+  const float *tap_table;   // TABLE, W = 7 or 8, L - 1 = W per_cell: rows i of T[a pc + i], a < kTapRow, i <= pc
   int per_cell;
   const float *table_max;   // TABLE: the largest |sample|
 };
@@ -119,7 +121,7 @@ struct wst_plan_s {
   double *l2d = nullptr;     // l_a^2 in FP64 (WST_FLAG_FP64_SCREEN)
   float *ktable = nullptr;   // TABLE kernel samples
   float *kmax = nullptr;     // TABLE: the largest |sample| (k_correction)
-  float2 *ktap = nullptr;    // TABLE samples in tap-major pairs (see KernelParams::tap_table)
+  float *ktap = nullptr;     // TABLE samples tap-major (see KernelParams::tap_table)
   double *wrange = nullptr;  // per image: w_lo, scale = n_w/(w_hi-w_lo), dw, w_hi
   float4 *wrange_ff = nullptr;  // per image: w_lo and scale as float-float pairs
   float2 *wcentre = nullptr; // per global plane: centre w_k as float-float
