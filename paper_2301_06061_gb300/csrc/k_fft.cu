@@ -832,10 +832,21 @@ k_cols_b16(const float2 *__restrict__ planes, int p0, int p1, int n_w, Tw tw,
 // rounding of a block therefore stays within one block (as the recurrence of k_cols_b16
 // stays within kAnchor - 1 steps), and the blocks are summed with compensation.
 // ---------------------------------------------------------------------------------
-constexpr int kColsBRing = 3;
+// BLOCKS: the most anchor blocks an image's planes of the call fall into, 1 or 2 (0: any).
+// The running sum and its compensation take 64 registers that only the end of a block
+// uses: one block's sum goes straight to the flush, two leave one array (the compensation of
+// the first sum is zero).  8 + 8 planes of 16384^2 12.87 -> 10.82 ms, 16 of 8192^2 2.00 -> 1.82,
+// 64 x 16 of 2048^2 7.03 -> 6.42 (one block); one block of 128-line tiles then fits four CTAs
+// per SM with a ring of two (11.75 ms with three and a ring of three), 64-line tiles were
+// faster with six and three (6.42 against 6.82 ms).
+template <int LA, int BLOCKS>
+struct ColsB {
+  static constexpr int RING = LA == 128 && BLOCKS == 1 ? 2 : 3;
+  static constexpr int CTAS = LA == 128 && BLOCKS == 1 ? 4 : 384 / LA;
+};
 
-template <int LA, bool FP64S, bool CROP>
-__global__ void __launch_bounds__(LA / 16 * kCB, LA == 128 ? 3 : 6)
+template <int LA, bool FP64S, bool CROP, int BLOCKS>
+__global__ void __launch_bounds__(LA / 16 * kCB, ColsB<LA, BLOCKS>::CTAS)
 k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, Tw tw, int n, ScreenCtx sc,
              float2 *__restrict__ image, float2 *__restrict__ comp, int flags, int n_img_arg, int crop_arg,
              unsigned long long *__restrict__ err, unsigned long long wait_ns, int first_lo, int last_hi, int ipz) {
@@ -847,13 +858,14 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
   if (p0 >= p1) return;
   constexpr int EPT = 16, TPL = LA / EPT, THREADS = TPL * kCB, R1 = LA / 16;
   static_assert(num_stages(LA, EPT) == 2 && stage_radix(LA, EPT, 1) == R1, "two stages");
+  constexpr int kRing = ColsB<LA, BLOCKS>::RING;
   constexpr uint32_t kTileBytes = LA * kCB * sizeof(float2);
   static_assert(EPT * THREADS <= LA * kCB, "anchor screens fit a slot");
-  __shared__ __align__(128) float2 ring[kColsBRing][LA * kCB];
+  __shared__ __align__(128) float2 ring[kRing][LA * kCB];
   __shared__ float2 s_cstep[EPT][THREADS];  // conj of each output's per-plane screen step
   constexpr int NTW = total_tw_count<LA, EPT>();
   __shared__ float2 s_tw1[NTW][TPL];
-  __shared__ __align__(8) unsigned long long s_mbar[kColsBRing];
+  __shared__ __align__(8) unsigned long long s_mbar[kRing];
   // l^2 (float-float) and the grid correction 1/Ghat of the tile's LA grid rows c + B m
   // and of its kCB columns, read once: every screen evaluation of the tile takes its
   // n - 1 arguments from here, and the flush its correction factors
@@ -877,7 +889,7 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
     for (int i = 0; i < NTW; ++i) s_tw1[i][threadIdx.x] = twr[i];
   }
   if (threadIdx.x == 0) {
-    for (int i = 0; i < kColsBRing; ++i) mbar_init(mbar0 + 8u * i, 1u);
+    for (int i = 0; i < kRing; ++i) mbar_init(mbar0 + 8u * i, 1u);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (!FP64S) {
@@ -892,11 +904,11 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
   const int nplanes = p1 - p0;
   int issued = 0;  // thread 0: planes (indices within the call) whose tile copy is issued
   auto issue = [&](int q) {
-    const int slot = q % kColsBRing;
+    const int slot = q % kRing;
     tma_load_tile3d(ring0 + (uint32_t)slot * kTileBytes, &tmap, 2 * col0, LA * c, z0 + q, mbar0 + 8u * slot, kTileBytes);
   };
   if (threadIdx.x == 0)
-    for (; issued < kColsBRing && issued < nplanes; ++issued) issue(issued);
+    for (; issued < kRing && issued < nplanes; ++issued) issue(issued);
   // output e = b R1 + r of this thread is line element jt + b TPL + 16 r, image row c + B (that)
   auto out_line = [&](int e) { return jt + (e / R1) * TPL + 16 * (e % R1); };
   auto out_row = [&](int e) { return c + B * out_line(e); };
@@ -926,13 +938,18 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
         s_cstep[e][threadIdx.x] = make_float2(st.x, -st.y);
       }
     }
-    float2 S[EPT], Cc[EPT], acc[EPT];
+    constexpr int NS = BLOCKS == 1 ? 1 : EPT, NC = BLOCKS == 0 ? EPT : 1;
+    float2 S[NS], Cc[NC], acc[EPT];
 #pragma unroll
-    for (int e = 0; e < EPT; ++e) S[e] = Cc[e] = acc[e] = make_float2(0.0f, 0.0f);
+    for (int e = 0; e < NS; ++e) S[e] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int e = 0; e < NC; ++e) Cc[e] = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int e = 0; e < EPT; ++e) acc[e] = make_float2(0.0f, 0.0f);
     for (; P < pend; ++P) {
       const int q = P - p0;
-      const int slot = q % kColsBRing;
-      const bool ok = mbar_wait_bounded(mbar0 + 8u * slot, (uint32_t)(q / kColsBRing) & 1u, wait_ns);
+      const int slot = q % kRing;
+      const bool ok = mbar_wait_bounded(mbar0 + 8u * slot, (uint32_t)(q / kRing) & 1u, wait_ns);
       float2 *tile = ring[slot];
       float2 v[EPT];
 #pragma unroll
@@ -967,7 +984,7 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
         acc[e] = make_float2(fmaf(acc[e].x, cs.x, fmaf(-acc[e].y, cs.y, v[e].x)),
                              fmaf(acc[e].x, cs.y, fmaf(acc[e].y, cs.x, v[e].y)));
       }
-      if ((P - pstart) % kAnchor == kAnchor - 1 || P == pend - 1) {
+      if ((BLOCKS != 1 && (P - pstart) % kAnchor == kAnchor - 1) || P == pend - 1) {
         // end of an anchor block: the exact screen of plane P (sign included) for each
         // output, through the slot of this plane once every thread is done with it
         __syncthreads();
@@ -992,9 +1009,18 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
 #pragma unroll
         for (int e = 0; e < EPT; ++e) {
           const float2 y = cmul(acc[e], s_anchor[e * THREADS + threadIdx.x]);
-          if (kahan) kahan_add(S[e], Cc[e], y);
-          else S[e] = cadd(S[e], y);
-          acc[e] = make_float2(0.0f, 0.0f);
+          if constexpr (BLOCKS == 1) {
+            acc[e] = y;
+          } else if constexpr (BLOCKS == 2) {  // acc: the compensation once the last block is in
+            float2 cmp = make_float2(0.0f, 0.0f);
+            if (kahan) kahan_add(S[e], cmp, y);
+            else S[e] = cadd(S[e], y);
+            acc[e] = P == pend - 1 ? cmp : make_float2(0.0f, 0.0f);
+          } else {
+            if (kahan) kahan_add(S[e], Cc[e], y);
+            else S[e] = cadd(S[e], y);
+            acc[e] = make_float2(0.0f, 0.0f);
+          }
         }
       }
     }
@@ -1009,7 +1035,9 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
       if (CROP && (kq < crop || kq >= crop + n_img || kp < crop || kp >= crop + n_img))
           continue;  // a grid row or column outside the image
       const float f = (flags & ACC_CORRECT) ? s_corp[col] * s_corq[out_line(e)] : 1.0f;
-      flush_pixel(im, cp, (size_t)(kq - crop) * n_img + (kp - crop), S[e], Cc[e], first_any, last_any, flags, f);
+      const float2 sum = BLOCKS == 1 ? acc[e] : S[BLOCKS == 1 ? 0 : e];
+      const float2 cmp = BLOCKS == 1 ? make_float2(0.0f, 0.0f) : BLOCKS == 2 ? acc[e] : Cc[BLOCKS == 0 ? e : 0];
+      flush_pixel(im, cp, (size_t)(kq - crop) * n_img + (kp - crop), sum, cmp, first_any, last_any, flags, f);
     }
   }
   if (failed) {
@@ -1017,7 +1045,7 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
       atomicExch(err, (unsigned long long)WST_ERR_TIMEOUT);
       // every copy issued must land before the CTA exits: bounded, with the full limit
       for (int q = P - p0; q < issued; ++q)
-        mbar_wait_bounded(mbar0 + 8u * (q % kColsBRing), (uint32_t)(q / kColsBRing) & 1u, kWaitLimitNs);
+        mbar_wait_bounded(mbar0 + 8u * (q % kRing), (uint32_t)(q / kRing) & 1u, kWaitLimitNs);
     }
     __syncthreads();
   }
@@ -1063,12 +1091,13 @@ __device__ __forceinline__ void bh_stages(float2 (&v)[ColCfg<LA>::EPT], int jt, 
 // the stage twiddles in a shared table (one row per line position), and the exchanges
 // alternate between two buffers, one barrier each.  With the steps and twiddle loads in
 // the way (141 registers: 8 warps per SM at LA = 128, four barriers per plane) 16 planes of
-// 8192^2 took 4.14 ms.  The arithmetic is that of the plain stages in the same order: the
+// 8192^2 took 4.14 ms, now 2.29 ms.  The arithmetic is that of the plain stages in the same order: the
 // grid correction multiplies the corners by up to 1e5 here and they cancel in the
 // degridded values, which would show any other rounding.
 template <int LA>
-struct BhCfg {
-  static constexpr int CTAS = 768 / ColCfg<LA>::THREADS > 24 ? 24 : 768 / ColCfg<LA>::THREADS;  // resident per SM
+struct BhCfg {  // resident CTAs per SM (128-line tiles: 2.29 ms with 1024 threads per SM, 2.44 with
+  // 768, 2.71 with 512; 64-line tiles of 16 x 2048^2: 144, 131 and 147 us)
+  static constexpr int N = (LA == 128 ? 1024 : 768) / ColCfg<LA>::THREADS, CTAS = N > 24 ? 24 : N;
 };
 template <int LA, bool FP64S>
 __global__ void __launch_bounds__(ColCfg<LA>::THREADS, BhCfg<LA>::CTAS)
@@ -1327,7 +1356,14 @@ static void launch_cols_b_variant(wst_plan_s *p, const float2 *planes, int p0, i
   if constexpr (LA >= 64) {
     CUtensorMap map;
     if (plane_tile_map(&map, planes, p->n, p1 - p0, LA)) {
-      k_cols_b_tma<LA, FP64S, CROP><<<grd, LA / 16 * kCB, 0, p->stream>>>(
+      // the planes of an image in this call: all n_w, or fewer if the call has fewer
+      const int run = p->n_w < p1 - p0 ? p->n_w : p1 - p0;
+      auto kern = k_cols_b_tma<LA, FP64S, CROP, 0>;
+      if constexpr (!FP64S) {
+        if (run <= kAnchor) kern = k_cols_b_tma<LA, FP64S, CROP, 1>;
+        else if (run <= 2 * kAnchor) kern = k_cols_b_tma<LA, FP64S, CROP, 2>;
+      }
+      kern<<<grd, LA / 16 * kCB, 0, p->stream>>>(
           map, p0, p1, p->n_w, tw_of(p), p->n, screen_ctx(p), image, comp, flags, p->n_img, p->crop,
           p->W_.counters + CNT_ERROR, p->wait_ns, (flags & ACC_RANGE_START) ? -1 : p0,
           (flags & ACC_RANGE_END) ? 0x7FFFFFFF : p1, ipz);
