@@ -828,7 +828,9 @@ static Tw tw_half(const wst_plan_s *p) {
 }
 
 // the grid of a persistent row kernel: every resident CTA, no more than there are rows for;
-// and the rows of a batch, so that each group gets eight batches or more of a long stream
+// and the rows of a batch, so that each group gets 32 batches or more of a long stream (dense
+// rows come in runs: with eight batches the gridder of 1M visibilities at 2048^2 x 16 ended on
+// a few groups, 245 us, now 157; rows one by one cost 4096^2 x 32 1428 instead of 1277 us)
 template <class C, class K>
 static cudaError_t persistent_grid(wst_plan_s *p, K kern, size_t smem, int64_t rows, int &grid, int &batch) {
   // always raised to the request: the 48 KB default counts the kernel's static shared
@@ -842,7 +844,7 @@ static cudaError_t persistent_grid(wst_plan_s *p, K kern, size_t smem, int64_t r
   if (e != cudaSuccess) return e;
   const int64_t resident = (int64_t)(per_sm > 0 ? per_sm : 1) * sms, need = (rows + C::ROWS - 1) / C::ROWS;
   grid = (int)(resident < need ? resident : need);
-  const int64_t b = rows / ((int64_t)grid * C::GROUPS * 8);
+  const int64_t b = rows / ((int64_t)grid * C::GROUPS * 32);
   for (batch = 1; 2 * batch <= b && 2 * batch <= kRowBatch;) batch *= 2;
   return cudaSuccess;
 }
