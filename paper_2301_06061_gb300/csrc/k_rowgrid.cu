@@ -32,7 +32,8 @@
 // fine quantum usable; but a cell or a single tap can exceed 2^31 delta = B/8 (a
 // dominant visibility, a coherent pile-up), so every integer atomic returns the old
 // value and the kernel checks for a wrapped partial sum or a saturated conversion: if
-// any occurred in the row, the row is zeroed and accumulated again with delta = B / 2^30.
+// any occurred in the row, the row is zeroed and accumulated again with delta = B / 2^32, or
+// B / 2^30.
 // Rows whose busiest bin holds fewer than 64 mean contributions take delta = B / 2^30,
 // which cannot overflow (sparse rows would otherwise overflow often; their cells are
 // few-term sums, for which the coarser quantum is precise enough).
@@ -53,7 +54,9 @@ namespace wst {
 // a dense row does not hold up the others, and empty rows cost no barrier of the CTA.  The
 // groups share the CTA's twiddle tables.  Rows shorter than 512 have fewer than 32 threads;
 // a group then takes GR rows in step.  CTAs of 128 threads, so that short workloads (a
-// 256^2 image has 16 rows per SM) still spread over the SMs.
+// 256^2 image has 16 rows per SM) still spread over the SMs.  With 256 threads on 2 to 16 rows
+// in step, an item and its offsets fetched row by row, 64 images of 2048^2 x 16 took 14.3 ms,
+// now 7.4, and a 256^2 one 20 us, now 6.8.
 template <int N, int MINT = 128>
 struct GroupCfg {
   static constexpr int EPT = RowCfg<N>::EPT, TPR = RowCfg<N>::TPR, PADL = RowCfg<N>::PADL;
@@ -381,17 +384,18 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
       ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps, pd);
     else grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
   }
-  // a tap or a partial sum left the int32 range: once more with delta = B / 2^30, which holds
-  // any row.  (Such a row has a cell of 1/64 of its busiest bin's magnitude or more, whose
-  // rounding in float would be as coarse.  Float atomics here are compare-and-swap loops that
-  // retry for every lane on the same cell, and these are the rows with many on one cell: with
-  // them a 2048^2 image of 1M visibilities on slow tracks spent 600 us in a few rows.)
-  if (sync.any(ovf < 0)) {
+  // a tap or a partial sum left the int32 range: once more with delta = B / 2^32, then with
+  // B / 2^30, which holds any row.  (Float atomics here are compare-and-swap loops that retry
+  // for every lane on the same cell, and these are the rows with many visibilities on one
+  // cell: with them a 2048^2 image of 1M visibilities on slow tracks spent 600 us in a few
+  // rows.)
+  for (int again = 0; again < 2 && sync.any(ovf < 0); ++again) {
     zero_row<N>(srow, jt);
     sync();
     if (nonempty && fixed) {
-      unit = 0x1p-30f;
-      grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps, pd);
+      unit = unit < 0x1p-32f ? 0x1p-32f : 0x1p-30f;
+      ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps,
+                                  pd);
     } else if (nonempty) {
       grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
     }
@@ -631,9 +635,12 @@ __device__ __forceinline__ void add_all(float *const (&at)[T], const float (&x)[
 // Rows are shared out as in k_grid_rows.  Degridding adds a record's row sum to its place in
 // sorted order (vacc, one 8-byte vector reduction; adjacent lanes hold adjacent records, so a
 // warp's reductions fall on whole sectors) and k_unsort hands the sums back in the caller's
-// order.  Two scalar reductions per record and row at the caller's index, the taps each
-// evaluated on their own and the records of each bucket shared out separately took 5.64 ms
-// for 10M visibilities on 16 planes of 8192^2.
+// order, or to the caller's place at once for few visibilities (dvis_order).  With two scalar
+// reductions per record and row at the caller's index, the records of each bucket shared out
+// on their own and 16 warps per SM, 10M visibilities on 16 planes of 8192^2 took 5.64 ms,
+// now 2.28 (32 warps).  Bound by the latency of a row's load, transform and records in turn
+// with two rows per SM; the taps stay evaluated one by one (the recurrence of the forward
+// gridder saves 0.13 ms here, but see below).
 template <int N, int WT, bool KGRAD>
 __global__ void __launch_bounds__(GroupCfg<N, KGRAD ? 256 : 128>::THREADS,
                                   N >= 16384 || (KGRAD && N == 8192) ? 1 : KGRAD || N == 8192 ? 2 : N == 4096 ? 3

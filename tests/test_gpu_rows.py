@@ -139,3 +139,22 @@ def test_table_gradient_with_shared_samples(wst, n, W, per_cell):
     got = plan.kernel_grad(dev(y[None])).cpu().numpy()
     ref = oracle.kernel_grad(ocfg, u, v, w, vis, y)
     assert np.abs(got - ref).max() <= 1e-4 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [2048, 8192])
+@pytest.mark.parametrize("n_w,chunk", [(16, 0), (17, 0), (32, 0), (33, 0), (33, 16), (20, 7)])
+def test_plane_sum_by_anchor_blocks(wst, n, n_w, chunk):
+    """The plane sum where the planes of an image in one call make one, two or more anchor
+    blocks of 16, whole and in chunks that cut them, at sampled pixels of the corrected
+    image's central half (64- and 128-line tiles)."""
+    fov, n_vis, n_pix = 0.1, 400, 48
+    rng = np.random.default_rng([n, n_w, chunk])
+    u, v, w = synth.disk_uvw(n_vis, 0.45 * n / fov, 150.0, rng)
+    vis = synth.random_visibilities(n_vis, rng)
+    cfg, ocfg = config(wst, n, fov, n_w, 7, planes_per_chunk=chunk)
+    plan = wst.Plan(cfg)
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis))
+    img = plan.image()[0].cpu().numpy()
+    pa, pb = rng.integers(n // 4, 3 * n // 4, (2, n_pix)).astype(np.int32)
+    ref = oracle.image_pixels(ocfg, u, v, w, vis, pa, pb)
+    assert np.abs(img[pb, pa] - ref).max() <= TOL * np.abs(ref).max()
