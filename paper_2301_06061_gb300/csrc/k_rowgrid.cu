@@ -730,9 +730,14 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
           aim = fmaf(gx, c.y, aim);
         });
         const float wt = __uint_as_float(__ldg(reinterpret_cast<const uint32_t *>(rec + s) + 5)) * gy;
-        const uint32_t at = dvis_order ? __ldg(&rec[s].index) : s;
-        asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(vacc + at), "f"(wt * are), "f"(wt * aim)
-                     : "memory");
+        float2 *at = vacc + (dvis_order ? __ldg(&rec[s].index) : s);
+        if (dvis_order && (reinterpret_cast<uintptr_t>(vacc) & 7u)) {  // a caller's array on 4 bytes
+          atomicAdd(&at->x, wt * are);
+          atomicAdd(&at->y, wt * aim);
+        } else {
+          asm volatile("red.relaxed.gpu.global.add.v2.f32 [%0], {%1, %2};" ::"l"(at), "f"(wt * are), "f"(wt * aim)
+                       : "memory");
+        }
       } else {
         // c_a = Re(conj(gh[q, i0 + a]) (w V)); x-profile tap a gets c_a G_y(d), the
         // y-profile tap d gets sum_a c_a G_x(a); each is split over the two table
@@ -816,10 +821,17 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
 
 // the sums of the sorted records back in the caller's order
 __global__ void k_unsort(const float2 *__restrict__ vacc, const Record *__restrict__ rec,
-                         const uint32_t *__restrict__ n_kept, float2 *__restrict__ dvis) {
+                         const uint32_t *__restrict__ n_kept, float *__restrict__ dvis) {
   const uint32_t n = *n_kept;
   for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    dvis[__ldcs(&rec[s].index)] = __ldcs(vacc + s);
+    const float2 x = __ldcs(vacc + s);
+    float *at = dvis + 2 * (size_t)__ldcs(&rec[s].index);
+    if (reinterpret_cast<uintptr_t>(dvis) & 7u) {  // a caller's array on 4 bytes
+      at[0] = x.x;
+      at[1] = x.y;
+    } else {
+      *reinterpret_cast<float2 *>(at) = x;
+    }
   }
 }
 
@@ -972,7 +984,7 @@ cudaError_t unsort_sums(wst_plan_s *p, float2 *dvis) {
   if (p->n_vis <= 0) return cudaSuccess;
   const int64_t blocks = (p->n_vis + 255) / 256;
   k_unsort<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, p->stream>>>(
-      p->W_.vacc, p->W_.records, p->W_.offsets + p->n_buckets, dvis);
+      p->W_.vacc, p->W_.records, p->W_.offsets + p->n_buckets, reinterpret_cast<float *>(dvis));
   p->launches += 1;
   return cudaGetLastError();
 }

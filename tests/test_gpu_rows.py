@@ -96,6 +96,12 @@ def test_degrid_in_either_summing_order(wst, n_vis):
         got = plan.degrid(dev(y[None]), flags=wst.WST_NO_CORRECTION).cpu().numpy()
         assert np.abs(got - want).max() <= TOL * np.abs(want).max()
         assert not got[::1001].any()
+    # an output that starts between two complex numbers' alignments (C callers)
+    raw = torch.empty(2 * n_vis + 1, dtype=torch.float32, device="cuda")
+    from paper_2301_06061_gb300.wst import WST_NO_CORRECTION, load_library
+    st = load_library().wst_degrid(plan.handle, dev(y[None]).data_ptr(), raw.data_ptr() + 4, WST_NO_CORRECTION)
+    odd = torch.view_as_complex(raw[1:].clone().view(-1, 2)).cpu().numpy()
+    assert st == 0 and np.abs(odd - want).max() <= TOL * np.abs(want).max()
 
 
 @pytest.mark.parametrize("n,batch,chunk,crop", [(64, 7, 0, 0), (256, 5, 4, 0), (512, 9, 0, 0), (512, 4, 3, 410),
