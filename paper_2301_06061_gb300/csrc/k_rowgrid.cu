@@ -41,7 +41,7 @@
 // per visibility-row (the bins count a visibility-row once per bin it reaches,
 // 1 + (W - 1)/64 bins on average) go straight to float atomics.  On the benchmark
 // workload the image error against the FP64 oracle equals that of all-float
-// accumulation.  Rows shorter than 8192 take finer steps of the quantum (log2_unit): shared
+// accumulation.  Rows shorter than 8192 step the quantum of sparse rows (unit_of): shared
 // float atomics are compare-and-swap loops, and integer ones took this kernel from 1.74 to
 // 1.30 ms at 4096^2 x 32 planes (4.08M visibilities), from 16.2 to 14.0 ms on 64 images of
 // 2048^2 x 16 (37.7M) and the 256^2 one from 26 to 20 us, at the same error against FP64.
@@ -192,17 +192,18 @@ template <int N>
 constexpr bool kBinnedRows = bins_per_row(N) > 1;
 
 // log2(delta / B) of a row shorter than 8192, n_eff the mean contributions in its busiest bin
-// (one bin: all of the row).  The rounding of a tap stays near 2^-28 of the mean magnitude
-// while the bins are sparse, that of a float sum of a few taps, and a cell may hold, before
-// the row is accumulated again, the whole bin of fewer than 16, above that 8 or more mean
-// contributions in phase at weight 1 (taps average a tenth of it).  With 2^-34 of a whole
-// row's magnitude for every count above 256 the error against FP64 at 4096^2 (4.08M
-// visibilities) was 8.7e-6, with this 5.1e-6, with float atomics 5.6e-6.
-__device__ __forceinline__ int log2_unit(float n_eff) {
-  if (n_eff < 16.0f) return -30;
-  if (n_eff < 64.0f) return -32;
-  if (n_eff < 256.0f) return -34;
-  return n_eff < 1024.0f ? -35 : n_eff < 4096.0f ? -36 : -37;
+// (one bin: all of the row).  Sparse bins hold sums of a few taps: up to 64 the quantum stays
+// near 2^-28 of the mean magnitude, the rounding of a float tap, and a cell may hold, before
+// the row is accumulated again, the whole bin below 16 and half of it below 64.  From 64 on
+// it is B / 2^34, a cell up to an eighth of the bin: dense bins round in float by more than
+// that (their partial sums grow with the count), and where their values are in phase a cell
+// holds about a sixtieth of the bin, so that a finer quantum would send dense rows through
+// twice or more (2^-37 from 4096 on: 24.0 instead of 13.3 ms for eight 2048^2 images of 3.3M
+// visibilities with the ES kernel of 10 cells).  With 2^-34 of a whole row's magnitude instead
+// of a bin's the error against FP64 at 4096^2 (4.08M visibilities) was 8.7e-6, with float
+// atomics it is 5.6e-6.
+__device__ __forceinline__ float unit_of(float n_eff) {
+  return n_eff < 16.0f ? 0x1p-30f : n_eff < 64.0f ? 0x1p-32f : 0x1p-34f;
 }
 
 // one tap into the planar row: float atomics, or (FIXED) the tap already in units of the
@@ -377,7 +378,7 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range
   float unit;
   if constexpr (N >= 8192) unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
-  else unit = __int_as_float((127 + log2_unit(n_eff)) << 23);
+  else unit = unit_of(n_eff);
   int ovf = 0;
   if (nonempty) {
     if (fixed)
