@@ -197,9 +197,8 @@ constexpr bool kBinnedRows = bins_per_row(N) > 1;
 // the row is accumulated again, the whole bin below 16 and half of it below 64.  From 64 on
 // it is B / 2^34, a cell up to an eighth of the bin: dense bins round in float by more than
 // that (their partial sums grow with the count), and where their values are in phase a cell
-// holds about a sixtieth of the bin, so that a finer quantum would send dense rows through
-// twice or more (2^-37 from 4096 on: 24.0 instead of 13.3 ms for eight 2048^2 images of 3.3M
-// visibilities with the ES kernel of 10 cells).  With 2^-34 of a whole row's magnitude instead
+// holds about a sixtieth of the bin, so that a finer quantum could send dense rows through
+// twice.  With 2^-34 of a whole row's magnitude instead
 // of a bin's the error against FP64 at 4096^2 (4.08M visibilities) was 8.7e-6, with float
 // atomics it is 5.6e-6.
 __device__ __forceinline__ float unit_of(float n_eff) {
@@ -865,7 +864,10 @@ static cudaError_t persistent_grid(wst_plan_s *p, K kern, size_t smem, int64_t r
   const int64_t resident = (int64_t)(per_sm > 0 ? per_sm : 1) * sms, need = (rows + C::ROWS - 1) / C::ROWS;
   grid = (int)(resident < need ? resident : need);
   const int64_t b = rows / ((int64_t)grid * C::GROUPS * 32);
-  for (batch = 1; 2 * batch <= b && 2 * batch <= kRowBatch;) batch *= 2;
+  // short rows have few threads for a dense row: eight at a time, 26.6M visibilities on eight
+  // 2048^2 images (W = 10) took 18.5 ms, two 8.0 (64 sparser images 7.4 and 7.8)
+  const int most = C::TPR <= 128 ? 2 : kRowBatch;
+  for (batch = 1; 2 * batch <= b && 2 * batch <= most;) batch *= 2;
   return cudaSuccess;
 }
 
