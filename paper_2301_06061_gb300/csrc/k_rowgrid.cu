@@ -41,10 +41,12 @@
 // per visibility-row (the bins count a visibility-row once per bin it reaches,
 // 1 + (W - 1)/64 bins on average) go straight to float atomics.  On the benchmark
 // workload the image error against the FP64 oracle equals that of all-float
-// accumulation.  Rows shorter than 8192 step the quantum of sparse rows (unit_of): shared
-// float atomics are compare-and-swap loops, and integer ones took this kernel from 1.74 to
-// 1.30 ms at 4096^2 x 32 planes (4.08M visibilities), from 16.2 to 14.0 ms on 64 images of
-// 2048^2 x 16 (37.7M) and the 256^2 one from 26 to 20 us, at the same error against FP64.
+// accumulation.  Rows shorter than 8192 keep float sums.  Integer ones took 1.30 instead of
+// 1.74 ms at 4096^2 x 32 planes (4.08M visibilities), but one quantum for the whole row takes
+// bits from every cell far below its busiest bin (the caller of wst_grid sees them), and a
+// grid correction of 1e5 or more shows the other rounding in the image: at the sizes of
+// those rows it repeats from call to call, and a 512^2 image of 6,300 visibilities with an
+// unpadded Kaiser-Bessel table of 8 came out 50% different.
 #include "fft_core.cuh"
 
 namespace wst {
@@ -186,24 +188,8 @@ __device__ __forceinline__ void for_taps(const KernelParams &kp, const float *ta
 }
 
 constexpr int kFixedBinCap = 8192;
-// rows whose bound comes from column bins (k_row_bounds); the others' is the sum of their W
-// buckets' magnitudes
 template <int N>
-constexpr bool kBinnedRows = bins_per_row(N) > 1;
-
-// log2(delta / B) of a row shorter than 8192, n_eff the mean contributions in its busiest bin
-// (one bin: all of the row).  Sparse bins hold sums of a few taps: up to 64 the quantum stays
-// near 2^-28 of the mean magnitude, the rounding of a float tap, and a cell may hold, before
-// the row is accumulated again, the whole bin below 16 and half of it below 64.  From 64 on
-// it is B / 2^34, a cell up to an eighth of the bin: dense bins round in float by more than
-// that (their partial sums grow with the count), and where their values are in phase a cell
-// holds about a sixtieth of the bin, so that a finer quantum could send dense rows through
-// twice.  With 2^-34 of a whole row's magnitude instead
-// of a bin's the error against FP64 at 4096^2 (4.08M visibilities) was 8.7e-6, with float
-// atomics it is 5.6e-6.
-__device__ __forceinline__ float unit_of(float n_eff) {
-  return n_eff < 16.0f ? 0x1p-30f : n_eff < 64.0f ? 0x1p-32f : 0x1p-34f;
-}
+constexpr bool kFixedRows = N >= kFixedMinN;
 
 // one tap into the planar row: float atomics, or (FIXED) the tap already in units of the
 // row's quantum (the record's value was scaled by 1/delta once), converted and added as
@@ -367,17 +353,13 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   const uint32_t cnt = nonempty ? bnd[d_lo + 1] - bnd[0] : 0u;
   const float mmax = mb.x, mtot = mb.y;
   const float bound = mmax * (gmax * gmax);
-  // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row (one
-  // bin: the row's visibilities)
-  const float n_eff = !kBinnedRows<N> ? (float)cnt
-                      : mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
-  const bool fixed = nonempty && cnt < (1u << 30) && bound >= 0x1p-87f && bound <= 0x1p+100f &&
+  // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row
+  const float n_eff = mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
+  const bool fixed = kFixedRows<N> && nonempty && cnt < (1u << 30) && bound >= 0x1p-87f && bound <= 0x1p+100f &&
                      n_eff <= (float)kFixedBinCap;
   // a bin of fewer than ~64 mean contributions may hold a single tap above B/8: such rows
   // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range
-  float unit;
-  if constexpr (N >= 8192) unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
-  else unit = unit_of(n_eff);
+  float unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
   int ovf = 0;
   if (nonempty) {
     if (fixed)
@@ -389,7 +371,8 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   // for every lane on the same cell, and these are the rows with many visibilities on one
   // cell: with them a 2048^2 image of 1M visibilities on slow tracks spent 600 us in a few
   // rows.)
-  for (int again = 0; again < 2 && sync.any(ovf < 0); ++again) {
+  if constexpr (!kFixedRows<N>) sync();
+  for (int again = 0; kFixedRows<N> && again < 2 && sync.any(ovf < 0); ++again) {
     zero_row<N>(srow, jt);
     sync();
     if (nonempty && fixed) {
@@ -462,7 +445,7 @@ __global__ void __launch_bounds__(GridCfg<N>::THREADS,
 k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, int p0, int np,
             KernelParams kp, float2 *__restrict__ out, uint8_t *__restrict__ occ,
             unsigned long long *__restrict__ counter, Tw tw, const float2 *__restrict__ rowbound,
-            const float *__restrict__ binmag, unsigned long long *__restrict__ rows_done, int batch, bool smem_taps) {
+            unsigned long long *__restrict__ rows_done, int batch, bool smem_taps) {
   using C = GridCfg<N>;
   constexpr int TPR = C::TPR, GT = C::GT, GR = C::GR, GROUPS = C::GROUPS;
   extern __shared__ __align__(16) float2 sm_rows[];
@@ -510,7 +493,8 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
         if (gt < W + batch && j >= 0)
           cp_async_small<4>(off_sm + (uint32_t)(buf * (kRowBatch + kMaxSupport + 1) + gt) * 4u,
                             off + (b0 + j) * kColBlocks);
-        if (gt < batch) cp_async_small<8>(rb_sm + (uint32_t)(buf * kRowBatch + gt) * 8u, rowbound + b0 + q0 + gt);
+        if (kFixedRows<N> && gt < batch)
+          cp_async_small<8>(rb_sm + (uint32_t)(buf * kRowBatch + gt) * 8u, rowbound + b0 + q0 + gt);
       }
     };
     // the transforming path of long rows writes each row during the next row's gridding
@@ -557,7 +541,8 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
         const long long item = base + r;
         const int pl = (int)(item / N), q = (int)(item % N);
         const int d_lo = min(q, W - 1);
-        grid_one_row<N, FFT, WT>(srow, &s_off[g][buf][r + W - 1 - d_lo], d_lo, s_rb[g][buf][r], rec, q, e & 1, kp,
+        const float2 mb = kFixedRows<N> ? s_rb[g][buf][r] : make_float2(0.0f, 0.0f);
+        grid_one_row<N, FFT, WT>(srow, &s_off[g][buf][r + W - 1 - d_lo], d_lo, mb, rec, q, e & 1, kp,
                                  out + ((int64_t)pl * N + q) * N, twt, jt, gmax, stg, stg_stride, taps, pd, sync);
       }
       if (cnt == 0) sync();  // s_item, s_cnt and the list are read before they are written again
@@ -566,8 +551,7 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
     asm volatile("cp.async.wait_all;" ::: "memory");
   } else {
     __shared__ uint32_t s_bnd[C::ROWS][kMaxSupport + 2];
-    __shared__ float s_mag[C::ROWS][kMaxSupport + 2];
-    static_assert(!kBinnedRows<N>, "one bin per row");
+    static_assert(!kFixedRows<N>, "float sums");
     long long next = group0 * GR;
     while (true) {
       const long long base = __shfl_sync(0xFFFFFFFFu, next, 0);  // a group is one warp here
@@ -579,21 +563,16 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
       const int q = valid ? (int)(item % N) : 0;
       const int64_t b0 = (int64_t)(p0 + pl) * N;
       const int d_lo = min(q, W - 1);
-      for (int i = jt; i <= d_lo + 1; i += TPR) {
-        s_bnd[rl][i] = off[(b0 + q - d_lo + i) * kColBlocks];
-        s_mag[rl][i] = i <= d_lo ? __ldg(binmag + b0 + q - d_lo + i) : 0.0f;
-      }
+      for (int i = jt; i <= d_lo + 1; i += TPR) s_bnd[rl][i] = off[(b0 + q - d_lo + i) * kColBlocks];
       __syncwarp();
       const bool empty = !valid || s_bnd[rl][0] == s_bnd[rl][d_lo + 1];
       if (valid && jt == 0) occ[item] = empty ? 0 : 1;
       if (rows_done && valid && jt == 0 && !empty) atomicAdd(rows_done, 1ull);
       if (!FFT || !__all_sync(0xFFFFFFFFu, empty)) {
-        float2 mb = make_float2(0.0f, 0.0f);
-        for (int i = 0; i <= d_lo; ++i) mb.x += s_mag[rl][i];
         float2 *orow = valid && (!FFT || !empty) ? out + ((int64_t)pl * N + q) * N : nullptr;
         NoPending none;
-        grid_one_row<N, FFT, WT>(srow, s_bnd[rl], d_lo, mb, rec, q, !empty, kp, orow, twt, jt, gmax, stg, stg_stride,
-                                 taps, none, sync);
+        grid_one_row<N, FFT, WT>(srow, s_bnd[rl], d_lo, make_float2(0.0f, 0.0f), rec, q, !empty, kp, orow, twt, jt, gmax,
+                                 stg, stg_stride, taps, none, sync);
       }
       __syncwarp();
     }
@@ -896,7 +875,7 @@ static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) 
   if (e != cudaSuccess) return e;
   unsigned long long *counter = p->W_.counters + CNT_WORK;  // cleared by the caller
   kern<<<grid, C::THREADS, smem, p->stream>>>(p->W_.records, p->W_.offsets, p0, np, kernel_params(p), out,
-                                             p->W_.occ, counter, tw_half(p), p->W_.rowbound, p->W_.binmag,
+                                             p->W_.occ, counter, tw_half(p), p->W_.rowbound,
                                              FFT ? p->W_.counters + CNT_ROWS : nullptr, batch, smem_taps);
   return cudaGetLastError();
 }

@@ -494,7 +494,7 @@ __global__ void k_scatter(const float2 *__restrict__ vis, const float *__restric
         vre = val[h].x * wt[h];
         vim = (ki[h].y ? -val[h].y : val[h].y) * wt[h];  // mirrored: conj
       }
-      {  // the whole warp: the first bin by runs, the second (rare) directly
+      if (binmag) {  // the whole warp: the first bin by runs, the second (rare) directly
         const float mag = fmaxf(fabsf(vre), fabsf(vim));
         const int i0 = (int)(ki[h].z >> 18);
         const int bl = min(i0 >> kBinShift, nb - 1), bh = min((i0 + W - 1) >> kBinShift, nb - 1);
@@ -630,9 +630,9 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
   if ((e = cudaGetLastError())) return e;
   if ((e = scan_exclusive(ws.offsets, nb1, ws.scan_tmp, s, p->launches, ws.cursor))) return e;
   k_scatter<<<grid_for(p->n_vis, 256, 152 * 16), 256, 0, s>>>(vis, weight, ws.keyinfo, ws.cursor, p->n_vis,
-                                                              ws.records, ws.binmag, nb, p->W, stash);
+                                                              ws.records, nb > 0 ? ws.binmag : nullptr, nb, p->W, stash);
   p->launches += 1;
-  if (nb > 1) {
+  if (nb > 0) {
     const int64_t n_rows = p->n_buckets / kColBlocks;
     const auto bounds = p->W <= 8 ? k_row_bounds<8> : k_row_bounds<kMaxSupport>;
     bounds<<<grid_for(n_rows * (32 / kBoundRows), 256, 152 * 8), 256, 0, s>>>(ws.binmag, ws.offsets, n_rows, p->n, nb,

@@ -76,7 +76,7 @@ Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
   L.occ = off;
   off += align_up((size_t)p->n_planes * p->n);
   L.rowbound = off;
-  if (bins_per_row(p->n) > 1) off += align_up((size_t)(p->n_buckets / kColBlocks) * sizeof(float2));
+  if (bins_per_row(p->n) > 0) off += align_up((size_t)(p->n_buckets / kColBlocks) * sizeof(float2));
   L.comp = off;
   if (p->chunk < p->n_planes) off += align_up((size_t)p->batch * p->n_img * p->n_img * sizeof(float2));
   L.vacc = off;

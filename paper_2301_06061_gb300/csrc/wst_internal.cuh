@@ -18,11 +18,10 @@ constexpr int kColBlocks = 1;    // sub-buckets per row (by tap-start column; a 
 constexpr uint32_t kDropKey = 0xFFFFFFFFu;
 // Column bins of the fixed-point gridder's bound: for every row bucket (image, plane, j0)
 // the sort sums max(|Re|, |Im|) of the weighted values whose W taps reach each bin of
-// kBinCols columns.  The shortest rows have one bin, the whole row: their calls are bound by
-// launches, and a bound over a few bins would cost one more (k_row_bounds).
+// kBinCols columns.  Only images whose rows use fixed-point accumulation have them.
 constexpr int kBinCols = 64, kBinShift = 6;
-constexpr int kBinnedMinN = 512;
-__host__ __device__ constexpr int bins_per_row(int n) { return n >= kBinnedMinN ? n / kBinCols : 1; }
+constexpr int kFixedMinN = 8192;
+__host__ __device__ constexpr int bins_per_row(int n) { return n >= kFixedMinN ? n / kBinCols : 0; }
 
 // counters[] slots in the workspace
 // CNT_ROWS: non-empty (plane, row) items the imaging path gridded since wst_image began
@@ -93,7 +92,7 @@ struct Workspace {
   uint32_t *wminmax;   // per image: ordered-int min and max of finite w
   uint8_t *occ;        // per (plane of the chunk, row): 1 if any visibility reaches the row
   float *binmag;       // per (row bucket, column bin): magnitude sum (fixed-point bound)
-  float2 *rowbound;    // binned rows only: (largest bin sum, total of the bin sums) over the W buckets
+  float2 *rowbound;    // per grid row: (largest bin sum, total of the bin sums) over its W buckets
   float2 *planes;      // chunk of planes
   float2 *comp;        // Kahan compensation image [batch][N*N]
   float2 *vacc;        // per sorted record: the degridded sum before its weight

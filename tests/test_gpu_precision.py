@@ -1,0 +1,64 @@
+"""GPU results held to FP32 precision where a shared quantum, a summation order or a reduced
+argument could take bits from them.  References: the FP64 oracle, or the same formula in
+numpy FP64; each test derives its bound."""
+import numpy as np
+import pytest
+
+import oracle
+from oracle import OracleConfig
+from paper_2301_06061_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def wst():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2301_06061_gb300 import build, wst as w
+
+    build.build()
+    w.load_library()
+    return w
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+# ------------------------------------------------------------------------------------------
+# gridder
+# ------------------------------------------------------------------------------------------
+
+def assert_cells(wst, cfg, ocfg, u, v, w, vis, adds):
+    """Every cell of wst_grid's planes within FP32 of its own terms: |error| <= eps S with S the
+    sum of the terms' magnitudes in that cell, eps = (adds + 32) 2^-24 (`adds` roundings of
+    partial sums; 32 for the two taps, whose argument of up to 4 cells is rounded to 2^-24
+    cell under a slope of at most 5 per cell, their exponentials and the products)."""
+    plan = wst.Plan(cfg)
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis))
+    g = torch.empty((cfg.n_w, cfg.n, cfg.n), dtype=torch.complex64, device="cuda")
+    wst.wst_grid(plan.handle, 0, cfg.n_w, g)
+    got = g.cpu().numpy()
+    ref = oracle.grid(ocfg, u, v, w, vis)
+    size = oracle.grid(ocfg, u, v, w, (np.abs(vis.real) + np.abs(vis.imag)).astype(np.complex64)).real
+    assert np.all(np.abs(got - ref) <= (adds + 32) * 2.0 ** -24 * size)
+
+
+@pytest.mark.parametrize("n", [64, 128, 256, 512, 1024, 2048, 4096])
+@pytest.mark.parametrize("W", [6, 7, 8])
+def test_cells_far_below_a_bright_one(wst, n, W):
+    """300 values of order one and one of 1e6 in the same rows: the other cells keep their own
+    precision (a quantum taken from the rows' brightest bin would leave them ten bits)."""
+    rng = np.random.default_rng([n, W])
+    fov, n_vis = 0.1, 301
+    u = (rng.uniform(-0.4, 0.4, n_vis) * n / fov).astype(np.float32)
+    v = np.full(n_vis, 3.3 / fov, np.float32)
+    w = np.zeros(n_vis, np.float32)
+    vis = synth.random_visibilities(n_vis, rng)
+    vis[0] = 1e6
+    sigma = {6: 0.81, 7: 0.875, 8: 0.925}[W]
+    cfg = wst.Config(n=n, fov=fov, n_w=1, w_min=-10.0, w_max=10.0, support=W, kparam=sigma)
+    ocfg = OracleConfig(n, fov, 1, -10.0, 10.0, W, "gauss", sigma)
+    assert_cells(wst, cfg, ocfg, u, v, w, vis, adds=301 if n == 64 else 64)
