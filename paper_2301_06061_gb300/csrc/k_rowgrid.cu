@@ -32,8 +32,7 @@
 // fine quantum usable; but a cell or a single tap can exceed 2^31 delta = B/8 (a
 // dominant visibility, a coherent pile-up), so every integer atomic returns the old
 // value and the kernel checks for a wrapped partial sum or a saturated conversion: if
-// any occurred in the row, the row is zeroed and accumulated again with delta = B / 2^32, or
-// B / 2^30.
+// any occurred in the row, the row is zeroed and accumulated again with float atomics.
 // Rows whose busiest bin holds fewer than 64 mean contributions take delta = B / 2^30,
 // which cannot overflow (sparse rows would otherwise overflow often; their cells are
 // few-term sums, for which the coarser quantum is precise enough).
@@ -280,7 +279,7 @@ struct NoPending {
 
 // With FIXED, qscale = 1/delta and gmax the largest |kernel value|: a record whose scaled
 // value times gmax comes within 0.2% of 2^31 (a margin for the rounding of the taps)
-// could saturate a conversion, and sends the row through again like a wrapped sum.
+// could saturate a conversion, and sends the row to float atomics like a wrapped sum.
 template <int N, int WT, bool FIXED, class PEND>
 __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__restrict__ rec,
                                         const uint32_t *bnd, int d_lo, const KernelParams &kp, int jt,
@@ -355,41 +354,37 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   const float bound = mmax * (gmax * gmax);
   // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row
   const float n_eff = mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
-  const bool fixed = kFixedRows<N> && nonempty && cnt < (1u << 30) && bound >= 0x1p-87f && bound <= 0x1p+100f &&
+  const bool fixed = kFixedRows<N> && nonempty && cnt < (1u << 30) && bound >= 0x1p-90f && bound <= 0x1p+100f &&
                      n_eff <= (float)kFixedBinCap;
   // a bin of fewer than ~64 mean contributions may hold a single tap above B/8: such rows
   // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range
-  float unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
+  const float unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
+  bool fx = fixed;
   int ovf = 0;
   if (nonempty) {
     if (fixed)
       ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps, pd);
     else grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
   }
-  // a tap or a partial sum left the int32 range: once more with delta = B / 2^32, then with
-  // B / 2^30, which holds any row.  (Float atomics here are compare-and-swap loops that retry
-  // for every lane on the same cell, and these are the rows with many visibilities on one
-  // cell: with them a 2048^2 image of 1M visibilities on slow tracks spent 600 us in a few
-  // rows.)
-  if constexpr (!kFixedRows<N>) sync();
-  for (int again = 0; kFixedRows<N> && again < 2 && sync.any(ovf < 0); ++again) {
+  // a tap or a partial sum left the int32 range: accumulate in float.  (A coarser quantum,
+  // B / 2^32 or B / 2^30, would hold the row too, but leaves the cells far below the busiest
+  // bin ten bits.)
+  bool redo = false;
+  if constexpr (kFixedRows<N>) redo = sync.any(ovf < 0);
+  else sync();
+  if (redo) {
     zero_row<N>(srow, jt);
     sync();
-    if (nonempty && fixed) {
-      unit = unit < 0x1p-32f ? 0x1p-32f : 0x1p-30f;
-      ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps,
-                                  pd);
-    } else if (nonempty) {
-      grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
-    }
+    if (nonempty) grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
+    fx = false;
     sync();
   }
   pd.write_all(jt);  // the previous row is out before this one's transform takes its place
-  const float delta = fixed ? bound * unit : 1.0f;
+  const float delta = fx ? bound * unit : 1.0f;
   const int *ire = reinterpret_cast<const int *>(sre), *iim = reinterpret_cast<const int *>(sim);
   if constexpr (FFT) {
     float2 v[EPT];
-    if (fixed) {
+    if (fx) {
 #pragma unroll
       for (int b = 0; b < EPT / R0; ++b)
 #pragma unroll
@@ -429,7 +424,7 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
     }
   } else {
     if (orow) {
-      if (fixed)
+      if (fx)
         for (int i = jt; i < N; i += TPR)
           orow[i] = make_float2(delta * __int2float_rn(ire[i]), delta * __int2float_rn(iim[i]));
       else
