@@ -606,23 +606,23 @@ __device__ __forceinline__ void add_all(float *const (&at)[T], const float (&x)[
     if (at[t] && got[t] != old[t]) atomicAdd(at[t] + offset, x[t]);
 }
 
-// Rows are shared out as in k_grid_rows.  Degridding adds a record's row sum to its place in
-// sorted order (vacc, one 8-byte vector reduction; adjacent lanes hold adjacent records, so a
-// warp's reductions fall on whole sectors) and k_unsort hands the sums back in the caller's
-// order, or to the caller's place at once for few visibilities (dvis_order).  With two scalar
-// reductions per record and row at the caller's index, the records of each bucket shared out
-// on their own and 16 warps per SM, 10M visibilities on 16 planes of 8192^2 took 5.64 ms,
-// now 2.28 (32 warps).  Bound by the latency of a row's load, transform and records in turn
-// with two rows per SM; the taps stay evaluated one by one (the recurrence of the forward
-// gridder saves 0.13 ms here, but see below).
+// Rows are shared out as in k_grid_rows.  Degridding adds a record's row sum to the caller's
+// element, one 8-byte vector reduction.  (Sums kept in sorted order, where a warp's
+// reductions fall on whole sectors, and handed back by a pass of their own took as long, the
+// whole call 6.69 against 6.66 ms at 10M visibilities on 16 planes of 8192^2 and 17.2 against
+// 16.9 at 20M on 8 of 16384^2, and 8 bytes of workspace per visibility.)  With two scalar
+// reductions per record and row, the records of each bucket shared out on their own and
+// 16 warps per SM, the former took 5.64 ms, now 2.28 (32 warps).  Bound by the latency of a
+// row's load, transform and records in turn with two rows per SM; the taps stay evaluated one
+// by one (the recurrence of the forward gridder saves 0.13 ms here, but see below).
 template <int N, int WT, bool KGRAD>
 __global__ void __launch_bounds__(GroupCfg<N, KGRAD ? 256 : 128>::THREADS,
                                   N >= 16384 || (KGRAD && N == 8192) ? 1 : KGRAD || N == 8192 ? 2 : N == 4096 ? 3
                                   : 1024 / GroupCfg<N>::THREADS)
 k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec,
                const uint32_t *__restrict__ off, int p0, int np, KernelParams kp,
-               float2 *__restrict__ vacc, float *__restrict__ dtab,
-               unsigned long long *__restrict__ counter, Tw tw, int batch, bool dvis_order) {
+               float2 *__restrict__ dvis, float *__restrict__ dtab,
+               unsigned long long *__restrict__ counter, Tw tw, int batch) {
   using C = GroupCfg<N, KGRAD ? 256 : 128>;
   constexpr int EPT = C::EPT, TPR = C::TPR, GT = C::GT, GR = C::GR, GROUPS = C::GROUPS;
   constexpr int NST = num_stages(N, EPT);
@@ -703,9 +703,10 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
           are = fmaf(gx, c.x, are);
           aim = fmaf(gx, c.y, aim);
         });
-        const float wt = __uint_as_float(__ldg(reinterpret_cast<const uint32_t *>(rec + s) + 5)) * gy;
-        float2 *at = vacc + (dvis_order ? __ldg(&rec[s].index) : s);
-        if (dvis_order && (reinterpret_cast<uintptr_t>(vacc) & 7u)) {  // a caller's array on 4 bytes
+        const uint2 tail = __ldg(reinterpret_cast<const uint2 *>(rec + s) + 2);  // index, weight
+        const float wt = __uint_as_float(tail.y) * gy;
+        float2 *at = dvis + tail.x;
+        if (reinterpret_cast<uintptr_t>(dvis) & 7u) {  // a caller's array on 4 bytes
           atomicAdd(&at->x, wt * are);
           atomicAdd(&at->y, wt * aim);
         } else {
@@ -793,22 +794,6 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
   }
 }
 
-// the sums of the sorted records back in the caller's order
-__global__ void k_unsort(const float2 *__restrict__ vacc, const Record *__restrict__ rec,
-                         const uint32_t *__restrict__ n_kept, float *__restrict__ dvis) {
-  const uint32_t n = *n_kept;
-  for (uint32_t s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
-    const float2 x = __ldcs(vacc + s);
-    float *at = dvis + 2 * (size_t)__ldcs(&rec[s].index);
-    if (reinterpret_cast<uintptr_t>(dvis) & 7u) {  // a caller's array on 4 bytes
-      at[0] = x.x;
-      at[1] = x.y;
-    } else {
-      *reinterpret_cast<float2 *>(at) = x;
-    }
-  }
-}
-
 // -------------------------------------------------------------------------------------
 // host side
 // -------------------------------------------------------------------------------------
@@ -889,7 +874,7 @@ static cudaError_t launch_rows_adjoint(wst_plan_s *p, int p0, int np, const floa
   if (e != cudaSuccess) return e;
   unsigned long long *counter = p->W_.counters + CNT_WORK;  // cleared by row_occupancy
   kern<<<grid, C::THREADS, smem, p->stream>>>(planes, p->W_.records, p->W_.offsets, p0, np, kernel_params(p),
-                                             dvis ? dvis : p->W_.vacc, dtab, counter, tw_half(p), batch, dvis != nullptr);
+                                             dvis, dtab, counter, tw_half(p), batch);
   return cudaGetLastError();
 }
 
@@ -953,15 +938,6 @@ cudaError_t row_occupancy(wst_plan_s *p, int p0, int p1) {
   if (rows <= 0) return cudaSuccess;
   k_row_occ<<<(unsigned)((rows + 255) / 256), 256, 0, p->stream>>>(p->W_.offsets, (int64_t)p0 * p->n, rows, p->n, p->W,
                                                                    p->W_.occ, p->W_.counters + CNT_WORK);
-  p->launches += 1;
-  return cudaGetLastError();
-}
-
-cudaError_t unsort_sums(wst_plan_s *p, float2 *dvis) {
-  if (p->n_vis <= 0) return cudaSuccess;
-  const int64_t blocks = (p->n_vis + 255) / 256;
-  k_unsort<<<(unsigned)(blocks < 152 * 16 ? blocks : 152 * 16), 256, 0, p->stream>>>(
-      p->W_.vacc, p->W_.records, p->W_.offsets + p->n_buckets, reinterpret_cast<float *>(dvis));
   p->launches += 1;
   return cudaGetLastError();
 }

@@ -42,14 +42,8 @@ int ilog2(int x) {
   return l;
 }
 
-// From this many visibilities on, degridding sums are kept per sorted record and handed back
-// by a pass of their own: whole sectors per reduction instead of scattered ones, for two more
-// launches.  1M visibilities of a 2048^2 image: 174 instead of 178 us; 168k of a 512^2 one: 85
-// instead of 76 us.
-constexpr int64_t kSortedSums = 1 << 19;
-
 struct Layout {
-  size_t keyinfo_planes, records, offsets, cursor, scan_tmp, counters, wminmax, occ, binmag, rowbound, comp, vacc, total;
+  size_t keyinfo_planes, records, offsets, cursor, scan_tmp, counters, wminmax, occ, binmag, rowbound, comp, total;
 };
 
 Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
@@ -79,8 +73,6 @@ Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
   if (bins_per_row(p->n) > 0) off += align_up((size_t)(p->n_buckets / kColBlocks) * sizeof(float2));
   L.comp = off;
   if (p->chunk < p->n_planes) off += align_up((size_t)p->batch * p->n_img * p->n_img * sizeof(float2));
-  L.vacc = off;
-  if (n_vis >= kSortedSums) off += align_up((size_t)n_vis * sizeof(float2));
   L.total = off;
   return L;
 }
@@ -357,7 +349,6 @@ static wst_status set_vis_common(wst_plan_s *p, int64_t n_vis, const VisCoords &
   W.binmag = (float *)(p->ws + L.binmag);
   W.rowbound = (float2 *)(p->ws + L.rowbound);
   W.comp = (p->chunk < p->n_planes) ? (float2 *)(p->ws + L.comp) : nullptr;
-  W.vacc = (float2 *)(p->ws + L.vacc);
   W.bytes = L.total;
   p->launches = 0;
   p->n_vis = n_vis;
@@ -506,21 +497,15 @@ wst_status wst_degrid(wst_plan p, const void *dimage, void *dvis, uint32_t flags
   if (flags & ~WST_NO_CORRECTION) return fail(p, WST_ERR_INVALID_ARG, "unknown flags");
   if (p->cfg.flags & WST_FLAG_WFOLD) return fail(p, WST_ERR_UNSUPPORTED, "no adjoint with WST_FLAG_WFOLD");
   const bool correct = !(flags & WST_NO_CORRECTION);
-  const bool sorted = p->n_vis >= kSortedSums;
-  if (p->n_vis > 0) {
-    WST_CUDA(p, cudaMemsetAsync(dvis, 0, sizeof(float2) * p->n_vis, p->stream), "memset");
-    if (sorted) WST_CUDA(p, cudaMemsetAsync(p->W_.vacc, 0, sizeof(float2) * p->n_vis, p->stream), "memset");
-  }
+  if (p->n_vis > 0) WST_CUDA(p, cudaMemsetAsync(dvis, 0, sizeof(float2) * p->n_vis, p->stream), "memset");
   float2 *planes = p->W_.planes;
   for (int p0 = 0; p0 < p->n_planes; p0 += p->chunk) {
     const int p1 = (p0 + p->chunk < p->n_planes) ? p0 + p->chunk : p->n_planes;
     WST_CUDA(p, fft_cols_bh_from_image(p, (const float2 *)dimage, p0, p1, planes, correct), "cols B^H");
     WST_CUDA(p, row_occupancy(p, p0, p1), "row occupancy");
     WST_CUDA(p, fft_cols_a(p, planes, p1 - p0, -1, true, p->W_.occ), "cols A^H");
-    WST_CUDA(p, rows_adjoint(p, p0, p1, planes, sorted ? nullptr : (float2 *)dvis, nullptr),
-             "rows^H + degrid");
+    WST_CUDA(p, rows_adjoint(p, p0, p1, planes, (float2 *)dvis, nullptr), "rows^H + degrid");
   }
-  if (sorted) WST_CUDA(p, unsort_sums(p, (float2 *)dvis), "unsort");
   return WST_OK;
 }
 

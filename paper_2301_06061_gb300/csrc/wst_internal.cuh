@@ -95,7 +95,6 @@ struct Workspace {
   float2 *rowbound;    // per grid row: (largest bin sum, total of the bin sums) over its W buckets
   float2 *planes;      // chunk of planes
   float2 *comp;        // Kahan compensation image [batch][N*N]
-  float2 *vacc;        // per sorted record: the degridded sum before its weight
   size_t bytes;
 };
 
@@ -345,11 +344,9 @@ int64_t scan_tmp_words(int64_t n);
 // k_rowgrid.cu
 cudaError_t grid_rows(wst_plan_s *p, int p0, int p1, float2 *out, bool fft);  // CNT_WORK zero before
 // adjoint rows.  dtab: the table gradient is added to it; else degridding, the sums added to
-// dvis in the caller's order or (dvis null) to W_.vacc in sorted order (unsort_sums hands
-// them over once every plane has been through)
+// dvis in the caller's order
 cudaError_t rows_adjoint(wst_plan_s *p, int p0, int p1, const float2 *planes, float2 *dvis, float *dtab);
 cudaError_t row_occupancy(wst_plan_s *p, int p0, int p1);  // W_.occ of planes [p0, p1); clears CNT_WORK
-cudaError_t unsort_sums(wst_plan_s *p, float2 *dvis);
 
 // k_fft.cu
 cudaError_t fft_rows(wst_plan_s *p, float2 *planes, int nplanes, int dir, bool presign,

@@ -82,3 +82,21 @@ def test_faint_cells_of_a_row_that_leaves_the_integer_range(wst, W):
     rows = np.flatnonzero(np.exp(-y * y / (2 * sigma * sigma)) >= 0.15)
     assert len(rows) >= 3
     assert_cells(wst, cfg, OracleConfig(n, fov, 1, -10.0, 10.0, W, "gauss", sigma), u, v, w, vis, adds=400, rows=rows)
+
+
+# ------------------------------------------------------------------------------------------
+# workspace
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("flags", [0, "fold"])
+@pytest.mark.parametrize("n", [256, 2048])
+def test_workspace_per_visibility(wst, n, flags):
+    """Below the planes' size only the sorted records (32 bytes) grow with the visibilities, at
+    any count: no second array of sums, least of all in a plan that cannot degrid."""
+    cfg = wst.Config(n=n, fov=0.1, n_w=2048 // n * 16, flags=wst.WST_FLAG_WFOLD if flags else 0)
+    plan = wst.Plan(cfg)
+    size = [wst.wst_plan_workspace_bytes(plan.handle, k) for k in (1000, 200_000, 600_000)]
+    planes = 8 * cfg.n_w * n * n
+    assert 32 * 600_000 <= planes  # the sort's keys fit the planes' place
+    assert size[1] - size[0] <= 32 * 199_000 + 256
+    assert size[2] - size[0] <= 32 * 599_000 + 256
