@@ -606,15 +606,31 @@ __device__ __forceinline__ void add_all(float *const (&at)[T], const float (&x)[
     if (at[t] && got[t] != old[t]) atomicAdd(at[t] + offset, x[t]);
 }
 
-// Rows are shared out as in k_grid_rows.  Degridding adds a record's row sum to the caller's
-// element, one 8-byte vector reduction.  (Sums kept in sorted order, where a warp's
-// reductions fall on whole sectors, and handed back by a pass of their own took as long, the
-// whole call 6.69 against 6.66 ms at 10M visibilities on 16 planes of 8192^2 and 17.2 against
-// 16.9 at 20M on 8 of 16384^2, and 8 bytes of workspace per visibility.)  With two scalar
-// reductions per record and row, the records of each bucket shared out on their own and
-// 16 warps per SM, the former took 5.64 ms, now 2.28 (32 warps).  Bound by the latency of a
-// row's load, transform and records in turn with two rows per SM; the taps stay evaluated one
-// by one (the recurrence of the forward gridder saves 0.13 ms here, but see below).
+// Rows are handed out to groups by the counter, when a group is free for one.  Degridding adds
+// a record's row sum to the caller's element, one 8-byte vector reduction.
+//
+// Order of the sums.  The W row sums of a visibility alternate in sign where the image's
+// edges dominate it (a strong grid correction), and cancel: added from the first tap row to
+// the last their partial sums stay as small as the sums themselves, in another order they
+// do not, and the result carries their rounding.  Rows are therefore claimed one by one, in
+// order and no earlier than they are worked on, and a row's records are walked from the
+// last bucket (its visibilities' first tap row) to the first: bucket by bucket up to 128
+// threads to a row (kByBucket), where the buckets' time keeps the rows of sparse images in
+// order too, in one even split from 256 on, where buckets are long enough for that.  With
+// two to eight rows to a batch, claimed ahead, and the records walked forward, an unpadded
+// Kaiser-Bessel table of 8 gave visibilities of a 2048^2 image 5.7e-5 off those in order, now
+// 8e-6, as two runs in order differ, and of an 8192^2 one 3.5e-5, now 1.9e-5 (in order 7e-6;
+// bucket by bucket 1.5e-5).  10M visibilities on 16 planes of 8192^2 took 6.62 ms then, now
+// 6.87 (bucket by bucket 7.41), 400,000 on 16 of 1024^2 191 us, now 186 (165 evenly split).
+//
+// Sums kept in sorted order, where a warp's reductions fall on whole sectors, and handed back
+// by a pass of their own took as long (the whole call 6.69 against 6.66 ms at 10M visibilities
+// on 16 planes of 8192^2, 17.2 against 16.9 at 20M on 8 of 16384^2) and 8 bytes of workspace
+// per visibility.  Bound by the latency of a row's load, transform and records in turn with
+// two rows per SM; the taps stay evaluated one by one (the recurrence of the forward gridder
+// saves 0.13 ms here, but see below).
+template <int TPR, bool KGRAD>
+constexpr bool kByBucket = !KGRAD && TPR <= 128;
 template <int N, int WT, bool KGRAD>
 __global__ void __launch_bounds__(GroupCfg<N, KGRAD ? 256 : 128>::THREADS,
                                   N >= 16384 || (KGRAD && N == 8192) ? 1 : KGRAD || N == 8192 ? 2 : N == 4096 ? 3
@@ -679,17 +695,8 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
         srow[idx] = x;
       }
     sync();
-    // the row's records are one contiguous range, split evenly over its threads (one head
-    // in flight); bnd[i] is where row j0 = q - d_lo + i starts
-    const uint32_t s_end = bnd[d_lo + 1];
-    uint32_t s = bnd[0] + jt;
-    RecHead nxt{};
-    if (s < s_end) nxt = rec_head(rec, s);
-    int i = 0;
-    for (; s < s_end; s += TPR) {
-      const RecHead rc = nxt;
-      if (s + TPR < s_end) nxt = rec_head(rec, s + TPR);
-      while (i < d_lo && bnd[i + 1] <= s) ++i;
+    // a record of bucket i (row j0 = q - d_lo + i), which bnd[i] .. bnd[i + 1] hold
+    auto take = [&](int i, uint32_t s, const RecHead &rc) {
       const float targ_y = (float)(d_lo - i) - kp.half + rec_gy(rc);
       const float gy = kernel_tap(kp, targ_y);
       const float gx0 = rec_gx(rc);
@@ -753,17 +760,30 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
         add_all<1>(at, lo, 0, false);
         add_all<1>(at, hi, 1, false);
       }
+    };
+    // from the last bucket to the first (the visibilities' first tap rows first): bucket by
+    // bucket, or all of the row's records split evenly over its threads, one head in flight
+    if constexpr (kByBucket<TPR, KGRAD>) {
+      for (int i = d_lo; i >= 0; --i)
+        for (uint32_t s = bnd[i] + jt; s < bnd[i + 1]; s += TPR) take(i, s, rec_head(rec, s));
+    } else {
+      const uint32_t last = bnd[d_lo + 1] - 1u, n_rec = bnd[d_lo + 1] - bnd[0];
+      RecHead nxt{};
+      if (jt < n_rec) nxt = rec_head(rec, last - jt);
+      int i = d_lo;
+      for (uint32_t k = jt; k < n_rec; k += TPR) {
+        const uint32_t s = last - k;
+        const RecHead rc = nxt;
+        if (k + TPR < n_rec) nxt = rec_head(rec, s - TPR);
+        while (bnd[i] > s) --i;  // the last row starting at or before the record
+        take(i, s, rc);
+      }
     }
     sync();  // the row buffer is reused by the next row
   };
-  const long long group0 = (long long)blockIdx.x * GROUPS + g, ngroups = (long long)gridDim.x * GROUPS;
-  long long next = group0 * (GR == 1 ? batch : GR);
   if constexpr (GR == 1) {
     while (true) {
-      if (gt == 0) {
-        s_item[g] = next;
-        next = ngroups * batch + (long long)atomicAdd(counter, (unsigned long long)batch);
-      }
+      if (gt == 0) s_item[g] = (long long)atomicAdd(counter, (unsigned long long)batch);
       sync();
       const long long base = s_item[g];
       if (base >= total) break;
@@ -779,9 +799,10 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
     }
   } else {
     while (true) {
-      const long long base = __shfl_sync(0xFFFFFFFFu, next, 0);  // a group is one warp here
+      long long base = 0;
+      if (gt == 0) base = (long long)atomicAdd(counter, (unsigned long long)GR);
+      base = __shfl_sync(0xFFFFFFFFu, base, 0);  // a group is one warp here
       if (base >= total) break;
-      if (gt == 0) next = ngroups * GR + (long long)atomicAdd(counter, (unsigned long long)GR);
       const long long item = base + rl % GR;
       const bool nonempty = item < total && !row_empty(item);
       if (__any_sync(0xFFFFFFFFu, nonempty)) do_row(item < total ? item : base, nonempty);
@@ -872,6 +893,7 @@ static cudaError_t launch_rows_adjoint(wst_plan_s *p, int p0, int np, const floa
   int grid = 0, batch = 0;
   cudaError_t e = persistent_grid<C>(p, kern, smem, (int64_t)np * N, grid, batch);
   if (e != cudaSuccess) return e;
+  if (!KGRAD) batch = 1;  // in order (k_rows_adjoint)
   unsigned long long *counter = p->W_.counters + CNT_WORK;  // cleared by row_occupancy
   kern<<<grid, C::THREADS, smem, p->stream>>>(planes, p->W_.records, p->W_.offsets, p0, np, kernel_params(p),
                                              dvis, dtab, counter, tw_half(p), batch);
