@@ -26,19 +26,19 @@ __device__ __forceinline__ ff ff_from_double(double d) {
 // Each product loses its half cycles before anything is summed: u l.hi + M is one fused
 // operation that rounds the exact product to a multiple of 1/2 (whose parity is the last bit
 // of the result), and the fused difference leaves the rest, |a| <= 1/4, rounded once (2^-27
-// cycle).  The low words' products and the three rests are summed and cis_small_cycles does
-// the remainder.  The kernel is bound by the FP32 multiply-add pipe: 39 operations a product
+// cycle).  The low words' products and the three rests are summed and cis_octant does the
+// remainder.  The kernel is bound by the FP32 multiply-add pipe: 39 operations a product
 // and pixel, 583 us for 2e5 visibilities at 2048 pixels; with rintf and the reductions inside
 // sincospi (cis_any), which go to a slower pipe, 827 us.
 constexpr float kCisMax = 0x1p+20f;
 __device__ __forceinline__ float2 cis_small(float u, float v, float w, const ff &l, const ff &m, const ff &t) {
-  constexpr float M = kHalfCycle;
+  constexpr float M = 6291456.0f;  // 1.5 2^22
   const float tu = __fmaf_rn(u, l.hi, M), tv = __fmaf_rn(v, m.hi, M), tw = __fmaf_rn(w, t.hi, M);
   const float a = __fmaf_rn(u, l.hi, -__fsub_rn(tu, M)), b = __fmaf_rn(v, m.hi, -__fsub_rn(tv, M));
   const float c = __fmaf_rn(w, t.hi, -__fsub_rn(tw, M));
   const float e = __fmaf_rn(w, t.lo, __fmaf_rn(v, m.lo, __fmul_rn(u, l.lo)));
-  return cis_small_cycles(__fadd_rn(__fadd_rn(a, b), __fadd_rn(c, e)),
-                          __float_as_uint(tu) ^ __float_as_uint(tv) ^ __float_as_uint(tw));
+  return cis_octant(__fadd_rn(__fadd_rn(a, b), __fadd_rn(c, e)),
+                    2u * (__float_as_uint(tu) + __float_as_uint(tv) + __float_as_uint(tw)));
 }
 
 // the same for any size: whole cycles by rint, product by product (p + e is the exact
