@@ -1,8 +1,8 @@
 // Direct transform core shared by k_dft (k_dft.cu) and k_dft_partials (wst_noalloc.cu):
 // the exact dirty image at a few pixels (the conjugate of Eq. 1 summed over the
-// visibilities), phases u l + v m + w (n-1) formed from float-float l, m, n-1 with the
-// cycles taken out product by product (cis_small, cis_any) before the FP32 sine and cosine,
-// so a phase of thousands of cycles keeps the accuracy of one below a cycle.
+// visibilities), phases u l + v m + w (n-1) formed in float-float (l, m, n-1 carried as
+// float-float) and reduced modulo one cycle before the FP32 sine and cosine (cis_small,
+// cis_any), so a phase of thousands of cycles keeps the accuracy of one below a cycle.
 #pragma once
 
 #include "wst_internal.cuh"
@@ -21,39 +21,39 @@ __device__ __forceinline__ ff ff_from_double(double d) {
   return {s.x, s.y};
 }
 
-// exp(2 pi i (u l + v m + w t)) for |u|, |v|, |w| <= kCisMax and |l|, |m|, |t| <= 1 (cis_small)
+// exp(2 pi i (u l + v m + w t)) for |u|, |v|, |w| <= kCisMax and |l|, |m|, |t| <= 1
 //
-// Each product loses its half cycles before anything is summed: u l.hi + M is one fused
-// operation that rounds the exact product to a multiple of 1/2 (whose parity is the last bit
-// of the result), and the fused difference leaves the rest, |a| <= 1/4, rounded once (2^-27
-// cycle).  The low words' products and the three rests are summed and cis_octant does the
-// remainder.  The kernel is bound by the FP32 multiply-add pipe: 39 operations a product
-// and pixel, 583 us for 2e5 visibilities at 2048 pixels; with rintf and the reductions inside
-// sincospi (cis_any), which go to a slower pipe, 827 us.
-constexpr float kCisMax = 0x1p+20f;
+// The phase as a float-float sum without its renormalisations: the products u l.hi with their
+// exact remainders (two_prod), summed exactly (two_sum); the remainders and the low words'
+// products go into one low word.  s + M, M = 1.5 2^22, rounds the high word (below 2^21 in
+// size) to a multiple of 1/2 whose last bit is its parity; what is left, at most 1/4, and
+// the low word are added with the phase's one rounding: 1.5e-8 cycle at most, 3.3e-9 rms (the
+// phase as a float-float reduced to half a cycle: 3.0e-8, 6.5e-9).  The kernel is bound by
+// instruction issue, most of it on the FP32 pipe: 2e5 visibilities at 2048 pixels and 25
+// sources 766 us.  With whole float-float operations and sincospi (cis_any), part of it on a
+// slower pipe, 1367 us; with each product rounded after its half cycles are taken out and
+// plain sums, phases 7e-8 cycle off, 640 us.
+constexpr float kCisMax = 0x1p+19f;
 __device__ __forceinline__ float2 cis_small(float u, float v, float w, const ff &l, const ff &m, const ff &t) {
-  constexpr float M = 6291456.0f;  // 1.5 2^22
-  const float tu = __fmaf_rn(u, l.hi, M), tv = __fmaf_rn(v, m.hi, M), tw = __fmaf_rn(w, t.hi, M);
-  const float a = __fmaf_rn(u, l.hi, -__fsub_rn(tu, M)), b = __fmaf_rn(v, m.hi, -__fsub_rn(tv, M));
-  const float c = __fmaf_rn(w, t.hi, -__fsub_rn(tw, M));
-  const float e = __fmaf_rn(w, t.lo, __fmaf_rn(v, m.lo, __fmul_rn(u, l.lo)));
-  return cis_octant(__fadd_rn(__fadd_rn(a, b), __fadd_rn(c, e)),
-                    2u * (__float_as_uint(tu) + __float_as_uint(tv) + __float_as_uint(tw)));
+  constexpr float M = 6291456.0f;
+  const float pu = __fmul_rn(u, l.hi), pv = __fmul_rn(v, m.hi), pw = __fmul_rn(w, t.hi);
+  const float eu = __fmaf_rn(u, l.lo, __fmaf_rn(u, l.hi, -pu));
+  const float ev = __fmaf_rn(v, m.lo, __fmaf_rn(v, m.hi, -pv));
+  const float ew = __fmaf_rn(w, t.lo, __fmaf_rn(w, t.hi, -pw));
+  const ff a = two_sum(pu, pv), b = two_sum(a.hi, pw);
+  const float e = __fadd_rn(__fadd_rn(eu, ev), __fadd_rn(ew, __fadd_rn(a.lo, b.lo)));
+  const float ts = __fadd_rn(b.hi, M);
+  return cis_octant(__fadd_rn(__fsub_rn(b.hi, __fsub_rn(ts, M)), e), 2u * __float_as_uint(ts));
 }
 
-// the same for any size: whole cycles by rint, product by product (p + e is the exact
-// product, p - rint(p) is exact), then sincospi
+// phi = u l + v m + w t with exact float products (two_prod) and float-float sums
+__device__ __forceinline__ ff phase_ff(float u, float v, float w, const ff &l, const ff &m, const ff &t) {
+  const ff a = ff_mul({u, 0.0f}, l), b = ff_mul({v, 0.0f}, m), c = ff_mul({w, 0.0f}, t);
+  return ff_add(ff_add(a, b), c);
+}
+// the same for any size
 static __device__ __noinline__ float2 cis_any(float u, float v, float w, ff l, ff m, ff t) {
-  const float pu = __fmul_rn(u, l.hi), pv = __fmul_rn(v, m.hi), pw = __fmul_rn(w, t.hi);
-  float e = __fmaf_rn(u, l.lo, __fmaf_rn(u, l.hi, -pu));
-  e = __fmaf_rn(v, m.lo, __fadd_rn(e, __fmaf_rn(v, m.hi, -pv)));
-  e = __fmaf_rn(w, t.lo, __fadd_rn(e, __fmaf_rn(w, t.hi, -pw)));
-  const float a = __fsub_rn(pu, rintf(pu)), b = __fsub_rn(pv, rintf(pv)), c = __fsub_rn(pw, rintf(pw));
-  const float s = __fadd_rn(__fadd_rn(a, b), c);
-  const float phi = __fadd_rn(__fsub_rn(s, rintf(s)), e);
-  float sn, cs;
-  sincospif(2.0f * phi, &sn, &cs);
-  return make_float2(cs, sn);
+  return cis_cycles_ff(phase_ff(u, v, w, l, m, t));
 }
 
 // The CTA's share of out_i = sum_j w_j V_j exp(2 pi i (u_j l_i + v_j m_i + w_j (n_i - 1)))

@@ -1,8 +1,8 @@
 // Direct transforms: the exact dirty image at chosen pixels (the conjugate of Eq. 1,
 // summed over visibilities) and Eq. 1 itself for a point-source sky.  Phases are
-// formed from float-float l, m, n - 1 and reduced modulo one cycle before the FP32 sine
-// and cosine (dft_core.cuh), so a phase of thousands of cycles keeps the accuracy of one
-// below a cycle.
+// formed in float-float (l, m, n - 1 carried as float-float) and reduced modulo one cycle
+// before the FP32 sine and cosine (dft_core.cuh), so a phase of thousands of cycles keeps
+// the accuracy of one below a cycle.
 #include "dft_core.cuh"
 
 namespace wst {

@@ -138,6 +138,50 @@ def test_sine_and_cosine(wst):
     assert np.abs(got.imag - np.sin(phase)).max() < 2.0 ** -24
 
 
+@pytest.mark.parametrize("scale", [100.0, 2.0 ** 14, 2.0 ** 17, 1.01 * 2.0 ** 19, 2.0 ** 20])
+@pytest.mark.parametrize("far", [False, True])
+def test_phases_in_float_float(wst, scale, far):
+    """The phase u l + v m + w (n - 1) in float-float, at and beyond the range that takes it
+    without renormalisations, and from a source outside the unit sphere (n - 1 counts as
+    zero there).  It is rounded to FP32 once, below or just above half a cycle: 2^-25 cycle;
+    l, m and n - 1 are pairs of floats, 2^-48 of a coordinate; the sine and cosine err by
+    2^-24 at most."""
+    rng = np.random.default_rng(int(scale) + far)
+    n_vis = 400_000
+    u, v, w = rng.uniform(-scale, scale, (3, n_vis)).astype(np.float32)
+    for _ in range(3):
+        l, m = rng.uniform(-0.6, 0.6, 2)
+        if far:
+            l += 1.5
+        r2 = l * l + m * m
+        t = -r2 / (1.0 + np.sqrt(1.0 - r2)) if r2 < 1.0 else 0.0
+        got = torch.empty(n_vis, dtype=torch.complex64, device="cuda")
+        wst.wst_predict_points(dev(u), dev(v), dev(w), dev(np.array([l])), dev(np.array([m])), dev(np.ones(1)), got)
+        phase = u.astype(np.longdouble) * l + v.astype(np.longdouble) * m + w.astype(np.longdouble) * t
+        phase = (phase - np.rint(phase)).astype(np.float64) * (-2.0 * np.pi)
+        err = got.cpu().numpy() - np.exp(1j * phase)
+        tol = 2.0 * np.pi * (2.0 ** -25 + 3.0 * scale * 2.0 ** -48) + 2.0 ** -24
+        assert max(np.abs(err.real).max(), np.abs(err.imag).max()) <= tol
+
+
+def test_direct_transform_phases(wst):
+    """The same for wst_dft at single visibilities: one visibility, every pixel its phase."""
+    n, fov, n_pix = 4096, 0.9, 4096
+    rng = np.random.default_rng(5)
+    pa, pb = rng.integers(0, n, (2, n_pix)).astype(np.int32)
+    l, m = (pa - n // 2) * (fov / n), (pb - n // 2) * (fov / n)
+    t = -(l * l + m * m) / (1.0 + np.sqrt(1.0 - l * l - m * m))
+    for scale in [3e3, 1e5]:
+        u, v, w = rng.uniform(-scale, scale, (3, 1)).astype(np.float32)
+        out = torch.empty(n_pix, dtype=torch.complex64, device="cuda")
+        wst.wst_dft(dev(u), dev(v), dev(w), dev(np.ones(1, np.complex64)), n, fov, dev(pa), dev(pb), out)
+        phase = u.astype(np.longdouble) * l + v.astype(np.longdouble) * m + w.astype(np.longdouble) * t
+        phase = (phase - np.rint(phase)).astype(np.float64) * (2.0 * np.pi)
+        err = out.cpu().numpy() - np.exp(1j * phase)
+        tol = 2.0 * np.pi * (2.0 ** -25 + 3.0 * scale * 2.0 ** -48) + 2.0 ** -24
+        assert max(np.abs(err.real).max(), np.abs(err.imag).max()) <= tol
+
+
 # ------------------------------------------------------------------------------------------
 # workspace
 # ------------------------------------------------------------------------------------------
