@@ -70,15 +70,20 @@ __global__ void k_l2(float2 *l2ff, double *l2d, int n, double dl) {
 // weights c_j = w_{P+j} G(j h/2) + w_{P-j} G(-j h/2) (FP64, h/6 and the Simpson factors in
 // them), and k_correction sums c_j cos(2 pi nu j h/2) for each nu >= 0; -nu has the same.
 //
-// Bound: the FP64 pipe (2 FMA per clock and SM).  Each thread takes every 128th node and
-// advances its cosine by the Chebyshev recurrence, one multiply-add per node beside the sum's
-// (its error grows with the square of the steps: 512 of them, for the longest table, leave
-// 3e-11 of Ghat(0), far below the FP32 result).  By rotations, 4 multiply-adds per node, the
-// 8193-sample table at n = 512 took 29 us, now 15; with a block per nu, the kernel evaluated
-// and three cospi taken in every panel, 1106 us, on every wst_plan_set_kernel_table, that is
-// on every training step.
+// Bound: the FP64 pipe (2 FMA per clock and SM).  Thread t takes the nodes j = t + 128 m.  With
+// d the half turns per node, cos(d j) = cos(d t) cos(128 d m) - sin(d t) sin(128 d m): the
+// block's 128 d m are evaluated once, into shared memory, and a thread sums two products per
+// node, every cosine as exact as if evaluated by itself.  (The absolute error matters: Ghat
+// falls to 1e-6 of Ghat(0) and less at the field's edge.  A recurrence from node to node
+// costs as many multiply-adds; its error grows with the square of the steps, 512 for the longest
+// table: at 4e-11 of Ghat(0) 2e-6 of the value, now 8e-8.)  8193 samples at n = 512 take 17 us; by
+// rotations, 4 multiply-adds per node, 29; with a block per nu, the kernel evaluated and
+// three cospi taken in every panel, 1106, on every wst_plan_set_kernel_table, that is on every
+// training step.
 constexpr int kNodePanels = 256;   // panels per cell, analytic kernels
 constexpr int kCorrThreads = 128;
+constexpr int kMaxTurns = 512;     // kCorrThreads kMaxTurns > P: tables of 65536 samples, W = 16
+static_assert(kCorrThreads * kMaxTurns >= 65536 && kMaxSupport * kNodePanels < 65536, "every node has a turn");
 
 static int node_panels(const wst_plan_s *p) {
   return p->cfg.kernel == WST_KERNEL_TABLE ? p->cfg.ktable_len - 1 : kNodePanels * p->W;
@@ -123,18 +128,26 @@ __global__ void __launch_bounds__(kCorrThreads) k_correction(float *corr, int n,
     if (threadIdx.x == 0) *tab_max = __uint_as_float(s_max);
     return;
   }
-  const double turn = (double)k * (double)W / ((double)n * (double)P);  // 2 nu h/2: half turns per node
-  // c_{m+1} = 2 cos(d) c_m - c_{m-1} from node to node of this thread
-  double acc = 0.0, c = cospi(turn * (double)threadIdx.x), before = cospi(turn * ((double)threadIdx.x - kCorrThreads));
-  const double twice = 2.0 * cospi(turn * (double)kCorrThreads);
-  for (int j = threadIdx.x; j <= P; j += kCorrThreads) {
-    acc = fma(__ldg(nodes + j), c, acc);
-    const double next = fma(twice, c, -before);
-    before = c;
-    c = next;
+  // 2 nu j h/2 in half turns: the numerator is below 2^53, so rounded once
+  auto turn = [&](int j) { return (double)((long long)k * W * j) / ((double)n * (double)P); };
+  __shared__ double2 s_turn[kMaxTurns];  // cos, sin of 128 d m
+  for (int m = threadIdx.x; m <= P / kCorrThreads; m += kCorrThreads) {
+    double s, c;
+    sincospi(turn(m * kCorrThreads), &s, &c);
+    s_turn[m] = make_double2(c, s);
   }
+  __syncthreads();
+  double ac = 0.0, as = 0.0;
+  for (int j = threadIdx.x, m = 0; j <= P; j += kCorrThreads, ++m) {
+    const double x = __ldg(nodes + j);
+    const double2 t = s_turn[m];
+    ac = fma(x, t.x, ac);
+    as = fma(x, t.y, as);
+  }
+  double s, c;
+  sincospi(turn(threadIdx.x), &s, &c);
   __shared__ double red[kCorrThreads];
-  red[threadIdx.x] = acc;
+  red[threadIdx.x] = ac * c - as * s;
   __syncthreads();
   for (int st = kCorrThreads / 2; st > 0; st >>= 1) {
     if (threadIdx.x < st) red[threadIdx.x] += red[threadIdx.x + st];

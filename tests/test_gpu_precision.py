@@ -183,6 +183,44 @@ def test_direct_transform_phases(wst):
 
 
 # ------------------------------------------------------------------------------------------
+# grid correction
+# ------------------------------------------------------------------------------------------
+
+@pytest.mark.parametrize("W,per_cell", [(16, 4095), (16, 2048), (8, 1024), (10, 128)])
+def test_correction_where_the_transform_is_small(wst, W, per_cell):
+    """1/Ghat of unpadded Kaiser-Bessel tables, whose transform falls to 1e-6 ... 1e-10 of
+    Ghat(0) at the field's edge.  wst_correct of a unit image gives corr_a corr_b: three FP32
+    roundings along the central row.  Beside them Ghat may err by the roundings of an FP64 sum:
+    each is 2^-53 of a partial sum, and over a thousand terms and more they average out to
+    an eighth of 2^-53 of the terms' magnitudes or less."""
+    from paper_2301_06061_gb300 import kernels
+
+    n, length = 64, W * per_cell + 1
+    tab = kernels.kaiser_bessel_table(W, kernels.kaiser_bessel_beta(W), per_cell)
+    assert len(tab) == length
+    t = tab.astype(np.float64)
+    x = np.linspace(-0.5 * W, 0.5 * W, 2 * length - 1)
+    g = np.empty(2 * length - 1)
+    g[::2], g[1::2] = t, 0.5 * (t[1:] + t[:-1])
+    wt = np.full(g.size, 2.0)
+    wt[1::2] = 4.0
+    wt[0] = wt[-1] = 1.0
+    c = wt * g * (1.0 / per_cell / 6.0)
+    at = np.array([0, 1, 2, 3, 4, 8, 16, 31, 32])
+    pi = np.longdouble("3.14159265358979323846264338327950288")
+    want = np.array([np.sum(np.cos(2 * pi * (a - n // 2) / n * x.astype(np.longdouble)) * c) for a in at])
+    want = want.astype(np.float64)
+    plan = wst.Plan(wst.Config(n=n, fov=0.1, n_w=1, support=W, kernel=wst.WST_KERNEL_TABLE, ktable_len=length))
+    plan.set_kernel_table(dev(tab))
+    img = torch.ones((1, n, n), dtype=torch.complex64, device="cuda")
+    wst.wst_plan_stream(plan.handle)
+    wst.wst_correct(plan.handle, img)
+    prod = img[0, n // 2, at].real.double().cpu().numpy()
+    got = 1.0 / (prod * want[-1])
+    assert np.all(np.abs(got - want) <= 3 * 2.0 ** -24 * np.abs(want) * 1.01 + 2.0 ** -56 * np.abs(c).sum())
+
+
+# ------------------------------------------------------------------------------------------
 # workspace
 # ------------------------------------------------------------------------------------------
 
