@@ -354,6 +354,7 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   const float bound = mmax * (gmax * gmax);
   // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row
   const float n_eff = mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
+  // (a NaN in a kernel table makes the bound NaN and takes float sums, which show it)
   const bool fixed = kFixedRows<N> && nonempty && cnt < (1u << 30) && bound >= 0x1p-90f && bound <= 0x1p+100f &&
                      n_eff <= (float)kFixedBinCap;
   // a bin of fewer than ~64 mean contributions may hold a single tap above B/8: such rows

@@ -118,12 +118,13 @@ __global__ void __launch_bounds__(kCorrThreads) k_correction(float *corr, int n,
                                                              float *__restrict__ tab_max) {
   const int k = blockIdx.x;  // nu = k / n, 0 <= k <= n/2
   if (k > n / 2) {  // a table's last block: its largest |sample|, for the gridder's bound
+    // (as integers, in which a NaN is the largest: the rows then take float sums and show it)
     __shared__ uint32_t s_max;
     if (threadIdx.x == 0) s_max = 0u;
     __syncthreads();
-    float m = 0.0f;
-    for (int i = threadIdx.x; i <= P; i += kCorrThreads) m = fmaxf(m, fabsf(__ldg(tab + i)));
-    atomicMax(&s_max, __float_as_uint(m));
+    uint32_t m = 0u;
+    for (int i = threadIdx.x; i <= P; i += kCorrThreads) m = max(m, __float_as_uint(fabsf(__ldg(tab + i))));
+    atomicMax(&s_max, m);
     __syncthreads();
     if (threadIdx.x == 0) *tab_max = __uint_as_float(s_max);
     return;

@@ -78,7 +78,7 @@ struct KernelParams {
   float table_scale;   // (L-1)/W
   const float *tap_table;   // TABLE, W = 7 or 8, L - 1 = W per_cell: rows i of T[a pc + i], a < kTapRow, i <= pc
   int per_cell;
-  const float *table_max;   // TABLE: the largest |sample|
+  const float *table_max;   // TABLE: the largest |sample|, NaN if one is
 };
 
 struct Workspace {

@@ -64,6 +64,27 @@ def test_cells_far_below_a_bright_one(wst, n, W):
     assert_cells(wst, cfg, ocfg, u, v, w, vis, adds=301 if n == 64 else 64)
 
 
+@pytest.mark.parametrize("n", [64, 256, 2048, 8192])
+@pytest.mark.parametrize("W", [6, 8])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_non_finite_kernel_samples_show(wst, n, W, bad):
+    """A kernel table that has diverged shows in the gridded planes and the uncorrected image:
+    integer sums must not swallow it."""
+    per_cell = 4
+    rng = np.random.default_rng(n + W)
+    u, v, w = synth.disk_uvw(500, 0.3 * n / 0.1, 5.0, rng)
+    tab = np.ones(W * per_cell + 1, np.float32)
+    tab[W * per_cell // 2 - 1] = bad
+    plan = wst.Plan(wst.Config(n=n, fov=0.1, n_w=1, w_min=-10.0, w_max=10.0, support=W, kernel=wst.WST_KERNEL_TABLE,
+                               ktable_len=tab.size))
+    plan.set_kernel_table(dev(tab))
+    plan.set_vis(dev(u), dev(v), dev(w), dev(synth.random_visibilities(500, rng)))
+    g = torch.empty((1, n, n), dtype=torch.complex64, device="cuda")
+    wst.wst_grid(plan.handle, 0, 1, g)
+    assert not torch.isfinite(torch.view_as_real(g)).all()
+    assert not torch.isfinite(torch.view_as_real(plan.image(flags=wst.WST_NO_CORRECTION))).all()
+
+
 @pytest.mark.parametrize("W", [7, 8])
 def test_faint_cells_of_a_row_that_leaves_the_integer_range(wst, W):
     """Rows of 8192 whose coherent pile-up of 400 equal values on one cell wraps the integer
