@@ -646,9 +646,9 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
   constexpr int R0 = stage_radix(N, EPT, 0);
   constexpr int RL = stage_radix(N, EPT, NST - 1);
   extern __shared__ __align__(16) float2 sm_rows[];
+  // (the table gradient keeps nothing else in static shared memory: its partial table takes
+  // what the rows leave, 6972 samples at 16384)
   __shared__ long long s_item[GROUPS];
-  __shared__ int s_list[GROUPS][kRowBatch], s_cnt[GROUPS];
-  __shared__ uint32_t s_bnd[C::ROWS][kMaxSupport + 2];
   float2 *twt = sm_rows + C::ROWS * C::PADL;  // twiddle tables (visible after the first barrier)
   fill_line_tables<N, C::EPT, TPR>(twt, tw);
   float *ptab = reinterpret_cast<float *>(twt + line_table_size<N, C::EPT, C::TPR>());  // KGRAD partial table
@@ -656,7 +656,6 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
   const int rl = threadIdx.x / TPR, jt = threadIdx.x % TPR;
   const GroupSync<GT, GROUPS> sync{g};
   float2 *srow = sm_rows + rl * C::PADL;
-  uint32_t *bnd = s_bnd[rl];
   auto smi = [](int i) { return i + i / EPT; };
   const long long total = (long long)np * N;
   const int W = WT > 0 ? WT : kp.support;
@@ -680,7 +679,14 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
 #pragma unroll
       for (int r = 0; r < R0; ++r)
         v[b * R0 + r] = nonempty ? __ldcs(grow + in_index<N, EPT, TPR, 0>(jt, b, r)) : make_float2(0.0f, 0.0f);
-    for (int i = jt; i <= d_lo + 1; i += TPR) bnd[i] = nonempty ? off[(b0 + q - d_lo + i) * kColBlocks] : 0u;
+    // where the rows j0 = q - d_lo ... q start, and the end (nothing if the row is empty)
+    static_assert(kColBlocks == 1, "a row's offsets are neighbours");
+    const uint32_t *bnd = off + (b0 + q - d_lo);
+    if constexpr (!KGRAD) {  // from shared memory: one latency for all of them, under the transform
+      __shared__ uint32_t s_bnd[C::ROWS][kMaxSupport + 2];
+      for (int i = jt; i <= d_lo + 1; i += TPR) s_bnd[rl][i] = nonempty ? bnd[i] : 0u;
+      bnd = s_bnd[rl];
+    }
     const TableTw<N, EPT, TPR, -1> twp{twt, jt};
     stage_compute_f<N, EPT, TPR, 0, -1>(v, jt, twp);
     middle_stages_f<N, EPT, TPR, 1, -1>(v, jt, srow, smi, twp, sync);
@@ -768,7 +774,7 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
       for (int i = d_lo; i >= 0; --i)
         for (uint32_t s = bnd[i] + jt; s < bnd[i + 1]; s += TPR) take(i, s, rec_head(rec, s));
     } else {
-      const uint32_t last = bnd[d_lo + 1] - 1u, n_rec = bnd[d_lo + 1] - bnd[0];
+      const uint32_t last = bnd[d_lo + 1] - 1u, n_rec = nonempty ? bnd[d_lo + 1] - bnd[0] : 0u;
       RecHead nxt{};
       if (jt < n_rec) nxt = rec_head(rec, last - jt);
       int i = d_lo;
@@ -788,15 +794,9 @@ k_rows_adjoint(const float2 *__restrict__ planes, const Record *__restrict__ rec
       sync();
       const long long base = s_item[g];
       if (base >= total) break;
-      if (gt < 32) {  // the rows of the batch that somebody reads
-        const bool listed = gt < batch && base + gt < total && !row_empty(base + gt);
-        const unsigned m = __ballot_sync(0xFFFFFFFFu, listed);
-        if (listed) s_list[g][__popc(m & ((1u << gt) - 1u))] = gt;
-        if (gt == 0) s_cnt[g] = __popc(m);
-      }
-      sync();
-      const int cnt = s_cnt[g];
-      for (int k = 0; k < cnt; ++k) do_row(base + s_list[g][k], true);
+      sync();  // s_item is read before it is written again
+      for (long long item = base; item < base + batch && item < total; ++item)
+        if (!row_empty(item)) do_row(item, true);  // (others nobody reads)
     }
   } else {
     while (true) {

@@ -257,3 +257,21 @@ def test_workspace_per_visibility(wst, n, flags):
     assert 32 * 600_000 <= planes  # the sort's keys fit the planes' place
     assert size[1] - size[0] <= 32 * 199_000 + 256
     assert size[2] - size[0] <= 32 * 599_000 + 256
+
+
+def test_table_gradient_takes_what_a_row_leaves(wst):
+    """At 16384 a table of 6972 samples fits the row kernel's shared memory beside the row and
+    its twiddles.  A flat table and one visibility at the phase centre, of value one: tap
+    (a, d) contributes Re(conj(gh) V) = 1 (the image is one pixel at the centre, its transform
+    one everywhere) to both its profiles, W of them each; every tap's share goes to the two
+    samples around it, so W^2 lands on the x profile and W^2 on the y profile."""
+    n, W, length = 16384, 7, 6972
+    plan = wst.Plan(wst.Config(n=n, fov=0.1, n_w=1, w_min=-10.0, w_max=10.0, support=W, kernel=wst.WST_KERNEL_TABLE,
+                               ktable_len=length))
+    plan.set_kernel_table(torch.ones(length, device="cuda"))
+    zero = torch.zeros(1, device="cuda")
+    plan.set_vis(zero, zero, zero, torch.ones(1, dtype=torch.complex64, device="cuda"))
+    y = torch.zeros((1, n, n), dtype=torch.complex64, device="cuda")
+    y[0, n // 2, n // 2] = 1.0
+    grad = plan.kernel_grad(y)
+    assert abs(float(grad.double().sum()) - 2 * W * W) < 1e-4
