@@ -230,7 +230,8 @@ wst_status wst_grid(wst_plan plan, int32_t plane_begin, int32_t plane_end, void 
  * Eq. 2 for planes [plane_begin, plane_end): transform each plane of grid_inout
  * (layout of wst_grid; overwritten) with the centred positive-exponent 2D FFT,
  * multiply by the plane's phase screen and ADD the central N x N into image_inout,
- * complex64 [batch x N x N].  No grid correction (see wst_correct).
+ * complex64 [batch x N x N].  No grid correction (see wst_correct).  grid_inout must
+ * start on a 16-byte boundary, else INVALID_ARG.
  */
 wst_status wst_fft_correct(wst_plan plan, int32_t plane_begin, int32_t plane_end, void *grid_inout,
                            void *image_inout);

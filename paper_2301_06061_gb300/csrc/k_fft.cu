@@ -1330,10 +1330,10 @@ static EncodeTiledFn tensor_map_encoder() {
 
 // Tensor map of nplanes complex64 n x n planes seen as FP32 [nplanes][n][2n], with a box of
 // one tile: kCB complex columns (128 bytes) x `rows` rows x 1 plane.  False if the encoder
-// is unavailable or the buffer is not 16-byte aligned (the copies need both).
+// is unavailable (k_cols_b16 takes the pass then).
 static bool plane_tile_map(CUtensorMap *m, const float2 *planes, int n, int nplanes, int rows) {
   const EncodeTiledFn enc = tensor_map_encoder();
-  if (!enc || ((uintptr_t)planes & 15u) || nplanes < 1) return false;
+  if (!enc || nplanes < 1) return false;
   const cuuint64_t dims[3] = {2ull * (cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)nplanes};
   const cuuint64_t strides[2] = {8ull * (cuuint64_t)n, 8ull * (cuuint64_t)n * (cuuint64_t)n};
   const cuuint32_t box[3] = {2u * kCB, (cuuint32_t)rows, 1u};

@@ -420,6 +420,8 @@ wst_status wst_fft_correct(wst_plan p, int32_t b, int32_t e, void *grid_inout, v
   if (b < 0 || e > p->n_planes || b > e) return fail(p, WST_ERR_INVALID_ARG, "plane range");
   if (e == b) return WST_OK;
   if (!grid_inout || !image_inout) return fail(p, WST_ERR_INVALID_ARG, "NULL buffer");
+  // every column pass copies 16 bytes at a time (cp.async, TMA)
+  if ((uintptr_t)grid_inout % 16) return fail(p, WST_ERR_INVALID_ARG, "planes not 16-byte aligned");
   float2 *g = (float2 *)grid_inout;
   WST_CUDA(p, fft_rows(p, g, e - b, +1, true, false), "rows");
   WST_CUDA(p, fft_cols_a(p, g, e - b, +1, false, nullptr), "cols A");
