@@ -40,6 +40,63 @@ def configs(wst, n, fov, n_w, W=7, **kw):
             OracleConfig(n, fov, n_w, -160.0, 160.0, W, "gauss", sigma))
 
 
+@pytest.mark.parametrize("n", [64, 256, 2048])
+@pytest.mark.parametrize("n_w,chunk", [(16, 0), (17, 0), (33, 0), (40, 0), (40, 20), (33, 7)])
+def test_adjoint_over_many_planes(wst, n, n_w, chunk):
+    """Degridding of one image where its planes make several runs of 16 (the screens' anchors
+    are renewed, and runs go to blocks of their own where the tiles are few), whole and in
+    chunks that cut runs."""
+    fov = 0.1
+    u, v, w, vis, rng = case(n, fov, 3000, [n, n_w, chunk])
+    cfg, ocfg = configs(wst, n, fov, n_w, planes_per_chunk=chunk)
+    plan = wst.Plan(cfg)
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis))
+    y = (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))).astype(np.complex64)
+    got = plan.degrid(dev(y[None]), flags=wst.WST_NO_CORRECTION).cpu().numpy()
+    want = oracle.degrid(ocfg, u, v, w, vis, y, correct=False)
+    assert np.abs(got - want).max() <= TOL * np.abs(want).max()
+
+
+@pytest.mark.parametrize("chunk", [0, 20])
+def test_adjoint_of_several_images_over_many_planes(wst, chunk):
+    n, fov, n_w, batch, per = 256, 0.1, 18, 3, 1500
+    u, v, w, vis, rng = case(n, fov, batch * per, chunk)
+    cfg, ocfg = configs(wst, n, fov, n_w, batch=batch, planes_per_chunk=chunk)
+    plan = wst.Plan(cfg)
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis), None, [per * i for i in range(batch + 1)])
+    y = (rng.standard_normal((batch, n, n)) + 1j * rng.standard_normal((batch, n, n))).astype(np.complex64)
+    got = plan.degrid(dev(y), flags=wst.WST_NO_CORRECTION).cpu().numpy()
+    for i in range(batch):
+        s = slice(per * i, per * (i + 1))
+        want = oracle.degrid(ocfg, u[s], v[s], w[s], vis[s], y[i], correct=False)
+        assert np.abs(got[s] - want).max() <= TOL * np.abs(want).max()
+
+
+@pytest.mark.parametrize("n,W,per_cell", [(512, 8, 511), (512, 8, 512), (512, 8, 1024), (256, 6, 512), (1024, 6, 1024),
+                                          (512, 13, 512)])
+def test_table_gradient_of_finely_sampled_tables(wst, n, W, per_cell):
+    """From 512 samples per cell the first attempts of a record's additions go out together:
+    half of the visibilities fall on a few positions, so that many lose the race and are added
+    the usual way; supports with an instance of their own and taps in fours with a rest."""
+    fov, n_w, n_vis = 0.1, 2, 4000
+    u, v, w, vis, rng = case(n, fov, n_vis, [n, W, per_cell])
+    h = n_vis // 2
+    u[:h] = (rng.integers(0, 2, h) + 0.25).astype(np.float32) / np.float32(fov)
+    v[:h] = np.float32(1.25 / fov)
+    w[:h] = 10.0
+    xs = np.linspace(-W / 2, W / 2, W * per_cell + 1)
+    tab = (np.exp(-xs**2 / 1.7) * (1 + 0.05 * np.sin(xs))).astype(np.float32)
+    plan = wst.Plan(wst.Config(n=n, fov=fov, n_w=n_w, w_min=-160.0, w_max=160.0, support=W, kernel=wst.WST_KERNEL_TABLE,
+                               ktable_len=tab.size))
+    plan.set_kernel_table(dev(tab))
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis))
+    ocfg = OracleConfig(n, fov, n_w, -160.0, 160.0, W, "table", 0.0, tab.astype(np.float64))
+    y = (rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))).astype(np.complex64)
+    got = plan.kernel_grad(dev(y[None])).cpu().numpy()
+    ref = oracle.kernel_grad(ocfg, u, v, w, vis, y)
+    assert np.abs(got - ref).max() <= 1e-4 * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("n", [64, 512, 1024, 4096, 16384])
 def test_planes_between_alignments_are_refused(wst, n):
     """wst_fft_correct's passes copy 16 bytes at a time: planes that start 8 bytes past such a
@@ -55,3 +112,39 @@ def test_planes_between_alignments_are_refused(wst, n):
     assert not torch.view_as_real(img).any()
     wst.wst_fft_correct(plan.handle, 0, 1, raw[:n * n].view(1, n, n), img)
     assert not torch.view_as_real(img).any()
+
+
+@pytest.mark.parametrize("n,batch,chunk", [(64, 7, 0), (512, 5, 4), (2048, 3, 4)])
+def test_fp64_screens_of_several_images(wst, n, batch, chunk):
+    fov, n_w, per = 0.1, 2, 1500
+    u, v, w, vis, _ = case(n, fov, batch * per, [n, batch])
+    cfg, ocfg = configs(wst, n, fov, n_w, batch=batch, planes_per_chunk=chunk, flags=wst.WST_FLAG_FP64_SCREEN)
+    plan = wst.Plan(cfg)
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis), None, [per * i for i in range(batch + 1)])
+    img = plan.image(flags=wst.WST_NO_CORRECTION).cpu().numpy()
+    for i in range(batch):
+        s = slice(per * i, per * (i + 1))
+        ref = oracle.image(ocfg, u[s], v[s], w[s], vis[s], None, correct=False)
+        assert np.abs(img[i] - ref).max() <= TOL * np.abs(ref).max()
+
+
+def test_sort_clear_beyond_one_kernel(wst):
+    """More than 4 MB of bucket counts are cleared by a memset (16385 planes' worth of 64 rows
+    and up); bound twice, so that a count left over would show."""
+    n, fov, n_w, batch = 64, 0.1, 4096, 5
+    per = 4000
+    u, v, w, vis, rng = case(n, fov, batch * per, 3)
+    cfg, _ = configs(wst, n, fov, n_w, batch=batch, planes_per_chunk=64)
+    plan = wst.Plan(cfg)
+    off = [per * i for i in range(batch + 1)]
+    for _ in range(2):
+        w = rng.uniform(-150, 150, batch * per).astype(np.float32)
+        plan.set_vis(dev(u), dev(v), dev(w), dev(vis), None, off)
+        k = torch.empty(batch * per, dtype=torch.int32, device="cuda")
+        i0, j0 = torch.empty_like(k), torch.empty_like(k)
+        wst.wst_vis_cells(plan.handle, k, i0, j0)
+        ko, io, jo, st = oracle.locate(OracleConfig(n, fov, n_w, -160.0, 160.0, 7, "gauss", 0.875), u, v, w, vis)
+        np.testing.assert_array_equal(k.cpu().numpy(), ko)
+        np.testing.assert_array_equal(i0.cpu().numpy(), io)
+        np.testing.assert_array_equal(j0.cpu().numpy(), jo)
+        assert plan.stats()["n_kept"] == int((st == 0).sum())
