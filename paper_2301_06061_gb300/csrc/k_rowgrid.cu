@@ -40,12 +40,29 @@
 // per visibility-row (the bins count a visibility-row once per bin it reaches,
 // 1 + (W - 1)/64 bins on average) go straight to float atomics.  On the benchmark
 // workload the image error against the FP64 oracle equals that of all-float
-// accumulation.  Rows shorter than 8192 keep float sums.  Integer ones took 1.30 instead of
-// 1.74 ms at 4096^2 x 32 planes (4.08M visibilities), but one quantum for the whole row takes
-// bits from every cell far below its busiest bin (the caller of wst_grid sees them), and a
-// grid correction of 1e5 or more shows the other rounding in the image: at the sizes of
-// those rows it repeats from call to call, and a 512^2 image of 6,300 visibilities with an
-// unpadded Kaiser-Bessel table of 8 came out 50% different.
+// accumulation.
+//
+// Rows shorter than 8192.  One quantum for a whole row takes bits from every cell far below
+// its busiest bin, and rounds otherwise than float sums do.  Neither may show:
+//   - wst_grid hands the cells to the caller: its rows are summed in float.
+//   - In an image a cell's rounding is one term of the row's transform, which rounds by about
+//     2^-25 of the row's root sum of squares, R.  The integers' roundings add up to
+//     0.76 sqrt(visibilities) delta over the row.  With m the mean magnitude, R is about
+//     1.2 m sqrt(visibilities) or more, and the steps of unit_of keep the sum below the
+//     transform's rounding up to 800 contributions in the busiest bin; beyond, float sums
+//     round as much themselves (their partial sums grow with the count).  A row that one
+//     value dominates (R near B) leaves the range with the finest quantum and is taken
+//     again with B / 2^32, half the transform's rounding at 8192 visibilities, but no
+//     coarser: then float.
+//   - A strong grid correction amplifies either rounding alike at the image's edge, by
+//     (Ghat(0) / Ghat(1/2))^2, and with it the difference between the two: 2e-5 of an image
+//     at 1e4.  Plans above that (kFixedMaxRatio, Gaussians of 9 and 10 and unpadded
+//     Kaiser-Bessel tables among them) and tables, whose transform only the device knows, take
+//     float sums, and so do rows below 1024, whose float sums repeat from call to call (an
+//     unpadded Kaiser-Bessel table of 8 came out 50% different at 512^2).
+// What it saves (float sums are compare-and-swap loops): 4096^2 x 32 planes, 4.08M
+// visibilities, 1.28 instead of 1.69 ms in this kernel, 64 images of 2048^2 x 16, 37.7M, 7.7
+// instead of 12.2, 9 of 1024^2 x 5, 5.9M, 0.96 instead of 3.4.
 #include "fft_core.cuh"
 
 namespace wst {
@@ -73,8 +90,19 @@ struct GroupCfg {
 // 1277 us on 32 planes of 4096^2 with 4.08M visibilities, 986 instead of 882 us on 21 planes
 // with the ES kernel).  Two rows of 8192 in a CTA leave 64 registers a thread: 5.90 instead of
 // 5.03 ms on 16 planes with 20M visibilities.
+// The configuration of float sums that dense rows bound (shared compare-and-swap loops): CTAs
+// of 256 threads on 256 / TPR rows in step, records read directly.  With the groups above,
+// which let a few dense rows finish last, wst_grid took 545 instead of 364 us at 2048^2 x 12
+// (1.33M visibilities, ES of 8), images 7.6 instead of 6.0 ms (24 of 1024^2 x 22, 12.9M, support
+// 6 in float); for supports 7 and 8, whose records are prefetched, the groups are faster (12.2
+// against 16.3 ms on 64 images of 2048^2 x 16), and below 512 they are even.
 template <int N>
-using GridCfg = GroupCfg<N, N == 4096 ? 1024 : 128>;
+struct StepCfg {
+  static constexpr int EPT = RowCfg<N>::EPT, TPR = RowCfg<N>::TPR, PADL = RowCfg<N>::PADL;
+  static constexpr int THREADS = RowCfg<N>::THREADS, GT = THREADS, GR = GT / TPR, GROUPS = 1, ROWS = GR;
+};
+template <int N, bool STEP = false>
+using GridCfg = std::conditional_t<STEP, StepCfg<N>, GroupCfg<N, N == 4096 ? 1024 : 128>>;
 // whether a group writes a row out during its next row's gridding: where it is alone
 template <int N>
 constexpr bool kPending = N >= 8192;
@@ -187,8 +215,16 @@ __device__ __forceinline__ void for_taps(const KernelParams &kp, const float *ta
 }
 
 constexpr int kFixedBinCap = 8192;
-template <int N>
-constexpr bool kFixedRows = N >= kFixedMinN;
+template <int N, bool FFT>
+constexpr bool kFixedRows = N >= kFixedMinN || (FFT && N >= kFixedImagingMinN);
+
+// delta / B of a row shorter than 8192, n_eff the mean contributions in its busiest bin.
+// Sparse bins hold sums of a few taps: up to 64 the quantum stays near 2^-27 of the mean
+// magnitude, and a cell may hold, before the row is accumulated again, the whole bin below
+// 16 and half of it below 64.  From 64 on it is B / 2^34, a cell up to an eighth of the bin.
+__device__ __forceinline__ float unit_of(float n_eff) {
+  return n_eff < 16.0f ? 0x1p-30f : n_eff < 64.0f ? 0x1p-32f : 0x1p-34f;
+}
 
 // one tap into the planar row: float atomics, or (FIXED) the tap already in units of the
 // row's quantum (the record's value was scaled by 1/delta once), converted and added as
@@ -280,13 +316,30 @@ struct NoPending {
 // With FIXED, qscale = 1/delta and gmax the largest |kernel value|: a record whose scaled
 // value times gmax comes within 0.2% of 2^31 (a margin for the rounding of the taps)
 // could saturate a conversion, and sends the row to float atomics like a wrapped sum.
-template <int N, int WT, bool FIXED, class PEND>
+template <int N, int WT, bool FIXED, bool STEP, class PEND>
 __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__restrict__ rec,
                                         const uint32_t *bnd, int d_lo, const KernelParams &kp, int jt,
                                         float qscale, float gmax, RecHead *stg, int stg_stride, const float *taps, PEND &pd) {
   constexpr int TPR = RowCfg<N>::TPR;
   int ovf = 0;
   const uint32_t s_end = bnd[d_lo + 1];
+  if constexpr (STEP) {
+    const int W = kp.support;
+    for (uint32_t s = bnd[0] + jt; s < s_end; s += TPR) {
+      int i = d_lo;
+      while (s < bnd[i]) --i;
+      const RecHead r = rec_head(rec, s);
+      const float gy = kernel_tap(kp, (float)(d_lo - i) - kp.half + rec_gy(r));
+      const float gx = rec_gx(r);
+      const int i0 = rec_i0(r);
+      const float vre = r.vre * gy, vim = r.vim * gy;
+      for (int a = 0; a < W; ++a) {
+        const float g = kernel_tap(kp, (float)a - kp.half + gx);
+        add_tap<false>(sre, sim, i0 + a, vre * g, vim * g, ovf);
+      }
+    }
+    return 0;
+  }
   const float q = exp2f(-2.0f * kp.l2c);
   // this thread's record heads are copied into its own three shared slots two records
   // ahead (cp.async), so two loads are in flight while a record is gridded
@@ -328,12 +381,12 @@ __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__
 // return).  bnd[0 .. d_lo + 1]: where the rows j0 = q - d_lo ... q start, and the end; mb:
 // the row's largest bin sum and the total of its bin sums.  Every thread of the row group
 // calls it; it ends with the row buffer free again.
-template <int N, bool FFT, int WT, class PEND, class SYNC>
+template <int N, bool FFT, int WT, bool STEP, class PEND, class SYNC>
 __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, int d_lo, float2 mb,
                                              const Record *__restrict__ rec, int q, bool nonempty,
                                              const KernelParams &kp, float2 *__restrict__ orow, const float2 *twt,
-                                             int jt, float gmax, RecHead *stg, int stg_stride, const float *taps, PEND &pd,
-                                             const SYNC &sync) {
+                                             int jt, float gmax, RecHead *stg, int stg_stride, const float *taps,
+                                             bool ints, PEND &pd, const SYNC &sync) {
   using C = RowCfg<N>;
   constexpr int EPT = C::EPT, TPR = C::TPR;
   constexpr int NST = num_stages(N, EPT);
@@ -355,28 +408,43 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   // n_eff: the busiest bin's magnitude in units of the row's mean per visibility-row
   const float n_eff = mmax * (float)cnt * (1.0f + (float)(W - 1) / (float)kBinCols) / fmaxf(mtot, 0x1p-126f);
   // (a NaN in a kernel table makes the bound NaN and takes float sums, which show it)
-  const bool fixed = kFixedRows<N> && nonempty && cnt < (1u << 30) && bound >= 0x1p-90f && bound <= 0x1p+100f &&
+  constexpr bool INTS = kFixedRows<N, FFT> && !STEP;
+  const bool fixed = INTS && ints && nonempty && cnt < (1u << 30) && bound >= 0x1p-90f && bound <= 0x1p+100f &&
                      n_eff <= (float)kFixedBinCap;
   // a bin of fewer than ~64 mean contributions may hold a single tap above B/8: such rows
   // take delta = B / 2^30, with which no tap or partial sum can leave the int32 range
-  const float unit = n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f;
+  float unit = N >= kFixedMinN ? (n_eff >= 64.0f ? 0x1p-34f : 0x1p-30f) : unit_of(n_eff);
   bool fx = fixed;
+  auto in_ints = [&] {
+    return grid_row<N, WT, INTS, STEP>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride,
+                                       taps, pd);
+  };
+  auto in_float = [&] {
+    grid_row<N, WT, false, STEP>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
+  };
   int ovf = 0;
   if (nonempty) {
-    if (fixed)
-      ovf = grid_row<N, WT, true>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f / (bound * unit), gmax, stg, stg_stride, taps, pd);
-    else grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
+    if (fixed) ovf = in_ints();
+    else in_float();
   }
-  // a tap or a partial sum left the int32 range: accumulate in float.  (A coarser quantum,
-  // B / 2^32 or B / 2^30, would hold the row too, but leaves the cells far below the busiest
-  // bin ten bits.)
+  // a tap or a partial sum left the int32 range: shorter rows once more with B / 2^32, then in
+  // float.  (B / 2^30 would hold any row, but rounds by twice what the row's transform does
+  // where one value dominates it.)
   bool redo = false;
-  if constexpr (kFixedRows<N>) redo = sync.any(ovf < 0);
+  if constexpr (INTS) redo = sync.any(ovf < 0);
   else sync();
+  if constexpr (INTS && N < kFixedMinN) {
+    if (redo && unit < 0x1p-32f) {
+      zero_row<N>(srow, jt);
+      sync();
+      unit = 0x1p-32f;
+      redo = sync.any(in_ints() < 0);
+    }
+  }
   if (redo) {
     zero_row<N>(srow, jt);
     sync();
-    if (nonempty) grid_row<N, WT, false>(sre, sim, rec, bnd, d_lo, kp, jt, 1.0f, gmax, stg, stg_stride, taps, pd);
+    in_float();
     fx = false;
     sync();
   }
@@ -435,14 +503,14 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
   sync();  // the row buffer is reused by the next row
 }
 
-template <int N, bool FFT, int WT>
-__global__ void __launch_bounds__(GridCfg<N>::THREADS,
-                                  N >= 4096 ? 1 : kRowThreadsPerSm / GridCfg<N>::THREADS)
+template <int N, bool FFT, int WT, bool STEP = false>
+__global__ void __launch_bounds__(GridCfg<N, STEP>::THREADS,
+                                  STEP ? (FFT ? 4 : 1) : N >= 4096 ? 1 : kRowThreadsPerSm / GridCfg<N>::THREADS)
 k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, int p0, int np,
             KernelParams kp, float2 *__restrict__ out, uint8_t *__restrict__ occ,
             unsigned long long *__restrict__ counter, Tw tw, const float2 *__restrict__ rowbound,
-            unsigned long long *__restrict__ rows_done, int batch, bool smem_taps) {
-  using C = GridCfg<N>;
+            unsigned long long *__restrict__ rows_done, int batch, bool smem_taps, bool ints) {
+  using C = GridCfg<N, STEP>;
   constexpr int TPR = C::TPR, GT = C::GT, GR = C::GR, GROUPS = C::GROUPS;
   extern __shared__ __align__(16) float2 sm_rows[];
   const int g = threadIdx.x / GT, gt = threadIdx.x % GT;   // group, thread of the group
@@ -489,7 +557,7 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
         if (gt < W + batch && j >= 0)
           cp_async_small<4>(off_sm + (uint32_t)(buf * (kRowBatch + kMaxSupport + 1) + gt) * 4u,
                             off + (b0 + j) * kColBlocks);
-        if (kFixedRows<N> && gt < batch)
+        if (kFixedRows<N, FFT> && ints && gt < batch)
           cp_async_small<8>(rb_sm + (uint32_t)(buf * kRowBatch + gt) * 8u, rowbound + b0 + q0 + gt);
       }
     };
@@ -537,9 +605,9 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
         const long long item = base + r;
         const int pl = (int)(item / N), q = (int)(item % N);
         const int d_lo = min(q, W - 1);
-        const float2 mb = kFixedRows<N> ? s_rb[g][buf][r] : make_float2(0.0f, 0.0f);
-        grid_one_row<N, FFT, WT>(srow, &s_off[g][buf][r + W - 1 - d_lo], d_lo, mb, rec, q, e & 1, kp,
-                                 out + ((int64_t)pl * N + q) * N, twt, jt, gmax, stg, stg_stride, taps, pd, sync);
+        const float2 mb = kFixedRows<N, FFT> && ints ? s_rb[g][buf][r] : make_float2(0.0f, 0.0f);
+        grid_one_row<N, FFT, WT, STEP>(srow, &s_off[g][buf][r + W - 1 - d_lo], d_lo, mb, rec, q, e & 1, kp,
+                                 out + ((int64_t)pl * N + q) * N, twt, jt, gmax, stg, stg_stride, taps, ints, pd, sync);
       }
       if (cnt == 0) sync();  // s_item, s_cnt and the list are read before they are written again
     }
@@ -547,12 +615,21 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
     asm volatile("cp.async.wait_all;" ::: "memory");
   } else {
     __shared__ uint32_t s_bnd[C::ROWS][kMaxSupport + 2];
-    static_assert(!kFixedRows<N>, "float sums");
+    static_assert(!kFixedRows<N, FFT> || STEP, "float sums");
     long long next = group0 * GR;
     while (true) {
-      const long long base = __shfl_sync(0xFFFFFFFFu, next, 0);  // a group is one warp here
+      long long base;
+      if constexpr (GT == 32) {  // a group is one warp, its next rows claimed ahead of time
+        base = __shfl_sync(0xFFFFFFFFu, next, 0);
+        if (gt == 0) next = ngroups * GR + (long long)atomicAdd(counter, (unsigned long long)GR);
+      } else {
+        __shared__ long long s_item;
+        if (gt == 0) s_item = (long long)atomicAdd(counter, (unsigned long long)GR);
+        sync();
+        base = s_item;
+        sync();
+      }
       if (base >= total) break;
-      if (gt == 0) next = ngroups * GR + (long long)atomicAdd(counter, (unsigned long long)GR);
       const long long item = base + rl % GR;
       const bool valid = item < total;
       const int pl = valid ? (int)(item / N) : 0;
@@ -560,17 +637,17 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
       const int64_t b0 = (int64_t)(p0 + pl) * N;
       const int d_lo = min(q, W - 1);
       for (int i = jt; i <= d_lo + 1; i += TPR) s_bnd[rl][i] = off[(b0 + q - d_lo + i) * kColBlocks];
-      __syncwarp();
+      sync();
       const bool empty = !valid || s_bnd[rl][0] == s_bnd[rl][d_lo + 1];
       if (valid && jt == 0) occ[item] = empty ? 0 : 1;
       if (rows_done && valid && jt == 0 && !empty) atomicAdd(rows_done, 1ull);
-      if (!FFT || !__all_sync(0xFFFFFFFFu, empty)) {
+      if (!FFT || sync.any(!empty)) {
         float2 *orow = valid && (!FFT || !empty) ? out + ((int64_t)pl * N + q) * N : nullptr;
         NoPending none;
-        grid_one_row<N, FFT, WT>(srow, s_bnd[rl], d_lo, make_float2(0.0f, 0.0f), rec, q, !empty, kp, orow, twt, jt, gmax,
-                                 stg, stg_stride, taps, none, sync);
+        grid_one_row<N, FFT, WT, STEP>(srow, s_bnd[rl], d_lo, make_float2(0.0f, 0.0f), rec, q, !empty, kp, orow, twt, jt,
+                                       gmax, stg, stg_stride, taps, false, none, sync);
       }
-      __syncwarp();
+      sync();
     }
   }
 }
@@ -852,17 +929,17 @@ static cudaError_t persistent_grid(wst_plan_s *p, K kern, size_t smem, int64_t r
   return cudaSuccess;
 }
 
-template <int N, bool FFT>
-static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) {
-  using C = GridCfg<N>;
+template <int N, bool FFT, bool STEP>
+static cudaError_t launch_grid_rows_as(wst_plan_s *p, int p0, int np, float2 *out) {
+  using C = GridCfg<N, STEP>;
   // the imaging path has the common supports unrolled
-  auto kern = k_grid_rows<N, FFT, 0>;
-  if constexpr (FFT) {
+  auto kern = k_grid_rows<N, FFT, 0, STEP>;
+  if constexpr (FFT && !STEP) {
     if (p->cfg.support == 7) kern = k_grid_rows<N, FFT, 7>;
     else if (p->cfg.support == 8) kern = k_grid_rows<N, FFT, 8>;
   }
   size_t smem = sizeof(float2) * (C::ROWS * C::PADL + (FFT ? line_table_size<N, C::EPT, C::TPR>() : 0)) +
-                3 * C::THREADS * sizeof(RecHead);
+                (STEP ? 0 : 3 * C::THREADS * sizeof(RecHead));
   bool smem_taps = false;
   if (FFT && kTapsShared<N> && p->ktap) {
     int most = 0;
@@ -878,8 +955,21 @@ static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) 
   unsigned long long *counter = p->W_.counters + CNT_WORK;  // cleared by the caller
   kern<<<grid, C::THREADS, smem, p->stream>>>(p->W_.records, p->W_.offsets, p0, np, kernel_params(p), out,
                                              p->W_.occ, counter, tw_half(p), p->W_.rowbound,
-                                             FFT ? p->W_.counters + CNT_ROWS : nullptr, batch, smem_taps);
+                                             FFT ? p->W_.counters + CNT_ROWS : nullptr, batch, smem_taps,
+                                             p->fixed_rows);
   return cudaGetLastError();
+}
+
+template <int N, bool FFT>
+static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) {
+  // float sums of supports without an instance of their own: rows in step (StepCfg)
+  if constexpr (FFT && (N == 1024 || N == 2048)) {
+    if (!p->fixed_rows && p->cfg.support != 7 && p->cfg.support != 8)
+      return launch_grid_rows_as<N, FFT, true>(p, p0, np, out);
+    return launch_grid_rows_as<N, FFT, false>(p, p0, np, out);
+  } else {
+    return launch_grid_rows_as<N, FFT, !FFT && N >= 512 && N <= 2048>(p, p0, np, out);
+  }
 }
 
 template <int N, bool KGRAD>

@@ -580,7 +580,7 @@ cudaError_t sort_visibilities(wst_plan_s *p, const VisCoords &coords, const floa
   cudaError_t e;
   // offsets and, after them in the workspace, the magnitude bins; both start on 256-byte
   // boundaries with padding up to the next array, so the clear may round up to 16 bytes
-  const int nb = bins_per_row(p->n);
+  const int nb = bins_per_row(p);
   const int64_t n_bins = p->n_buckets / kColBlocks * nb;
   const size_t clear = (size_t)((char *)(ws.binmag + n_bins) - (char *)ws.offsets);
   const uint32_t n_clear = clear <= kInitClear ? (uint32_t)((clear + 15) / 16) : 0u;

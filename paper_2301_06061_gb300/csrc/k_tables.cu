@@ -103,6 +103,23 @@ __device__ __forceinline__ double node_value(int kind, int i, int P, double half
   return exp(param * (sqrt(fmax(0.0, 1.0 - z * z)) - 1.0));
 }
 
+// Ghat(0) / Ghat(nu), nu = n_img / (2 n): how much the grid correction raises the edge of the
+// image's rows over their centre (host, for the analytic kernels: Simpson, 64 panels a cell)
+double kernel_edge_ratio(const wst_plan_s *p) {
+  const int W = p->W, P = 64 * W;
+  const double h = (double)W / P, nu = 0.5 * p->n_img / p->n;
+  double g0 = 0.0, g1 = 0.0;
+  for (int i = 0; i <= 2 * P; ++i) {
+    const double x = 0.5 * h * (i - P), z = 2.0 * x / W;
+    const double g = p->cfg.kernel == WST_KERNEL_GAUSS ? exp(-(x * x) / (2.0 * p->cfg.kparam * p->cfg.kparam))
+                                                       : exp(p->cfg.kparam * (sqrt(fmax(0.0, 1.0 - z * z)) - 1.0));
+    const double w = (i & 1) ? 4.0 : (i == 0 || i == 2 * P) ? 1.0 : 2.0;
+    g0 += w * g;
+    g1 += w * g * cos(2.0 * M_PI * nu * x);
+  }
+  return fabs(g0 / g1);
+}
+
 __global__ void k_kernel_nodes(double *nodes, int P, int kind, int W, double param, const float *tab) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j > P) return;

@@ -58,7 +58,7 @@ Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
   L.offsets = off;
   off += align_up((size_t)(p->n_buckets + 1) * sizeof(uint32_t));
   L.binmag = off;  // directly after the offsets: one memset clears both
-  off += align_up((size_t)(p->n_buckets / kColBlocks) * bins_per_row(p->n) * sizeof(float));
+  off += align_up((size_t)(p->n_buckets / kColBlocks) * bins_per_row(p) * sizeof(float));
   L.cursor = off;
   off += align_up((size_t)(p->n_buckets + 1) * sizeof(uint32_t));
   L.scan_tmp = off;
@@ -70,7 +70,7 @@ Layout layout_for(const wst_plan_s *p, int64_t n_vis) {
   L.occ = off;
   off += align_up((size_t)p->n_planes * p->n);
   L.rowbound = off;
-  if (bins_per_row(p->n) > 0) off += align_up((size_t)(p->n_buckets / kColBlocks) * sizeof(float2));
+  if (bins_per_row(p) > 0) off += align_up((size_t)(p->n_buckets / kColBlocks) * sizeof(float2));
   L.comp = off;
   if (p->chunk < p->n_planes) off += align_up((size_t)p->batch * p->n_img * p->n_img * sizeof(float2));
   L.total = off;
@@ -198,6 +198,8 @@ wst_status wst_plan_create(const wst_config *cfg, void *cuda_stream, wst_plan *o
   p->fa = c.n / p->fb;
   p->n_buckets = n_buckets;
   p->timing = (c.flags & WST_FLAG_TIMING) != 0;
+  p->fixed_rows = c.n >= kFixedMinN || (c.n >= kFixedImagingMinN && c.kernel != WST_KERNEL_TABLE &&
+                                        kernel_edge_ratio(p) <= kFixedMaxRatio);
 
   cudaError_t e = cudaSuccess;
 #define ALLOC(ptr, count)                                                  \

@@ -18,10 +18,11 @@ constexpr int kColBlocks = 1;    // sub-buckets per row (by tap-start column; a 
 constexpr uint32_t kDropKey = 0xFFFFFFFFu;
 // Column bins of the fixed-point gridder's bound: for every row bucket (image, plane, j0)
 // the sort sums max(|Re|, |Im|) of the weighted values whose W taps reach each bin of
-// kBinCols columns.  Only images whose rows use fixed-point accumulation have them.
+// kBinCols columns.  Only plans whose rows use fixed-point accumulation have them.
 constexpr int kBinCols = 64, kBinShift = 6;
-constexpr int kFixedMinN = 8192;
-__host__ __device__ constexpr int bins_per_row(int n) { return n >= kFixedMinN ? n / kBinCols : 0; }
+constexpr int kFixedMinN = 8192;        // rows from here on use it throughout,
+constexpr int kFixedImagingMinN = 1024; // rows from here on in the imaging path of plans with
+constexpr double kFixedMaxRatio = 100.0;  // Ghat(0) / Ghat(nu) up to this at the image's edge
 
 // counters[] slots in the workspace
 // CNT_ROWS: non-empty (plane, row) items the imaging path gridded since wst_image began
@@ -126,6 +127,7 @@ struct wst_plan_s {
   double *wcentre_d = nullptr;  // per global plane: centre w_k (FP64)
   float2 *dwff = nullptr;    // per image: plane spacing dw as float-float
   bool table_set = false;
+  bool fixed_rows = false;   // rows accumulated in fixed point (build_tables' caller decides)
   cudaStream_t centres_stream = nullptr;  // where the centres of a configured w range were built last
   // limit of the device-side waits for data (the row kernel's bulk copies), nanoseconds;
   // 0 = expire at once (failure-path testing, wst_plan_set_wait_limit)
@@ -151,6 +153,10 @@ struct wst_plan_s {
   int64_t launches = 0;       // incremented by every launcher
   std::string last_error;
 };
+
+namespace wst {
+inline int bins_per_row(const wst_plan_s *p) { return p->fixed_rows ? p->n / kBinCols : 0; }
+}  // namespace wst
 
 namespace wst {
 
@@ -297,6 +303,7 @@ cudaError_t build_tap_table(wst_plan_s *p);
 // k_tables.cu
 cudaError_t build_tables(wst_plan_s *p);
 int64_t kernel_node_count(const wst_plan_s *p);
+double kernel_edge_ratio(const wst_plan_s *p);  // Ghat(0) / Ghat(nu) at the image's edge, Gaussian and ES kernels
 cudaError_t build_correction(wst_plan_s *p);
 cudaError_t build_plane_centres(wst_plan_s *p);
 

@@ -148,3 +148,51 @@ def test_sort_clear_beyond_one_kernel(wst):
         np.testing.assert_array_equal(i0.cpu().numpy(), io)
         np.testing.assert_array_equal(j0.cpu().numpy(), jo)
         assert plan.stats()["n_kept"] == int((st == 0).sum())
+
+
+@pytest.mark.parametrize("n,W,grid_n", [(1024, 7, 0), (1024, 6, 0), (2048, 9, 0), (2048, 8, 0), (4096, 7, 0), (820, 6, 1024),
+                                        (1640, 8, 2048)])
+@pytest.mark.parametrize("ratio", [95.0, 105.0])
+def test_images_at_both_sides_of_the_integer_rule(wst, n, W, grid_n, ratio):
+    """Rows of 1024 to 4096 are summed in integers where the grid correction raises an image's
+    edge by less than 100, else in float (supports without an instance of their own then by
+    rows in step): a Gaussian exp(-x^2 / 2 sigma^2) raises it by exp((pi sigma n / M)^2 / 2).
+    The bins of the integer path show in the workspace."""
+    fov, n_vis, n_w = 0.1, 9000, 2
+    m = grid_n or n
+    sigma = np.sqrt(2.0 * np.log(ratio)) / np.pi * m / n
+    u, v, w, vis, rng = case(n, fov, n_vis, [n, W, int(ratio)])
+    cfg = wst.Config(n=n, fov=fov, n_w=n_w, w_min=-160.0, w_max=160.0, support=16, kparam=sigma, grid_n=grid_n)
+    bins = 4 * n_w * m * m // 64
+    size = wst.wst_plan_workspace_bytes(wst.Plan(cfg).handle, n_vis)
+    other = wst.Config(n=n, fov=fov, n_w=n_w, w_min=-160.0, w_max=160.0, support=16, kparam=2 * sigma, grid_n=grid_n)
+    float_size = wst.wst_plan_workspace_bytes(wst.Plan(other).handle, n_vis)
+    assert (size >= float_size + bins) if ratio < 100 else size == float_size
+    # the narrower kernel's image (its edge is cut off at W/2, which leaves the side it is on)
+    cfg.support = W
+    plan = wst.Plan(cfg)
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis))
+    img = plan.image(flags=wst.WST_NO_CORRECTION)[0].cpu().numpy()
+    ocfg = OracleConfig(n, fov, n_w, -160.0, 160.0, W, "gauss", sigma)
+    ref = oracle.image_on_grid(ocfg, m, u, v, w, vis, None, correct=False)
+    assert np.abs(img - ref).max() <= TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [64, 512, 1024, 2048, 4096])
+@pytest.mark.parametrize("W,chunk", [(5, 0), (8, 2), (16, 1)])
+def test_planes_of_every_row_length(wst, n, W, chunk):
+    """wst_grid, whose rows of 512 to 2048 are worked on in step: empty rows, rows at the mesh's
+    edges, plane ranges that do not start at the first plane."""
+    fov, n_w = 0.1, 3
+    u, v, w, vis, rng = case(n, fov, 4000, [n, W])
+    v[:2000] *= 0.01  # most rows empty, a few busy
+    v[-50:] = np.float32((0.5 * n - 0.5 * W - 0.01) / fov)
+    wt = rng.uniform(0.25, 2.0, 4000).astype(np.float32)
+    sigma = 0.875 * np.sqrt(W / 7.0)
+    plan = wst.Plan(wst.Config(n=n, fov=fov, n_w=n_w, w_min=-160.0, w_max=160.0, support=W, kparam=sigma))
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis), dev(wt))
+    ref = oracle.grid(OracleConfig(n, fov, n_w, -160.0, 160.0, W, "gauss", sigma), u, v, w, vis, wt)
+    g = torch.full((n_w, n, n), float("nan"), dtype=torch.complex64, device="cuda")
+    for a, b in [(0, n_w)] if not chunk else [(k, min(k + chunk, n_w)) for k in range(0, n_w, chunk)]:
+        wst.wst_grid(plan.handle, a, b, g[a:b])
+    assert np.abs(g.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
