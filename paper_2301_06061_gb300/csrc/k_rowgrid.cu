@@ -90,12 +90,14 @@ struct GroupCfg {
 // 1277 us on 32 planes of 4096^2 with 4.08M visibilities, 986 instead of 882 us on 21 planes
 // with the ES kernel).  Two rows of 8192 in a CTA leave 64 registers a thread: 5.90 instead of
 // 5.03 ms on 16 planes with 20M visibilities.
-// The configuration of float sums that dense rows bound (shared compare-and-swap loops): CTAs
-// of 256 threads on 256 / TPR rows in step, records read directly.  With the groups above,
-// which let a few dense rows finish last, wst_grid took 545 instead of 364 us at 2048^2 x 12
-// (1.33M visibilities, ES of 8), images 7.6 instead of 6.0 ms (24 of 1024^2 x 22, 12.9M, support
-// 6 in float); for supports 7 and 8, whose records are prefetched, the groups are faster (12.2
-// against 16.3 ms on 64 images of 2048^2 x 16), and below 512 they are even.
+// The configuration of float sums, which dense rows bound (shared compare-and-swap loops): CTAs
+// of 256 threads on 256 / TPR rows in step.  With the groups above, which let a few dense
+// rows finish last, wst_grid took 545 instead of 364 us at 2048^2 x 12 (1.33M visibilities, ES
+// of 8), four images of 1024^2 x 8 (4M, support 7) 3.60 instead of 2.23 ms, 16 of 512^2 x 8 (2M)
+// 1.66 instead of 1.29.  Rows shorter than 1024 need two rounds of CTAs for that: with 4096
+// rows of 512 in all the groups are ahead (623 against 660 us, 200,000 visibilities), and a
+// 256^2 x 8 image has too few rows for either.  Integer sums are faster in groups.
+constexpr int kStepCtas = 4;  // per SM
 template <int N>
 struct StepCfg {
   static constexpr int EPT = RowCfg<N>::EPT, TPR = RowCfg<N>::TPR, PADL = RowCfg<N>::PADL;
@@ -323,7 +325,7 @@ __device__ __forceinline__ int grid_row(float *sre, float *sim, const Record *__
   constexpr int TPR = RowCfg<N>::TPR;
   int ovf = 0;
   const uint32_t s_end = bnd[d_lo + 1];
-  if constexpr (STEP) {
+  if constexpr (STEP && WT == 0) {
     const int W = kp.support;
     for (uint32_t s = bnd[0] + jt; s < s_end; s += TPR) {
       int i = d_lo;
@@ -505,7 +507,7 @@ __device__ __forceinline__ void grid_one_row(float2 *srow, const uint32_t *bnd, 
 
 template <int N, bool FFT, int WT, bool STEP = false>
 __global__ void __launch_bounds__(GridCfg<N, STEP>::THREADS,
-                                  STEP ? (FFT ? 4 : 1) : N >= 4096 ? 1 : kRowThreadsPerSm / GridCfg<N>::THREADS)
+                                  STEP ? (FFT ? kStepCtas : 1) : N >= 4096 ? 1 : kRowThreadsPerSm / GridCfg<N>::THREADS)
 k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, int p0, int np,
             KernelParams kp, float2 *__restrict__ out, uint8_t *__restrict__ occ,
             unsigned long long *__restrict__ counter, Tw tw, const float2 *__restrict__ rowbound,
@@ -934,12 +936,13 @@ static cudaError_t launch_grid_rows_as(wst_plan_s *p, int p0, int np, float2 *ou
   using C = GridCfg<N, STEP>;
   // the imaging path has the common supports unrolled
   auto kern = k_grid_rows<N, FFT, 0, STEP>;
-  if constexpr (FFT && !STEP) {
-    if (p->cfg.support == 7) kern = k_grid_rows<N, FFT, 7>;
-    else if (p->cfg.support == 8) kern = k_grid_rows<N, FFT, 8>;
+  const bool own = FFT && (p->cfg.support == 7 || p->cfg.support == 8);
+  if constexpr (FFT) {
+    if (p->cfg.support == 7) kern = k_grid_rows<N, FFT, 7, STEP>;
+    else if (p->cfg.support == 8) kern = k_grid_rows<N, FFT, 8, STEP>;
   }
   size_t smem = sizeof(float2) * (C::ROWS * C::PADL + (FFT ? line_table_size<N, C::EPT, C::TPR>() : 0)) +
-                (STEP ? 0 : 3 * C::THREADS * sizeof(RecHead));
+                (STEP && !own ? 0 : 3 * C::THREADS * sizeof(RecHead));
   bool smem_taps = false;
   if (FFT && kTapsShared<N> && p->ktap) {
     int most = 0;
@@ -962,14 +965,15 @@ static cudaError_t launch_grid_rows_as(wst_plan_s *p, int p0, int np, float2 *ou
 
 template <int N, bool FFT>
 static cudaError_t launch_grid_rows(wst_plan_s *p, int p0, int np, float2 *out) {
-  // float sums of supports without an instance of their own: rows in step (StepCfg)
-  if constexpr (FFT && (N == 1024 || N == 2048)) {
-    if (!p->fixed_rows && p->cfg.support != 7 && p->cfg.support != 8)
+  if constexpr (N <= 2048) {  // float sums on rows in step (StepCfg) where two rounds of their CTAs fill the SMs
+    int sms = 0;
+    const cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, p->device);
+    if (e != cudaSuccess) return e;
+    const int64_t ctas = (int64_t)np * N / StepCfg<N>::ROWS;
+    if (!(FFT && p->fixed_rows) && (N >= 1024 || ctas >= (int64_t)2 * kStepCtas * sms))
       return launch_grid_rows_as<N, FFT, true>(p, p0, np, out);
-    return launch_grid_rows_as<N, FFT, false>(p, p0, np, out);
-  } else {
-    return launch_grid_rows_as<N, FFT, !FFT && N >= 512 && N <= 2048>(p, p0, np, out);
   }
+  return launch_grid_rows_as<N, FFT, false>(p, p0, np, out);
 }
 
 template <int N, bool KGRAD>

@@ -196,3 +196,29 @@ def test_planes_of_every_row_length(wst, n, W, chunk):
     for a, b in [(0, n_w)] if not chunk else [(k, min(k + chunk, n_w)) for k in range(0, n_w, chunk)]:
         wst.wst_grid(plan.handle, a, b, g[a:b])
     assert np.abs(g.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [64, 128, 256, 512])
+@pytest.mark.parametrize("W", [7, 9])
+@pytest.mark.parametrize("more", [-1, 0])
+def test_short_rows_below_and_from_two_rounds_of_blocks(wst, n, W, more):
+    """Float rows shorter than 1024 are worked on in step from two rounds of blocks (four of
+    4096 / N rows per SM) on, by groups below: images and planes at both sides, some planes and
+    rows without visibilities."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n_w, fov = 2 * 4 * sms * 4096 // (n * n) + more, 0.1
+    u, v, w, vis, rng = case(n, fov, 6000, [n, W])
+    v[:3000] *= 0.01
+    w[:1000] = 3.0
+    wt = rng.uniform(0.25, 2.0, 6000).astype(np.float32)
+    sigma = 0.875 * np.sqrt(W / 7.0)
+    plan = wst.Plan(wst.Config(n=n, fov=fov, n_w=n_w, w_min=-160.0, w_max=160.0, support=W, kparam=sigma))
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis), dev(wt))
+    ocfg = OracleConfig(n, fov, n_w, -160.0, 160.0, W, "gauss", sigma)
+    img = plan.image(flags=wst.WST_NO_CORRECTION)[0].cpu().numpy()
+    ref = oracle.image(ocfg, u, v, w, vis, wt, correct=False)
+    assert np.abs(img - ref).max() <= TOL * np.abs(ref).max()
+    g = torch.full((n_w, n, n), float("nan"), dtype=torch.complex64, device="cuda")
+    wst.wst_grid(plan.handle, 0, n_w, g)
+    ref = oracle.grid(ocfg, u, v, w, vis, wt)
+    assert np.abs(g.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
