@@ -814,8 +814,8 @@ k_cols_b16(const float2 *__restrict__ planes, int p0, int p1, int n_w, Tw tw,
 //
 // Tiles (LA rows x 16 columns of a plane, 128-byte row segments) are copied by the
 // tensor engine: one thread issues cp.async.bulk.tensor for a plane's tile into a ring of
-// three shared slots, each with an mbarrier that counts the copy's bytes; the ring runs
-// two planes ahead.  Every wait on a slot is bounded (wait_ns; on expiry the CTA records
+// three shared slots (two where BLOCKS is 1 at 128 lines), each with an mbarrier that counts
+// the copy's bytes; a slot is refilled as soon as its plane's stage 0 has read it.  Every wait on a slot is bounded (wait_ns; on expiry the CTA records
 // WST_ERR_TIMEOUT, lets its copies in flight land and returns).  The transform is that of
 // k_cols_b16 (radix 16, in-place exchange in the slot, then LA/16), with two CTA barriers
 // per plane: one after the stage-0 reads (the slot of the previous plane is then free
@@ -919,7 +919,7 @@ k_cols_b_tma(const __grid_constant__ CUtensorMap tmap, int p0, int p1, int n_w, 
     const int pstart = P;
     const int pend = min(p1, (img + 1) * n_w);
     // the per-plane step of each output for this image (exact), conjugated.  The screen
-    // evaluations are long dependent chains (n - 1, float-float product, sincospi): four
+    // evaluations are long dependent chains (n - 1, float-float product, cis_octant): four
     // outputs at a time give the scheduler independent work without keeping all sixteen
     // live; the results reach the unrolled plane loop through thread-private shared slots
     {

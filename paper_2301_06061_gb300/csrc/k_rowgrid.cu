@@ -47,12 +47,12 @@
 //   - wst_grid hands the cells to the caller: its rows are summed in float.
 //   - In an image a cell's rounding is one term of the row's transform, which rounds by about
 //     2^-25 of the row's root sum of squares, R.  The integers' roundings add up to
-//     0.76 sqrt(visibilities) delta over the row.  With m the mean magnitude, R is about
-//     1.2 m sqrt(visibilities) or more, and the steps of unit_of keep the sum below the
-//     transform's rounding up to 800 contributions in the busiest bin; beyond, float sums
+//     0.76 sqrt(visibilities) delta over the row (seven taps).  With m the mean magnitude, R
+//     is about 0.6 m sqrt(visibilities) or more, and the steps of unit_of keep the sum below
+//     the transform's rounding up to 400 contributions in the busiest bin; beyond, float sums
 //     round as much themselves (their partial sums grow with the count).  A row that one
 //     value dominates (R near B) leaves the range with the finest quantum and is taken
-//     again with B / 2^32, half the transform's rounding at 8192 visibilities, but no
+//     again with B / 2^32, about half the transform's rounding at 8192 visibilities, but no
 //     coarser: then float.
 //   - A strong grid correction amplifies either rounding alike at the image's edge, by
 //     (Ghat(0) / Ghat(1/2))^2, and with it the difference between the two: 2e-5 of an image
@@ -74,7 +74,7 @@ namespace wst {
 // a group then takes GR rows in step.  CTAs of 128 threads, so that short workloads (a
 // 256^2 image has 16 rows per SM) still spread over the SMs.  With 256 threads on 2 to 16 rows
 // in step, an item and its offsets fetched row by row, 64 images of 2048^2 x 16 took 14.3 ms,
-// now 7.4, and a 256^2 one 20 us, now 6.8.
+// now 7.7 (integer sums).
 template <int N, int MINT = 128>
 struct GroupCfg {
   static constexpr int EPT = RowCfg<N>::EPT, TPR = RowCfg<N>::TPR, PADL = RowCfg<N>::PADL;
@@ -221,7 +221,7 @@ template <int N, bool FFT>
 constexpr bool kFixedRows = N >= kFixedMinN || (FFT && N >= kFixedImagingMinN);
 
 // delta / B of a row shorter than 8192, n_eff the mean contributions in its busiest bin.
-// Sparse bins hold sums of a few taps: up to 64 the quantum stays near 2^-27 of the mean
+// Sparse bins hold sums of a few taps: up to 64 the quantum stays below 2^-26 of the mean
 // magnitude, and a cell may hold, before the row is accumulated again, the whole bin below
 // 16 and half of it below 64.  From 64 on it is B / 2^34, a cell up to an eighth of the bin.
 __device__ __forceinline__ float unit_of(float n_eff) {
@@ -662,7 +662,8 @@ k_grid_rows(const Record *__restrict__ rec, const uint32_t *__restrict__ off, in
 // trips; with `together` the first attempts of all T go out at once and only what lost a race
 // (another lane or an equal address in the same run) is added the usual way.  That pays
 // where the lanes of a warp seldom share a sample: at kTogether samples per cell and more,
-// less than one pair of 32 (8193 samples, a 512^2 training step: 132 -> 107 us).
+// less than one pair of 32 (8193 samples, a 512^2 training step: 132 -> 107 us; 92 with rows
+// claimed when a group is free).
 constexpr float kTogether = 512.0f;
 template <int T>
 __device__ __forceinline__ void add_all(float *const (&at)[T], const float (&x)[T], int offset, bool together) {
@@ -701,7 +702,8 @@ __device__ __forceinline__ void add_all(float *const (&at)[T], const float (&x)[
 // Kaiser-Bessel table of 8 gave visibilities of a 2048^2 image 5.7e-5 off those in order, now
 // 8e-6, as two runs in order differ, and of an 8192^2 one 3.5e-5, now 1.9e-5 (in order 7e-6;
 // bucket by bucket 1.5e-5).  10M visibilities on 16 planes of 8192^2 took 6.62 ms then, now
-// 6.87 (bucket by bucket 7.41), 400,000 on 16 of 1024^2 191 us, now 186 (165 evenly split).
+// 6.75, 2.56 of it here (bucket by bucket 7.41), 400,000 on 16 of 1024^2 191 us, now 185 (165
+// evenly split).
 //
 // Sums kept in sorted order, where a warp's reductions fall on whole sectors, and handed back
 // by a pass of their own took as long (the whole call 6.69 against 6.66 ms at 10M visibilities
@@ -909,7 +911,7 @@ static Tw tw_half(const wst_plan_s *p) {
 // the grid of a persistent row kernel: every resident CTA, no more than there are rows for;
 // and the rows of a batch, so that each group gets 32 batches or more of a long stream (dense
 // rows come in runs: with eight batches the gridder of 1M visibilities at 2048^2 x 16 ended on
-// a few groups, 245 us, now 157; rows one by one cost 4096^2 x 32 1428 instead of 1277 us)
+// a few groups, 245 us, now 152; rows one by one cost 4096^2 x 32 1428 instead of 1277 us)
 template <class C, class K>
 static cudaError_t persistent_grid(wst_plan_s *p, K kern, size_t smem, int64_t rows, int &grid, int &batch) {
   // always raised to the request: the 48 KB default counts the kernel's static shared
@@ -925,7 +927,7 @@ static cudaError_t persistent_grid(wst_plan_s *p, K kern, size_t smem, int64_t r
   grid = (int)(resident < need ? resident : need);
   const int64_t b = rows / ((int64_t)grid * C::GROUPS * 32);
   // short rows have few threads for a dense row: eight at a time, 26.6M visibilities on eight
-  // 2048^2 images (W = 10) took 18.5 ms, two 8.0 (64 sparser images 7.4 and 7.8)
+  // 2048^2 images (W = 8) took 15.5 ms, two 8.6 (64 sparser images 7.3 and 7.7)
   const int most = C::TPR <= 128 ? 2 : kRowBatch;
   for (batch = 1; 2 * batch <= b && 2 * batch <= most;) batch *= 2;
   return cudaSuccess;
