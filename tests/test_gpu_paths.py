@@ -222,3 +222,21 @@ def test_short_rows_below_and_from_two_rounds_of_blocks(wst, n, W, more):
     wst.wst_grid(plan.handle, 0, n_w, g)
     ref = oracle.grid(ocfg, u, v, w, vis, wt)
     assert np.abs(g.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("n", [1024, 2048, 4096])
+def test_rows_too_dense_for_the_integer_bound(wst, n):
+    """Rows whose busiest 64 columns hold more than 8192 times the row's mean magnitude go
+    straight to float sums, beside ordinary rows in integers (300,000 values over three bins
+    of seven rows)."""
+    fov, dense, rest = 0.1, 300_000, 20_000
+    rng = np.random.default_rng(n)
+    u = (np.concatenate([rng.uniform(-90.0, 90.0, dense), rng.uniform(-0.45, 0.45, rest) * n]) / fov).astype(np.float32)
+    v = (np.concatenate([np.zeros(dense), rng.uniform(-0.45, 0.45, rest) * n]) / fov).astype(np.float32)
+    w = rng.uniform(-10.0, 10.0, dense + rest).astype(np.float32)
+    vis = synth.random_visibilities(dense + rest, rng)
+    plan = wst.Plan(wst.Config(n=n, fov=fov, n_w=1, w_min=-10.0, w_max=10.0))
+    plan.set_vis(dev(u), dev(v), dev(w), dev(vis))
+    img = plan.image(flags=wst.WST_NO_CORRECTION)[0].cpu().numpy()
+    ref = oracle.image(OracleConfig(n, fov, 1, -10.0, 10.0, 7, "gauss", 0.875), u, v, w, vis, None, correct=False)
+    assert np.abs(img - ref).max() <= TOL * np.abs(ref).max()
